@@ -212,6 +212,9 @@ void derive_consts(const HostInst& h, StepConsts<R>& K) {
   const R v_top = std::sqrt(K.e_hi * K.K_V[kElectron]);
   K.vb_cap = std::min(K.vlim[kElectron], v_top);
   K.P0 = (K.ndt * K.vb_cap) * smax;
+  // u = (k + 1/2) 2^-23 < P0 for the integers k below P0 2^23 - 1/2
+  const double thr = std::ceil(std::ldexp((double)K.P0, 23) - 0.5);
+  K.cand_thr = !(thr > 0.0) ? 0u : (thr < 8388608.0 ? (uint32_t)thr : 8388608u);
 }
 
 // Derive the constants of instance i (everything that does not need
@@ -263,22 +266,13 @@ T* carve(char*& p, size_t n) {
   return r;
 }
 
-// Bytes of a store of n slots whose five real streams have rsz bytes each.
-size_t soa_bytes(size_t n, size_t rsz) {
-  return 2 * ((n * 4 + 255) & ~size_t(255)) + 5 * ((n * rsz + 255) & ~size_t(255));
+// Seven arrays of n markers (reals of rsz bytes) carved from p, each from a
+// 256-byte boundary: field order cell, off, vx, vy, vz, w_j, id.
+void carve_arrays(char* p, size_t n, size_t rsz, void* f[7]) {
+  for (int k = 0; k < 7; ++k) f[k] = carve<char>(p, n * (k == 0 || k == 6 ? 4 : rsz));
 }
-
-SoA carve_soa(char*& p, size_t n, size_t rsz) {
-  SoA s;
-  s.cell = carve<int32_t>(p, n);
-  s.off = reinterpret_cast<float*>(carve<char>(p, n * rsz));
-  s.vx = reinterpret_cast<float*>(carve<char>(p, n * rsz));
-  s.vy = reinterpret_cast<float*>(carve<char>(p, n * rsz));
-  s.vz = reinterpret_cast<float*>(carve<char>(p, n * rsz));
-  s.wj = reinterpret_cast<float*>(carve<char>(p, n * rsz));
-  s.id = carve<uint32_t>(p, n);
-  return s;
-}
+// Room for them beyond n * (8 + 5 rsz) bytes.
+constexpr size_t kArraysPad = 7 * 256;
 
 int dmalloc(slpic_ctx* c, void** p, size_t bytes, const char* what) {
   cudaError_t e = cudaMalloc(p, bytes);
@@ -415,20 +409,21 @@ int commit(slpic_ctx* c) {
       SpeciesDev& S = P.sp[s];
       S.cap_tiles = cap_tiles[s];
       const size_t slots = (size_t)cap_tiles[s] * kTile;
-      const size_t stage_b = s == kElectron ? (size_t)cap_tiles[kIon] * kTile : 0;
+      const size_t stage_w = s == kElectron ? (size_t)cap_tiles[kIon] * kTile : 0;
       const size_t cand_slots = s == kElectron ? slots : 0;
       const size_t arr = ((size_t)cap_tiles[s] + 1) * 4 + 256;
       const size_t rsz = c->fp64 ? 8 : 4;
       const size_t crsz = c->fp64 ? sizeof(CandRec<double>) : sizeof(CandRec<float>);
-      size_t b = 2 * soa_bytes(slots, rsz) + soa_bytes(stage_b, rsz) + 4 * arr +
-                 cand_slots * crsz + 512;
+      // (a buffer can also hold a caller's arrays of as many markers: the
+      // one not in use stages loads and reads)
+      const size_t store = slots * (8 + 5 * rsz) + kArraysPad;
+      size_t b = 2 * (store + 256) + stage_w * rsz + 4 * arr + cand_slots * crsz + 1024;
       void* sb;
       if (int rc = dmalloc(c, &sb, b, "marker buffers")) return rc;
       char* q = (char*)sb;
-      S.buf[0] = carve_soa(q, slots, rsz);
-      S.buf[1] = carve_soa(q, slots, rsz);
-      if (stage_b) S.stage_b = carve_soa(q, stage_b, rsz);
-      else std::memset(&S.stage_b, 0, sizeof(SoA));
+      S.buf[0] = carve<unsigned char>(q, store);
+      S.buf[1] = carve<unsigned char>(q, store);
+      S.stage_w = stage_w ? (void*)carve<char>(q, stage_w * rsz) : nullptr;
       S.fill[0] = carve<uint32_t>(q, cap_tiles[s] + 1);
       S.fill[1] = carve<uint32_t>(q, cap_tiles[s] + 1);
       S.births = carve<uint32_t>(q, cap_tiles[s] + 1);
@@ -497,11 +492,10 @@ int commit(slpic_ctx* c) {
   // otherwise deposits use global atomics
   int smem_nodes = max_nodes <= 16385 ? max_nodes : 0;
   int bps = 0, warps = 0;
-  size_t sbytes = 0;
-  int e = push_config(c->fp64, smem_nodes, &warps, &bps, &sbytes);
+  int e = push_config(c->fp64, smem_nodes, &warps, &bps);
   if (e != 0 || bps == 0) {
     smem_nodes = 0;
-    e = push_config(c->fp64, 0, &warps, &bps, &sbytes);
+    e = push_config(c->fp64, 0, &warps, &bps);
     if (e != 0 || bps == 0) return fail(c, SLPIC_ERR_CUDA, "particle kernel cannot be launched");
   }
   c->refs.smem_nodes = smem_nodes;
@@ -513,8 +507,7 @@ int commit(slpic_ctx* c) {
   if (smem_nodes) {
     // more warps per CTA may fit when the deposits go to global memory
     int gw = 0, gbps = 0;
-    size_t gbytes = 0;
-    if (int e2 = push_config(c->fp64, 0, &gw, &gbps, &gbytes))
+    if (int e2 = push_config(c->fp64, 0, &gw, &gbps))
       return cuda_fail(c, (cudaError_t)e2, "particle kernel configuration");
     if (gbps > 0 && gw > warps) max_warps = gw;
   }
@@ -1078,6 +1071,34 @@ extern "C" int slpic_seed(slpic_ctx* c, int inst, int species, int64_t n, int mo
 
 namespace {
 
+// Whether a kernel of the context's device can read `bytes` bytes at p as
+// values of `align` bytes: inside one allocation of the device, aligned.
+bool kernel_readable(slpic_ctx* c, const void* p, size_t bytes, size_t align) {
+  cudaPointerAttributes a;
+  if (reinterpret_cast<uintptr_t>(p) % align) return false;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (a.type != cudaMemoryTypeDevice || a.device != c->device) return false;
+  typedef CUresult (*range_fn)(CUdeviceptr*, size_t*, CUdeviceptr);
+  static const range_fn range = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault,
+                                         &q) != cudaSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return reinterpret_cast<range_fn>(f);
+  }();
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
+  if (!range || range(&base, &size, at) != CUDA_SUCCESS) return false;
+  return at + bytes <= base + size;
+}
+
 int load_common(slpic_ctx* c, int inst, int species, const Arrays& src, int64_t n,
                 uint32_t next_id, cudaMemcpyKind kind) {
   if (!valid_inst(c, inst) || (species != 0 && species != 1) || n < 0)
@@ -1095,21 +1116,27 @@ int load_common(slpic_ctx* c, int inst, int species, const Arrays& src, int64_t 
     return fail(c, SLPIC_ERR_CAPACITY, "%lld markers exceed the capacity", (long long)n);
   SpeciesState st;
   if (int rc = read_state(c, inst, species, &st)) return rc;
-  const SoA& d = S.buf[st.cur];
-  if (n > 0) {
-    void* dst[7] = {d.cell, d.off, d.vx, d.vy, d.vz, d.wj, d.id};
+  // arrays on the device are read where they are; host arrays (and whatever a
+  // kernel must not read) are copied to the buffer that is not in use first,
+  // by a copy that returns an error for what is no such memory
+  void* f[7];
+  std::memcpy(f, src.f, sizeof f);
+  bool direct = kind == cudaMemcpyDeviceToDevice;
+  for (int k = 0; k < 7 && direct && n > 0; ++k)
+    direct = kernel_readable(c, f[k], field_bytes(c, k, (size_t)n), field_bytes(c, k, 1));
+  if (n > 0 && !direct) {
+    carve_arrays(reinterpret_cast<char*>(S.buf[st.cur ^ 1u]), (size_t)n, c->fp64 ? 8 : 4, f);
     for (int k = 0; k < 7; ++k)
-      CK(cudaMemcpyAsync(dst[k], src.f[k], field_bytes(c, k, (size_t)n), kind, c->stream),
-         "load");
+      CK(cudaMemcpyAsync(f[k], src.f[k], field_bytes(c, k, (size_t)n), kind, c->stream), "load");
   }
-  // validate on the device: a marker outside the gap would make the step
+  // validated on the device: a marker outside the gap would make the step
   // read and write outside the field and charge arrays
   unsigned int* scratch = c->d_scratch;
   unsigned int bad_init[4] = {0xFFFFFFFFu, 0u, 0u, 0u};
   CK(cudaMemcpyAsync(scratch, bad_init, 16, cudaMemcpyHostToDevice, c->stream), "load");
-  launch_validate(c->fp64, d, (uint32_t)n, P.n_cells, P.charge_shift, scratch,
-                  reinterpret_cast<unsigned long long*>(scratch + 2), c->stream);
-  CK(cudaGetLastError(), "validate");
+  launch_place(c->fp64, f, S.buf[st.cur], (uint32_t)n, P.n_cells, P.charge_shift, scratch,
+               reinterpret_cast<unsigned long long*>(scratch + 2), c->stream);
+  CK(cudaGetLastError(), "load");
   unsigned int res[4];
   CK(cudaMemcpyAsync(res, scratch, 16, cudaMemcpyDeviceToHost, c->stream), "load");
   CK(cudaStreamSynchronize(c->stream), "load");
@@ -1286,22 +1313,31 @@ int read_common(slpic_ctx* c, int inst, int species, const Arrays& host, int64_t
   if (st.n_live > 0) {
     if (int r3 = arrays_check(c, host)) return r3;
     const SpeciesDev& S = c->h_inst[inst].sp[species];
-    const SoA& d = S.buf[st.cur];
-    std::vector<uint32_t> fill(st.n_tiles);
-    CK(cudaMemcpy(fill.data(), S.fill[st.cur], st.n_tiles * 4, cudaMemcpyDeviceToHost), "read");
-    const size_t slots = (size_t)st.n_tiles * kTile;
-    std::vector<char> tmp(field_bytes(c, 1, slots));
-    const void* srcs[7] = {d.cell, d.off, d.vx, d.vy, d.vz, d.wj, d.id};
-    for (int f = 0; f < 7; ++f) {
-      const size_t esz = field_bytes(c, f, 1);
-      CK(cudaMemcpy(tmp.data(), srcs[f], slots * esz, cudaMemcpyDeviceToHost), "read");
-      char* out = static_cast<char*>(host.f[f]);
-      size_t o = 0;
-      for (uint32_t k = 0; k < st.n_tiles; ++k) {
-        std::memcpy(out + o * esz, tmp.data() + (size_t)k * kTile * esz, (size_t)fill[k] * esz);
-        o += fill[k];
-      }
+    // live markers before each tile, in the fills of the buffer that is not
+    // in use; the markers go through that buffer, in order
+    std::vector<uint32_t> pre(st.n_tiles);
+    CK(cudaMemcpy(pre.data(), S.fill[st.cur], st.n_tiles * 4, cudaMemcpyDeviceToHost), "read");
+    uint32_t before = 0;
+    for (uint32_t& p : pre) {
+      const uint32_t m = p;
+      p = before;
+      before += m;
     }
+    CK(cudaMemcpyAsync(S.fill[st.cur ^ 1u], pre.data(), st.n_tiles * 4, cudaMemcpyHostToDevice,
+                       c->stream),
+       "read");
+    // (after a failed step the fills hold what that step left)
+    const size_t n = std::min<size_t>(before, st.n_live);
+    void* f[7];
+    carve_arrays(reinterpret_cast<char*>(S.buf[st.cur ^ 1u]), before, c->fp64 ? 8 : 4, f);
+    launch_gather(c->fp64, S.buf[st.cur], S.fill[st.cur], S.fill[st.cur ^ 1u], st.n_tiles, f,
+                  c->stream);
+    CK(cudaGetLastError(), "read");
+    for (int k = 0; k < 7; ++k)
+      CK(cudaMemcpyAsync(host.f[k], f[k], field_bytes(c, k, n), cudaMemcpyDeviceToHost,
+                         c->stream),
+         "read");
+    CK(cudaStreamSynchronize(c->stream), "read");
   }
   return rc;
 }

@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(kCollThreads, 4) k_collide(DeviceRefs r) {
     const uint32_t T = ion_chunk ? (uint32_t)kCollMaxChunkTiles : Te;
     const uint32_t wt = T / kCollWarps;
     const uint32_t kw = (ion_chunk ? local - e_chunks : local) * T + warp * wt;
-    const SoAT<R> me = soa_as<R>(E.buf[se.cur]);
+    const Markers<R> me{E.buf[se.cur]};
     const StepConsts<R>& K = consts<R>(P);
     const R kv = K.K_V[kElectron], vlim = K.vlim[kElectron];
     // events of the tiles (electron chunks: queued candidates; ion chunks:
@@ -162,9 +162,10 @@ __global__ void __launch_bounds__(kCollThreads, 4) k_collide(DeviceRefs r) {
       const size_t kbase = (size_t)kw * kTile;
       // the new velocity of slot o, and the deposit with it
       auto finish_one = [&](uint32_t o, int cell, R off, R wj, const Velocity<R>& nv) {
-        me.vx[o] = nv.vx;
-        me.vy[o] = nv.vy;
-        me.vz[o] = nv.vz;
+        const Slot<R> m = me[o];
+        m.vx() = nv.vx;
+        m.vy() = nv.vy;
+        m.vz() = nv.vz;
         if (dep)
           deposit(rho_e, cell, off,
                   fixed_charge(beta_of(r_sqrt(nv.vx * nv.vx + nv.vy * nv.vy + nv.vz * nv.vz),
@@ -328,7 +329,7 @@ __global__ void __launch_bounds__(kCollThreads, 4) k_collide(DeviceRefs r) {
     if (warp_births) {
       const uint32_t app_e = tail_slot(E, se), app_i = tail_slot(I, si);
       const uint32_t cap_e = E.cap_tiles * (uint32_t)kTile, cap_i = I.cap_tiles * (uint32_t)kTile;
-      const SoAT<R> mi = soa_as<R>(I.buf[si.cur]);
+      const Markers<R> mi{I.buf[si.cur]};
       if (!ion_chunk) {
         // the ionized candidates in candidate order, queued (in the elastic
         // queue's index array, free after pass 1) and placed 32 at a time:
@@ -349,10 +350,10 @@ __global__ void __launch_bounds__(kCollThreads, 4) k_collide(DeviceRefs r) {
               atomicCAS(&ctrl->error, 0, kErrCapacity);
             } else {
               if (P.field_mode == 1)
-                born_pair<R>(P, me, mi, pe, pi, cr.cell, cr.off, cr.wj, cr.id, step, cr.vx,
+                born_pair<R>(P, me[pe], mi[pi], cr.cell, cr.off, cr.wj, cr.id, step, cr.vx,
                              se.next_id + rank, si.next_id + rank);
               else
-                born_pair<R, false>(P, me, mi, pe, pi, cr.cell, cr.off, cr.wj, cr.id, step, cr.vx,
+                born_pair<R, false>(P, me[pe], mi[pi], cr.cell, cr.off, cr.wj, cr.id, step, cr.vx,
                                     se.next_id + rank, si.next_id + rank);
             }
           }
@@ -381,7 +382,7 @@ __global__ void __launch_bounds__(kCollThreads, 4) k_collide(DeviceRefs r) {
         if (b_tail != b_head) drain_births(b_tail - b_head);
       } else {
         // electrons emitted at the cathode, after every ionization electron
-        const SoAT<R> sb = soa_as<R>(E.stage_b);
+        const R* sw = reinterpret_cast<const R*>(E.stage_w);
         for (uint32_t c0 = 0; c0 < total; c0 += 32) {
           const uint32_t ce = c0 + lane;
           uint32_t q;
@@ -394,7 +395,7 @@ __global__ void __launch_bounds__(kCollThreads, 4) k_collide(DeviceRefs r) {
             continue;
           }
           const size_t o = (size_t)(kw + j) * kTile + q;
-          write_marker(me, pe, sb.cell[o], sb.off[o], sb.vx[o], sb.vy[o], sb.vz[o], sb.wj[o],
+          write_marker(me[pe], 0, (R)0, (R)0, (R)0, (R)0, sw[o],
                        kGenBit | ((se.next_id + rank) & kSerialMask));
         }
       }

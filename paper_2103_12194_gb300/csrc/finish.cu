@@ -41,7 +41,7 @@ __device__ __forceinline__ void plan_totals(const DeviceRefs& r, int n_seg, unsi
   r.seg_wstart[n_seg] = wstart;
   r.coll_start[r.n_inst] = coll;
   r.move_start[n_seg] = move;
-  r.ctrl->n_super = start;
+  r.ctrl->n_tiles = start;
   r.ctrl->w_total = wstart;
   r.ctrl->n_seg = n_seg;
   r.ctrl->n_coll_chunks = coll;
@@ -57,7 +57,6 @@ __device__ __forceinline__ void plan_totals(const DeviceRefs& r, int n_seg, unsi
 __device__ void plan_next_warp(const DeviceRefs& r) {
   const int lane = threadIdx.x & 31;
   const int n_seg = r.n_inst * 2;
-  const long long W = r.push_warps;
   long long ns[kPlanPerLane], w[kPlanPerLane], mv[kPlanPerLane], nc[kPlanPerLane / 2];
   long long s_ns = 0, s_w = 0, s_mv = 0, s_nc = 0;
 #pragma unroll
@@ -65,7 +64,7 @@ __device__ void plan_next_warp(const DeviceRefs& r) {
     const int sg = lane * kPlanPerLane + j;
     ns[j] = w[j] = mv[j] = 0;
     if (sg < n_seg) {
-      ns[j] = ((long long)r.sstate[sg].n_tiles + W - 1) / W;
+      ns[j] = r.sstate[sg].n_tiles;
       w[j] = ns[j] * ((sg & 1) ? kWeightIon : kWeightElectron);
       const Transfer& x = r.xfer[sg];
       if (x.compact) mv[j] = ((long long)x.n_tiles_old + kMoveChunkTiles - 1) / kMoveChunkTiles;
@@ -113,8 +112,7 @@ __device__ void plan_next_warp(const DeviceRefs& r) {
 }
 
 // Plan the next step from the tiles in use (all threads of one CTA):
-// particle-kernel super-tiles (push_warps tiles each) and their weights per
-// segment, repacking chunks per segment and collision chunks per instance,
+// particle-kernel tiles and their weights per segment, repacking chunks per segment and collision chunks per instance,
 // as exclusive block scans in rounds of kFinThreads entries.
 __device__ void plan_next(const DeviceRefs& r, long long* s_buf) {
   __shared__ long long s_carry[4];
@@ -123,7 +121,6 @@ __device__ void plan_next(const DeviceRefs& r, long long* s_buf) {
     if (threadIdx.x < 32) plan_next_warp(r);
     return;
   }
-  const long long W = r.push_warps;
   const int t = threadIdx.x;
   if (t < 4) s_carry[t] = 0;
   __syncthreads();
@@ -131,7 +128,7 @@ __device__ void plan_next(const DeviceRefs& r, long long* s_buf) {
     const int sg = base + t;
     long long ns = 0, w = 0, mv = 0;
     if (sg < n_seg) {
-      ns = ((long long)r.sstate[sg].n_tiles + W - 1) / W;
+      ns = r.sstate[sg].n_tiles;
       w = ns * ((sg & 1) ? kWeightIon : kWeightElectron);
       const Transfer& x = r.xfer[sg];
       if (x.compact) mv = ((long long)x.n_tiles_old + kMoveChunkTiles - 1) / kMoveChunkTiles;
@@ -354,16 +351,16 @@ __global__ void __launch_bounds__(256) k_deposit(DeviceRefs r, int inst) {
     const int sp = it < ne ? 0 : 1;
     const uint32_t k = it < ne ? it : it - ne;
     const SpeciesState& st = sp ? si : se;
-    const SoAT<R> m = soa_as<R>(P.sp[sp].buf[st.cur]);
+    const Markers<R> mk{P.sp[sp].buf[st.cur]};
     const R vlim = K.vlim[sp];
     const bool limited = vlim < (R)INFINITY;
     unsigned long long* rho = reinterpret_cast<unsigned long long*>(P.rho_last[sp]);
     const uint32_t n = P.sp[sp].fill[st.cur][k];
     for (uint32_t i = lane; i < n; i += 32) {
-      const size_t o = (size_t)k * kTile + i;
-      const R vx = m.vx[o], vy = m.vy[o], vz = m.vz[o];
+      const Slot<R> m = mk.at(k, i);
+      const R vx = m.vx(), vy = m.vy(), vz = m.vz();
       const R b = limited ? beta_of(r_sqrt(vx * vx + vy * vy + vz * vz), vlim) : (R)1;
-      deposit(rho, m.cell[o], m.off[o], fixed_charge(b * m.wj[o], K.wscale));
+      deposit(rho, m.cell(), m.off(), fixed_charge(b * m.wj(), K.wscale));
     }
   }
 }
@@ -511,19 +508,11 @@ __global__ void __launch_bounds__(kMoveThreads) k_move(DeviceRefs r) {
     }
     __syncthreads();
     // one warp per tile, in order of the tiles
-    const SoAT<R> src = soa_as<R>(S.buf[x.src]), dst = soa_as<R>(S.buf[x.dst]);
+    const Markers<R> src{S.buf[x.src]}, dst{S.buf[x.dst]};
     for (int j = warp; j < kMoveChunkTiles; j += kMoveThreads / 32) {
       const uint32_t n = s_fill[j];
-      const size_t from = (size_t)(k0 + j) * kTile, to = s_pre[j];
-      for (uint32_t i = lane; i < n; i += 32) {
-        dst.cell[to + i] = src.cell[from + i];
-        dst.off[to + i] = src.off[from + i];
-        dst.vx[to + i] = src.vx[from + i];
-        dst.vy[to + i] = src.vy[from + i];
-        dst.vz[to + i] = src.vz[from + i];
-        dst.wj[to + i] = src.wj[from + i];
-        dst.id[to + i] = src.id[from + i];
-      }
+      const uint32_t to = s_pre[j];
+      for (uint32_t i = lane; i < n; i += 32) copy_marker(dst[to + i], src.at(k0 + j, i));
     }
     // fills of the repacked store: full tiles, the last one partial
     const uint32_t nt_new = (x.n_new + kTile - 1) / kTile;
@@ -553,7 +542,7 @@ __global__ void k_seed(DeviceRefs r, int inst, int sp, uint32_t base, uint32_t f
   const InstDev& P = r.inst[inst];
   const SpeciesDev& S = P.sp[sp];
   const StepConsts<R>& K = consts<R>(P);
-  const SoAT<R> d = soa_as<R>(S.buf[r.sstate[inst * 2 + sp].cur]);
+  const Markers<R> d{S.buf[r.sstate[inst * 2 + sp].cur]};
   const R ekin = (R)ekin_d, elo = (R)elo_d, lr = (R)lr_d, wj = (R)wj_d;
   const uint32_t id = first_id + i;
   R u[4];
@@ -599,14 +588,7 @@ __global__ void k_seed(DeviceRefs r, int inst, int sp, uint32_t base, uint32_t f
       vz = sig * (r2 * r_cos(a2));
     }
   }
-  const uint32_t o = base + i;
-  d.cell[o] = cell;
-  d.off[o] = off;
-  d.vx[o] = vx;
-  d.vy[o] = vy;
-  d.vz[o] = vz;
-  d.wj[o] = wj;
-  d.id[o] = id & kSerialMask;
+  write_marker(d[base + i], cell, off, vx, vy, vz, wj, id & kSerialMask);
 }
 
 void launch_seed(const DeviceRefs& r, int inst, int species, uint32_t base, uint32_t first_id,
@@ -623,38 +605,88 @@ void launch_seed(const DeviceRefs& r, int inst, int species, uint32_t base, uint
                                           lr, wj);
 }
 
-// Check loaded markers (cell in [0, N), offset in [0, 1), finite velocities,
-// non-negative weight below 2^39 charge units); records the smallest bad index in *bad and the
-// fixed-point sum of the weights in *wsum.
+// Copy a caller's markers into a tiled store and check them (cell in [0, N),
+// offset in [0, 1), finite velocities, non-negative weight below 2^39 charge
+// units); records the smallest bad index in *bad and the fixed-point sum of
+// the weights in *wsum.  One pass: each marker is read and written once.
 template <typename R>
-__global__ void k_validate(SoA dv, uint32_t n, int N, int shift, unsigned int* bad,
-                           unsigned long long* wsum) {
-  const SoAT<R> d = soa_as<R>(dv);
+__global__ void __launch_bounds__(256) k_place(SoAT<R> src, Markers<R> dst, uint32_t n, int N,
+                                               int shift, unsigned int* bad,
+                                               unsigned long long* wsum) {
   const R wscale = (R)ldexp(1.0, shift);  // 2^shift, exact
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   unsigned long long w = 0;
   if (i < n) {
-    const R o = d.off[i], x = d.vx[i], y = d.vy[i], z = d.vz[i], wj = d.wj[i];
-    const int c = d.cell[i];
+    const R o = src.f[0][i], x = src.f[1][i], y = src.f[2][i], z = src.f[3][i], wj = src.f[4][i];
+    const int c = src.cell[i];
     // the fixed-point weight must stay below 2^39 units so that the 24-bit
     // linear split of the deposit cannot overflow 64 bits
     const bool ok = c >= 0 && c < N && o >= (R)0 && o < (R)1 && isfinite(x) && isfinite(y) &&
                     isfinite(z) && wj >= (R)0 && wj * wscale < (R)549755813888.0;
     if (!ok) atomicMin(bad, i);
     else w = (unsigned long long)fixed_charge(wj, wscale);
+    write_marker(dst[i], c, o, x, y, z, wj, src.id[i]);
   }
   for (int o = 16; o > 0; o >>= 1) w += __shfl_down_sync(0xFFFFFFFFu, w, o);
   if ((threadIdx.x & 31) == 0 && w) atomicAdd(wsum, w);
 }
 
-void launch_validate(int fp64, const SoA& d, uint32_t n, int N, int shift, unsigned int* bad,
-                     unsigned long long* wsum, cudaStream_t s) {
+template <typename R>
+static void place(const void* const src[7], unsigned char* buf, uint32_t n, int N, int shift,
+                  unsigned int* bad, unsigned long long* wsum, cudaStream_t s) {
+  SoAT<R> a;
+  a.cell = static_cast<const int32_t*>(src[0]);
+  for (int k = 0; k < 5; ++k) a.f[k] = static_cast<const R*>(src[1 + k]);
+  a.id = static_cast<const uint32_t*>(src[6]);
+  k_place<R><<<(n + 255) / 256, 256, 0, s>>>(a, Markers<R>{buf}, n, N, shift, bad, wsum);
+}
+
+void launch_place(int fp64, const void* const src[7], unsigned char* buf, uint32_t n, int N,
+                  int shift, unsigned int* bad, unsigned long long* wsum, cudaStream_t s) {
   if (n == 0) return;
-  const int threads = 256;
-  if (fp64)
-    k_validate<double><<<(n + threads - 1) / threads, threads, 0, s>>>(d, n, N, shift, bad, wsum);
-  else
-    k_validate<float><<<(n + threads - 1) / threads, threads, 0, s>>>(d, n, N, shift, bad, wsum);
+  if (fp64) place<double>(src, buf, n, N, shift, bad, wsum, s);
+  else place<float>(src, buf, n, N, shift, bad, wsum, s);
+}
+
+// The live markers of a tiled store, in store order, into seven arrays (one
+// warp per tile).
+template <typename R>
+__global__ void __launch_bounds__(256) k_gather(Markers<R> src, const uint32_t* fill,
+                                                const uint32_t* prefix, uint32_t n_tiles,
+                                                int32_t* cell, R* off, R* vx, R* vy, R* vz,
+                                                R* wj, uint32_t* id) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (k >= n_tiles) return;
+  const uint32_t n = fill[k], to = prefix[k];
+  for (uint32_t i = lane; i < n; i += 32) {
+    const Slot<R> m = src.at(k, i);
+    const size_t o = to + i;
+    cell[o] = m.cell();
+    off[o] = m.off();
+    vx[o] = m.vx();
+    vy[o] = m.vy();
+    vz[o] = m.vz();
+    wj[o] = m.wj();
+    id[o] = m.id();
+  }
+}
+
+template <typename R>
+static void gather(const unsigned char* buf, const uint32_t* fill, const uint32_t* prefix,
+                   uint32_t n_tiles, void* const d[7], cudaStream_t s) {
+  k_gather<R><<<(n_tiles + 7) / 8, 256, 0, s>>>(
+      Markers<R>{const_cast<unsigned char*>(buf)}, fill, prefix, n_tiles,
+      static_cast<int32_t*>(d[0]), static_cast<R*>(d[1]), static_cast<R*>(d[2]),
+      static_cast<R*>(d[3]), static_cast<R*>(d[4]), static_cast<R*>(d[5]),
+      static_cast<uint32_t*>(d[6]));
+}
+
+void launch_gather(int fp64, const unsigned char* buf, const uint32_t* fill,
+                   const uint32_t* prefix, uint32_t n_tiles, void* const dst[7], cudaStream_t s) {
+  if (n_tiles == 0) return;
+  if (fp64) gather<double>(buf, fill, prefix, n_tiles, dst, s);
+  else gather<float>(buf, fill, prefix, n_tiles, dst, s);
 }
 
 __global__ void k_philox(uint32_t k0, uint32_t k1, const uint4* ctr, uint4* out, long long n) {

@@ -14,25 +14,35 @@ constexpr uint32_t kSerialMask = 0x7FFFFFFFu;
 constexpr uint32_t kSeedStep = 0xFFFFFFFFu;
 
 // Marker stores are sequences of tiles of kTile slots.  The particle kernel
-// gives every tile to one warp (kPerLane slots per lane: lane l holds slots
-// l, l + 32, ...); a CTA of up to kPushMaxWarps warps takes super-tiles of
-// one tile per warp, and each warp streams its tiles through kPushStages
-// shared-memory stages.
+// gives every tile to one warp, which advances it in kHalves passes of
+// kPerHalf neighbouring slots per lane; a warp streams its tiles through
+// kPushStages shared-memory stages.
 constexpr int kTile = 128;
 constexpr int kPerLane = kTile / 32;
 constexpr int kPushMaxWarps = 20;
 constexpr int kPushStages = 2;
-// The particle kernel advances a lane's kPerLane slots in kHalves passes.
 constexpr int kHalves = 2;
 constexpr int kPerHalf = kPerLane / kHalves;
-// Shared-memory stage of one tile: cell and id (4 bytes each), then the five
-// real streams (off, vx, vy, vz, w_j) of sizeof(R) bytes.
+// A tile is one block of memory: its seven fields in runs of kTile values, in
+// the order cell, off, vx, w_j, id, vy, vz (cell and id of 4 bytes, the others
+// reals).  All fields of a slot are at constant distances from one address,
+// and what a step of unlimited ions reads is the front of the block (up to vx,
+// or w_j when the step deposits; electrons need all): the particle kernel
+// fetches a tile with one bulk copy and forms one address per tile.  With the fields in seven
+// arrays of the whole store the copies and addresses took a quarter of its
+// instructions.
 template <typename R>
-__host__ __device__ constexpr int stage_bytes() {
-  return kTile * (8 + 5 * (int)sizeof(R));
+__host__ __device__ constexpr size_t tile_bytes() {
+  return kTile * (8 + 5 * sizeof(R));
 }
-// Relative cost of a super-tile of each species in the particle kernel's
-// static split of the super-tiles over the CTAs (ions draw no collision test).
+template <typename R>
+__host__ __device__ constexpr size_t tile_bytes_read(bool all, bool w) {
+  return all ? tile_bytes<R>() : kTile * (4 + (w ? 3 : 2) * sizeof(R));
+}
+// Relative cost of a tile of each species in the particle kernel's static
+// split of the tiles over the CTAs.  (4 : 5, and 4 : 8 under a speed limit,
+// nearer to the instruction counts, ran the same on shared-memory grids and
+// 18 % slower on a grid of 21832 cells, whose ions wait for global atomics.)
 constexpr unsigned int kWeightElectron = 3;
 constexpr unsigned int kWeightIon = 2;
 
@@ -87,28 +97,47 @@ struct TallyRec {
   double w_gain_gen0;
 };
 
-// Structure-of-arrays marker store in the arithmetic type R of the marker
-// path (float in FP32 contexts, double in FP64 contexts).  The device
-// descriptors hold the float view; kernels of an FP64 context take the double
-// view of the same pointers.
+// A caller's markers: one array per field, the five reals in the marker
+// path's type R (float in FP32 contexts, double in FP64 contexts).
 template <typename R>
 struct SoAT {
-  int32_t* cell;
-  R* off;
-  R* vx;
-  R* vy;
-  R* vz;
-  R* wj;
-  uint32_t* id;
+  const int32_t* cell;
+  const R* f[5];  // off, vx, vy, vz, w_j
+  const uint32_t* id;
 };
-using SoA = SoAT<float>;
 
+// The fields of one slot of a tiled store.
 template <typename R>
-__host__ __device__ inline SoAT<R> soa_as(const SoA& s) {
-  return SoAT<R>{s.cell, reinterpret_cast<R*>(s.off), reinterpret_cast<R*>(s.vx),
-                 reinterpret_cast<R*>(s.vy), reinterpret_cast<R*>(s.vz),
-                 reinterpret_cast<R*>(s.wj), s.id};
-}
+struct Slot {
+  int32_t* c;
+  R* r;
+  static constexpr int kPer4 = sizeof(R) / 4;        // 4-byte words per real
+  static constexpr int kV = 3 * kTile + kTile / kPer4;  // reals from off to vy
+  __host__ __device__ __forceinline__ int32_t& cell() const { return c[0]; }
+  __host__ __device__ __forceinline__ R& off() const { return r[0]; }
+  __host__ __device__ __forceinline__ R& vx() const { return r[kTile]; }
+  __host__ __device__ __forceinline__ R& wj() const { return r[2 * kTile]; }
+  __host__ __device__ __forceinline__ uint32_t& id() const {
+    return reinterpret_cast<uint32_t*>(c)[kTile + 3 * kTile * kPer4];
+  }
+  __host__ __device__ __forceinline__ R& vy() const { return r[kV]; }
+  __host__ __device__ __forceinline__ R& vz() const { return r[kV + kTile]; }
+};
+
+// A tiled store in the marker path's type.
+template <typename R>
+struct Markers {
+  unsigned char* b;
+  // slot i of tile k
+  __host__ __device__ __forceinline__ Slot<R> at(size_t k, uint32_t i) const {
+    unsigned char* p = b + k * tile_bytes<R>();
+    return Slot<R>{reinterpret_cast<int32_t*>(p) + i, reinterpret_cast<R*>(p + kTile * 4) + i};
+  }
+  // slot o of the store
+  __host__ __device__ __forceinline__ Slot<R> operator[](uint32_t o) const {
+    return at(o / kTile, o % kTile);
+  }
+};
 
 // Processes of an electron collision: elastic, up to three excitation
 // levels, ionization.
@@ -133,6 +162,7 @@ struct StepConsts {
   R K_E;          // m_e / (2 e): eV per (m/s)^2
   R ndt;          // n_g dt
   R P0;           // null-collision majorant probability
+  uint32_t cand_thr;  // a draw's top 23 bits are below it exactly when u < P0
   R vb_cap;       // cap of beta v in the majorant
   R R2;           // 2 m_e / M
   R e_ex[kMaxExc];  // excitation thresholds [eV]
@@ -196,9 +226,10 @@ constexpr uint32_t kIonizedMark = 0x80000000u;
 
 // Configuration of one species of one instance (constant during a run).
 struct SpeciesDev {
-  SoA buf[2];         // tiled marker store (cap_tiles * kTile slots each)
+  unsigned char* buf[2];  // tiled marker store (cap_tiles tiles each; see Markers)
   uint32_t* fill[2];  // [cap_tiles] live markers per tile of each buffer
-  SoA stage_b;        // electrons only: emission births, slot = ion tile * kTile + rank
+  void* stage_w;      // electrons only: w_j of the electrons emitted at the cathode
+                      // (at rest at x = 0), slot = ion tile * kTile + rank
   uint32_t* births;   // ions: [cap_tiles] electrons emitted by each tile in the step
   void* crec;         // electrons: [cap_tiles * kTile] CandRec<R>, the tile's
                       // null-collision candidates in slot order
@@ -256,7 +287,7 @@ struct InstState {
 // Global state of the batched step.
 struct Control {
   unsigned int epoch;        // step epoch of the look-back records
-  unsigned int n_super;      // particle-kernel super-tiles this step
+  unsigned int n_tiles;      // particle-kernel tiles this step
   unsigned int w_total;      // their summed weights
   unsigned int n_seg;        // segments = instances * 2
   unsigned int finish_done;  // CTAs of the finish kernel that completed
@@ -306,8 +337,8 @@ struct DeviceRefs {
   SpeciesState* sstate;   // [n_inst * 2]
   Transfer* xfer;         // [n_inst * 2]
   Control* ctrl;
-  unsigned int* seg_start;   // [n_seg + 1] first super-tile of each segment
-  unsigned int* seg_wstart;  // [n_seg + 1] summed super-tile weights before each segment
+  unsigned int* seg_start;   // [n_seg + 1] first tile of each segment
+  unsigned int* seg_wstart;  // [n_seg + 1] summed tile weights before each segment
   unsigned int* coll_start;  // [n_inst + 1] first collision chunk of each instance
   unsigned int* coll_tiles;  // [n_inst] tiles per electron collision chunk
   unsigned int* move_start;  // [n_seg + 1] first repacking chunk of each segment
@@ -315,7 +346,7 @@ struct DeviceRefs {
   ChunkStatus* move_scan;    // [max repacking chunks]
   int n_inst;
   int smem_nodes;         // deposit grid nodes in shared memory (0: global atomics)
-  int push_warps;         // warps per particle-kernel CTA = tiles per super-tile
+  int push_warps;         // warps per particle-kernel CTA
   int fp64;               // marker path in double precision (else float)
   int finish_net_nodes;   // k_finish keeps the net deposit of up to this many nodes in shared memory
 };
@@ -323,8 +354,8 @@ struct DeviceRefs {
 // Launchers (defined in the .cu files).
 void launch_push(const DeviceRefs& r, int grid, cudaStream_t s);
 // Particle-kernel shape for a shared-memory deposit grid of smem_nodes nodes:
-// warps per CTA, resident CTAs per SM and dynamic shared memory per CTA.
-int push_config(int fp64, int smem_nodes, int* warps, int* blocks_per_sm, size_t* smem_bytes);
+// warps per CTA and resident CTAs per SM.
+int push_config(int fp64, int smem_nodes, int* warps, int* blocks_per_sm);
 // Resident particle-kernel CTAs per SM for `warps` warps per CTA.
 int push_blocks_per_sm(int fp64, int warps, int smem_nodes, int* blocks_per_sm);
 // mode 0: finish a step and plan the next; mode 1: plan only (one CTA).
@@ -347,8 +378,16 @@ int collide_config();
 void launch_seed(const DeviceRefs& r, int inst, int species, uint32_t base, uint32_t first_id,
                  uint32_t n, int mode, double e0, double e_lo, double lr, double wj,
                  cudaStream_t s);
-void launch_validate(int fp64, const SoA& d, uint32_t n, int N, int shift, unsigned int* bad,
-                     unsigned long long* wsum, cudaStream_t s);
+// Copy n markers of a caller's arrays on the device (field order: cell, off,
+// vx, vy, vz, w_j, id) into slots 0 .. n - 1 of a tiled store, checking them:
+// *bad gets the smallest index of a marker that must not be stepped, *wsum the
+// fixed-point sum of the weights.
+void launch_place(int fp64, const void* const src[7], unsigned char* buf, uint32_t n, int N,
+                  int shift, unsigned int* bad, unsigned long long* wsum, cudaStream_t s);
+// The reverse: the live markers of n_tiles tiles, in store order, into seven
+// arrays (prefix: live markers before each tile).
+void launch_gather(int fp64, const unsigned char* buf, const uint32_t* fill,
+                   const uint32_t* prefix, uint32_t n_tiles, void* const dst[7], cudaStream_t s);
 int philox_preload();
 void launch_philox(uint32_t k0, uint32_t k1, const uint32_t* ctr, uint32_t* out,
                    long long n, cudaStream_t s);

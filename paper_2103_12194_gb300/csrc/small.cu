@@ -82,17 +82,16 @@ __device__ void deposit_all(const InstDev& P, const SmallShared& sh, unsigned lo
   const int ne = (int)sh.st[0].n_tiles, n_items = ne + (int)sh.st[1].n_tiles;
   for (int it = warp; it < n_items; it += kSmallWarps) {
     const int sp = it < ne ? 0 : 1, k = it < ne ? it : it - ne;
-    const SoAT<R> m = soa_as<R>(P.sp[sp].buf[sh.st[sp].cur]);
+    const Markers<R> mk{P.sp[sp].buf[sh.st[sp].cur]};
     const R vlim = K.vlim[sp];
     const bool limited = vlim < (R)INFINITY;
     unsigned long long* rho = sp ? rho1 : rho0;
     const uint32_t n = sh.fill[sp][k];
-    const size_t base = (size_t)k * kTile;
     for (uint32_t i = lane; i < n; i += 32) {
-      const size_t o = base + i;
-      const R vx = m.vx[o], vy = m.vy[o], vz = m.vz[o];
+      const Slot<R> m = mk.at(k, i);
+      const R vx = m.vx(), vy = m.vy(), vz = m.vz();
       const R b = limited ? beta_of(r_sqrt(vx * vx + vy * vy + vz * vz), vlim) : (R)1;
-      deposit(rho, m.cell[o], m.off[o], fixed_charge(b * m.wj[o], K.wscale));
+      deposit(rho, m.cell(), m.off(), fixed_charge(b * m.wj(), K.wscale));
     }
   }
 }
@@ -219,7 +218,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
       for (int it = warp; it < n_items; it += kSmallWarps) {
         const int sp = it < ne ? 0 : 1, kt = it < ne ? it : it - ne;
         const SpeciesDev& S = P.sp[sp];
-        const SoAT<R> m = soa_as<R>(S.buf[sh.st[sp].cur]);
+        const Markers<R> mk{S.buf[sh.st[sp].cur]};
         const uint32_t fill = sh.fill[sp][kt];
         const size_t tbase = (size_t)kt * kTile;
         uint32_t n_surv = 0, n_event = 0;
@@ -231,14 +230,14 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
         for (int j = 0; j < kPerLane; ++j) {
           const int i = j * 32 + lane;
           live[j] = i < (int)fill;
-          const size_t o = tbase + i;
-          cell[j] = live[j] ? m.cell[o] : 0;
-          off[j] = live[j] ? m.off[o] : (R)0;
-          vx[j] = live[j] ? m.vx[o] : (R)0;
-          vy[j] = live[j] ? m.vy[o] : (R)0;
-          vz[j] = live[j] ? m.vz[o] : (R)0;
-          wj[j] = live[j] ? m.wj[o] : (R)0;
-          id[j] = live[j] ? m.id[o] : 0u;
+          const Slot<R> m = mk.at(kt, i);
+          cell[j] = live[j] ? m.cell() : 0;
+          off[j] = live[j] ? m.off() : (R)0;
+          vx[j] = live[j] ? m.vx() : (R)0;
+          vy[j] = live[j] ? m.vy() : (R)0;
+          vz[j] = live[j] ? m.vz() : (R)0;
+          wj[j] = live[j] ? m.wj() : (R)0;
+          id[j] = live[j] ? m.id() : 0u;
         }
         const R qmdt = K.qmdt[sp], vlim = K.vlim[sp], dtdx = K.dtdx, P0 = K.P0;
         const uint32_t Nc = (uint32_t)N;
@@ -334,20 +333,13 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
         for (int j = 0; j < kPerLane; ++j) {
           if (!alive[j]) continue;
           if (!compact) {
-            const size_t o = tbase + j * 32 + lane;
-            m.cell[o] = cell[j];
-            m.off[o] = off[j];
-            m.vx[o] = vx[j];
+            const Slot<R> m = mk.at(kt, j * 32 + lane);
+            m.cell() = cell[j];
+            m.off() = off[j];
+            m.vx() = vx[j];
           } else {
-            const size_t o =
-                tbase + pre_alive[j] + (uint32_t)__popc(b_alive[j] & lanemask_lt);
-            m.cell[o] = cell[j];
-            m.off[o] = off[j];
-            m.vx[o] = vx[j];
-            m.vy[o] = vy[j];
-            m.vz[o] = vz[j];
-            m.wj[o] = wj[j];
-            m.id[o] = id[j];
+            write_marker(mk.at(kt, pre_alive[j] + (uint32_t)__popc(b_alive[j] & lanemask_lt)),
+                         cell[j], off[j], vx[j], vy[j], vz[j], wj[j], id[j]);
           }
         }
         if (lane == 0) {
@@ -366,8 +358,8 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
     }
     __syncthreads();
     const SpeciesState se = sh.st[0], si = sh.st[1];
-    const SoAT<R> me = soa_as<R>(E.buf[se.cur]);
-    const SoAT<R> mi = soa_as<R>(I.buf[si.cur]);
+    const Markers<R> me{E.buf[se.cur]};
+    const Markers<R> mi{I.buf[si.cur]};
     const uint32_t app_e = se.n_tiles ? (se.n_tiles - 1) * (uint32_t)kTile + sh.fill[0][se.n_tiles - 1] : 0u;
     const uint32_t app_i = si.n_tiles ? (si.n_tiles - 1) * (uint32_t)kTile + sh.fill[1][si.n_tiles - 1] : 0u;
     const uint32_t cap_e = E.cap_tiles * (uint32_t)kTile, cap_i = I.cap_tiles * (uint32_t)kTile;
@@ -401,9 +393,10 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
                                           cr.wj, sh.acc, &e2, &proc);
         if (proc < 3) ++n_proc[proc];
         if (proc < 3) {
-          me.vx[o] = nv.vx;
-          me.vy[o] = nv.vy;
-          me.vz[o] = nv.vz;
+          const Slot<R> m = me[(uint32_t)o];
+          m.vx() = nv.vx;
+          m.vy() = nv.vy;
+          m.vz() = nv.vz;
           if (proc == 2) {
             flags |= (unsigned __int128)1 << (16 * u);
             es[u] = e2;
@@ -441,15 +434,16 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
           if (pe >= cap_e || pi >= cap_i) {
             atomicCAS(&ctrl->error, 0, kErrCapacity);
           } else {
-            born_pair<R, false>(P, me, mi, pe, pi, me.cell[o], me.off[o], me.wj[o], me.id[o],
-                                step, es[u], se.next_id + rank, si.next_id + rank);
+            const Slot<R> m = me[o];
+            born_pair<R, false>(P, me[pe], mi[pi], m.cell(), m.off(), m.wj(), m.id(), step,
+                                es[u], se.next_id + rank, si.next_id + rank);
           }
         }
         before += (uint32_t)(rows >> (16 * u)) & 0xFFFFu;
       }
       // electrons emitted at the cathode, after every ionization electron
       const uint32_t n_ionz = before;
-      const SoAT<R> sb = soa_as<R>(E.stage_b);
+      const R* sw = reinterpret_cast<const R*>(E.stage_w);
       for (uint32_t e = t; e < sh.tot[1]; e += kSmallThreads) {
         const int j = tile_of_event(sh.pre[1], (int)si.n_tiles, e);
         const size_t o = (size_t)j * kTile + (e - sh.pre[1][j]);
@@ -459,13 +453,8 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
           atomicCAS(&ctrl->error, 0, kErrCapacity);
           continue;
         }
-        me.cell[pe] = sb.cell[o];
-        me.off[pe] = sb.off[o];
-        me.vx[pe] = sb.vx[o];
-        me.vy[pe] = sb.vy[o];
-        me.vz[pe] = sb.vz[o];
-        me.wj[pe] = sb.wj[o];
-        me.id[pe] = kGenBit | ((se.next_id + rank) & kSerialMask);
+        write_marker(me[pe], 0, (R)0, (R)0, (R)0, (R)0, sw[o],
+                     kGenBit | ((se.next_id + rank) & kSerialMask));
       }
     }
     __syncthreads();
@@ -506,19 +495,11 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
       if (warp == 0) warp_prefix(sh.fill[sp], (int)sh.nt[sp], sh.pre[sp]);
       __syncthreads();
       const SpeciesDev& S = P.sp[sp];
-      const SoAT<R> src = soa_as<R>(S.buf[sh.st[sp].cur]), dst = soa_as<R>(S.buf[sh.st[sp].cur ^ 1u]);
+      const Markers<R> src{S.buf[sh.st[sp].cur]}, dst{S.buf[sh.st[sp].cur ^ 1u]};
       for (uint32_t k = warp; k < sh.nt[sp]; k += kSmallWarps) {
         const uint32_t n = sh.fill[sp][k];
-        const size_t from = (size_t)k * kTile, to = sh.pre[sp][k];
-        for (uint32_t i = lane; i < n; i += 32) {
-          dst.cell[to + i] = src.cell[from + i];
-          dst.off[to + i] = src.off[from + i];
-          dst.vx[to + i] = src.vx[from + i];
-          dst.vy[to + i] = src.vy[from + i];
-          dst.vz[to + i] = src.vz[from + i];
-          dst.wj[to + i] = src.wj[from + i];
-          dst.id[to + i] = src.id[from + i];
-        }
+        const uint32_t to = sh.pre[sp][k];
+        for (uint32_t i = lane; i < n; i += 32) copy_marker(dst[to + i], src.at(k, i));
       }
       __syncthreads();
       const uint32_t nt_new = (sh.n_new[sp] + kTile - 1) / kTile;

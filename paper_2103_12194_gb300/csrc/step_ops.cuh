@@ -45,18 +45,11 @@ __device__ __noinline__ bool absorb(const InstDev& P, int sp, int side, R wj, ui
   return true;
 }
 
-// Stage an electron emitted at the cathode (x = 0, at rest, the ion's w_j);
-// with kDeposit, deposit it too.
+// Stage an electron emitted at the cathode (x = 0, at rest: only the ion's
+// w_j is kept); with kDeposit, deposit it too.
 template <typename R, bool kDeposit = true>
 __device__ __noinline__ void stage_emission(const InstDev& P, size_t o, R wj) {
-  const SoAT<R> sb = soa_as<R>(P.sp[kElectron].stage_b);
-  sb.cell[o] = 0;
-  sb.off[o] = (R)0;
-  sb.vx[o] = (R)0;
-  sb.vy[o] = (R)0;
-  sb.vz[o] = (R)0;
-  sb.wj[o] = wj;
-  sb.id[o] = kGenBit;
+  reinterpret_cast<R*>(P.sp[kElectron].stage_w)[o] = wj;
   // at rest: beta = 1, all the charge on node 0
   if (kDeposit)
     atomicAdd(P.rho_acc[kElectron], (unsigned long long)fixed_charge(wj, consts<R>(P).wscale));
@@ -255,14 +248,29 @@ __device__ __noinline__ Velocity<R> collide(const InstDev& P, R kv, R vlim, R vx
   return {vx, vy, vz};
 }
 
-// Write the electron and Ar+ born by an ionization at slots pe (electron
-// store) and pi (ion store) with their serial numbers, and (kDeposit) deposit
+template <typename R>
+__device__ __forceinline__ void write_marker(const Slot<R>& d, int cell, R off, R vx, R vy, R vz,
+                                             R wj, uint32_t id) {
+  d.cell() = cell;
+  d.off() = off;
+  d.vx() = vx;
+  d.vy() = vy;
+  d.vz() = vz;
+  d.wj() = wj;
+  d.id() = id;
+}
+
+template <typename R>
+__device__ __forceinline__ void copy_marker(const Slot<R>& d, const Slot<R>& m) {
+  write_marker(d, m.cell(), m.off(), m.vx(), m.vy(), m.vz(), m.wj(), m.id());
+}
+
+// Write the electron and Ar+ born by an ionization to their slots with their serial numbers, and (kDeposit) deposit
 // both.  The secondary gets energy es along an isotropic direction (block 1
 // of the primary's draws); the ion a gas-temperature Maxwellian (Box-Muller
 // on block 2).
 template <typename R, bool kDeposit = true>
-__device__ void born_pair(const InstDev& P, const SoAT<R>& me, const SoAT<R>& mi, uint32_t pe,
-                          uint32_t pi, int cell, R off, R wj, uint32_t id, uint32_t step, R es,
+__device__ void born_pair(const InstDev& P, const Slot<R>& me, const Slot<R>& mi, int cell, R off, R wj, uint32_t id, uint32_t step, R es,
                           uint32_t serial_e, uint32_t serial_i) {
   const StepConsts<R>& K = consts<R>(P);
   const uint32_t gen = id & kGenBit;
@@ -270,13 +278,7 @@ __device__ void born_pair(const InstDev& P, const SoAT<R>& me, const SoAT<R>& mi
   R bx, by, bz;
   isotropic(r_sqrt(es * K.K_V[kElectron]), uniform01r<R>(r1.y), uniform01r<R>(r1.z), K.two_pi,
             bx, by, bz);
-  me.cell[pe] = cell;
-  me.off[pe] = off;
-  me.vx[pe] = bx;
-  me.vy[pe] = by;
-  me.vz[pe] = bz;
-  me.wj[pe] = wj;
-  me.id[pe] = gen | (serial_e & kSerialMask);
+  write_marker(me, cell, off, bx, by, bz, wj, gen | (serial_e & kSerialMask));
   if (kDeposit)
     deposit(P.rho_acc[kElectron], cell, off,
             fixed_charge(beta_of(r_sqrt(bx * bx + by * by + bz * bz), K.vlim[kElectron]) * wj,
@@ -290,13 +292,7 @@ __device__ void born_pair(const InstDev& P, const SoAT<R>& me, const SoAT<R>& mi
   const R ix = K.sigT_ion * (rr1 * r_cos(a1));
   const R iy = K.sigT_ion * (rr1 * r_sin(a1));
   const R iz = K.sigT_ion * (rr2 * r_cos(a2));
-  mi.cell[pi] = cell;
-  mi.off[pi] = off;
-  mi.vx[pi] = ix;
-  mi.vy[pi] = iy;
-  mi.vz[pi] = iz;
-  mi.wj[pi] = wj;
-  mi.id[pi] = gen | (serial_i & kSerialMask);
+  write_marker(mi, cell, off, ix, iy, iz, wj, gen | (serial_i & kSerialMask));
   if (kDeposit)
     deposit(P.rho_acc[kIon], cell, off,
             fixed_charge(beta_of(r_sqrt(ix * ix + iy * iy + iz * iz), K.vlim[kIon]) * wj,
@@ -308,18 +304,6 @@ __device__ void born_pair(const InstDev& P, const SoAT<R>& me, const SoAT<R>& mi
 __device__ __forceinline__ uint32_t tail_slot(const SpeciesDev& S, const SpeciesState& st) {
   return st.n_tiles ? (st.n_tiles - 1) * (uint32_t)kTile + S.fill[st.cur][st.n_tiles - 1]
                     : 0u;
-}
-
-template <typename R>
-__device__ __forceinline__ void write_marker(const SoAT<R>& d, size_t o, int cell, R off, R vx,
-                                             R vy, R vz, R wj, uint32_t id) {
-  d.cell[o] = cell;
-  d.off[o] = off;
-  d.vx[o] = vx;
-  d.vy[o] = vy;
-  d.vz[o] = vz;
-  d.wj[o] = wj;
-  d.id[o] = id;
 }
 
 // Record of null-collision candidate i of an electron store (the tile's
