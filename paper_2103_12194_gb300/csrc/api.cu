@@ -436,15 +436,15 @@ int commit(slpic_ctx* c) {
   }
   void* blk;
   const size_t nseg = 2 * (size_t)c->n_inst;
-  // ordered-scan records: at most one chunk per kCollMinChunkTiles
-  // (kMoveChunkTiles) tiles of every store, plus one partial chunk per store
-  const size_t coll_chunks = total_tiles / kCollMinChunkTiles + nseg + 2;
+  // ordered-scan records: at most one chunk per tile (kMoveChunkTiles tiles) of
+  // every store, plus one partial chunk per store
+  const size_t coll_chunks = total_tiles + nseg + 2;
   const size_t move_chunks = total_tiles / kMoveChunkTiles + nseg + 2;
   size_t bytes = ((sizeof(InstDev) * c->n_inst + 255) & ~size_t(255)) +
                  ((sizeof(InstState) * c->n_inst + 255) & ~size_t(255)) +
                  ((sizeof(SpeciesState) * nseg + 255) & ~size_t(255)) +
                  ((sizeof(Transfer) * nseg + 255) & ~size_t(255)) + 256 +
-                 5 * ((4 * (nseg + 1) + 255) & ~size_t(255)) + 256 +
+                 6 * ((4 * (nseg + 1) + 255) & ~size_t(255)) + 256 +
                  ((sizeof(ChunkStatus) * coll_chunks + 255) & ~size_t(255)) +
                  ((sizeof(ChunkStatus) * move_chunks + 255) & ~size_t(255));
   if (int rc = dmalloc(c, &blk, bytes, "control")) return rc;
@@ -461,6 +461,7 @@ int commit(slpic_ctx* c) {
   c->refs.coll_start = carve<unsigned int>(p, nseg + 1);
   c->refs.move_start = carve<unsigned int>(p, nseg + 1);
   c->refs.coll_tiles = carve<unsigned int>(p, nseg + 1);
+  c->refs.coll_room = carve<unsigned int>(p, nseg + 1);
   c->refs.coll_scan = carve<ChunkStatus>(p, coll_chunks);
   c->refs.move_scan = carve<ChunkStatus>(p, move_chunks);
   c->refs.inst = c->d_inst;
@@ -474,15 +475,15 @@ int commit(slpic_ctx* c) {
   {
     // first step's electron collision chunks from the majorant probability:
     // about P0 kTile candidates per full tile
-    std::vector<unsigned int> t(c->n_inst, (unsigned int)kCollMaxChunkTiles);
+    std::vector<unsigned int> t(c->n_inst, (unsigned int)kCollMaxRoom);
     for (int i = 0; i < c->n_inst; ++i) {
       const double P0 = c->fp64 ? c->h_inst[i].c64.P0 : (double)c->h_inst[i].c32.P0;
       const double per_tile = P0 * kTile;
-      while (t[i] > (unsigned int)kCollMinChunkTiles &&
+      while (t[i] > (unsigned int)kCollWarps &&
              t[i] / kCollWarps * per_tile > kCollTargetPerWarp)
         t[i] >>= 1;
     }
-    CK(cudaMemcpy(c->refs.coll_tiles, t.data(), t.size() * 4, cudaMemcpyHostToDevice),
+    CK(cudaMemcpy(c->refs.coll_room, t.data(), t.size() * 4, cudaMemcpyHostToDevice),
        "control");
   }
   c->refs.seg_start = c->d_seg;

@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(kCollThreads, 4) k_collide(DeviceRefs r) {
     const uint32_t nt = ion_chunk ? si.n_tiles : se.n_tiles;
     // this warp's tiles: wt consecutive ones, tile kw + j at lane j
     const uint32_t T = ion_chunk ? (uint32_t)kCollMaxChunkTiles : Te;
-    const uint32_t wt = T / kCollWarps;
+    const uint32_t wt = T >= (uint32_t)kCollWarps ? T / kCollWarps : (warp < (int)T ? 1u : 0u);
     const uint32_t kw = (ion_chunk ? local - e_chunks : local) * T + warp * wt;
     const Markers<R> me{E.buf[se.cur]};
     const StepConsts<R>& K = consts<R>(P);
@@ -430,9 +430,7 @@ static_assert(kCollThreads == 32 * kCollWarps, "kCollWarps warps per chunk");
 static_assert(kCollMaxChunkTiles / kCollWarps <= 32, "per-tile counts live one per lane");
 static_assert(kTile <= 128 && kCollMaxChunkTiles / kCollWarps <= 32,
               "pack_idx: 5 bits of tile, 7 of rank, 7 of slot");
-static_assert((kCollMinChunkTiles & (kCollMinChunkTiles - 1)) == 0 &&
-                  kCollMinChunkTiles % kCollWarps == 0,
-              "chunk sizes are powers of two of whole warps");
+static_assert((kCollWarps & (kCollWarps - 1)) == 0, "chunk sizes are powers of two");
 static_assert((uint32_t)kTile < kIonizedMark, "candidate slots leave the top bit for the ionization mark");
 
 }  // namespace slpic

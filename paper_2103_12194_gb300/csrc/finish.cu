@@ -52,6 +52,19 @@ __device__ __forceinline__ void plan_totals(const DeviceRefs& r, int n_seg, unsi
   r.ctrl->finish_done = 0;
 }
 
+// Tiles per electron collision chunk of an instance of n_tiles electron tiles:
+// `room` of them hold kCollTargetPerWarp candidates per warp.  Fewer where the
+// instance would not give its share of kCollSpread chunks, but not below an
+// eighth of room (a round of 32 candidates per warp) in float.
+__device__ __forceinline__ unsigned int chunk_tiles(unsigned long long room, uint32_t n_tiles,
+                                                    int n_inst, int fp64) {
+  const unsigned long long share = (unsigned long long)n_tiles * n_inst / kCollSpread;
+  const unsigned long long most = min(room, max(share, fp64 ? 1ull : room / 8u));
+  unsigned int T = kCollMaxChunkTiles;
+  while (T > 1u && T > most) T >>= 1;
+  return T;
+}
+
 // The plan below by one warp (n_seg <= 32 kPlanPerLane), with shuffle scans
 // and no block barrier.
 __device__ void plan_next_warp(const DeviceRefs& r) {
@@ -78,7 +91,9 @@ __device__ void plan_next_warp(const DeviceRefs& r) {
     const int i = lane * (kPlanPerLane / 2) + j;
     nc[j] = 0;
     if (i < r.n_inst) {
-      const long long T = r.coll_tiles[i];
+      const long long T = chunk_tiles(r.coll_room[i], r.sstate[2 * i].n_tiles, r.n_inst,
+                                      r.fp64);
+      r.coll_tiles[i] = (unsigned int)T;
       nc[j] = ((long long)r.sstate[2 * i].n_tiles + T - 1) / T +
               ((long long)r.sstate[2 * i + 1].n_tiles + kCollMaxChunkTiles - 1) /
                   kCollMaxChunkTiles;
@@ -153,7 +168,9 @@ __device__ void plan_next(const DeviceRefs& r, long long* s_buf) {
     const int i = base + t;
     long long nc = 0;
     if (i < r.n_inst) {
-      const long long T = r.coll_tiles[i];
+      const long long T = chunk_tiles(r.coll_room[i], r.sstate[2 * i].n_tiles, r.n_inst,
+                                      r.fp64);
+      r.coll_tiles[i] = (unsigned int)T;
       nc = ((long long)r.sstate[2 * i].n_tiles + T - 1) / T +
            ((long long)r.sstate[2 * i + 1].n_tiles + kCollMaxChunkTiles - 1) / kCollMaxChunkTiles;
     }
@@ -258,16 +275,14 @@ __global__ void __launch_bounds__(kFinThreads) k_finish(DeviceRefs r, int mode, 
     x.tail = tail;
     x.end = end;
     if (sp == kElectron) {
-      // electron collision chunks of the next step: the largest power of two
-      // (tiles) with about kCollTargetPerWarp candidates per warp at this
-      // step's candidates per tile
+      // tiles of an electron collision chunk of the next step: about
+      // kCollTargetPerWarp candidates per warp at this step's candidates per tile
       const unsigned long long cand = s_acc[ACC_CAND];
       const unsigned long long room =
           cand ? (unsigned long long)kCollTargetPerWarp * kCollWarps * s0.n_tiles / cand
-               : (unsigned long long)kCollMaxChunkTiles;
-      unsigned int T = kCollMaxChunkTiles;
-      while (T > (unsigned int)kCollMinChunkTiles && T > room) T >>= 1;
-      r.coll_tiles[inst] = T;
+               : (unsigned long long)kCollMaxRoom;
+      r.coll_room[inst] = (unsigned int)min(max(room, (unsigned long long)kCollWarps),
+                                            (unsigned long long)kCollMaxRoom);
     }
     SpeciesState s1;
     s1.cur = x.dst;

@@ -316,15 +316,22 @@ struct ChunkStatus {
 };
 
 // Collision chunks: kCollWarps warps of T / kCollWarps consecutive tiles
-// each.  Electron chunks have T = coll_tiles[inst] tiles, a power of two in
-// [kCollMinChunkTiles, kCollMaxChunkTiles] chosen from the instance's last
-// step so that a warp meets about kCollTargetPerWarp candidates (many
-// collisions per step: small chunks, more warps); ion chunks (the electrons
-// emitted at the cathode, rare) have kCollMaxChunkTiles.  Repacking chunks:
-// kMoveChunkTiles tiles.
+// each (below kCollWarps tiles, one tile for each of the first T warps).
+// Electron chunks have T = coll_tiles[inst] tiles, a power of two up to
+// kCollMaxChunkTiles: small enough that a warp meets about kCollTargetPerWarp
+// candidates at the instance's last step's density (many collisions per step:
+// small chunks, more warps), and, down to a round of 32 candidates per warp
+// (in double, where the FP64 unit of each SM counts, down to one tile), that
+// the instance gives its share of kCollSpread chunks (two per SM: with few
+// tiles, fewer per CTA, so that every SM has some; 1e5 electrons of a 256-cell
+// gap: k_collide 36 -> 19 us, in double 487 -> 55 us).
+// Ion chunks (the electrons emitted at the cathode, rare) have
+// kCollMaxChunkTiles.  Repacking chunks: kMoveChunkTiles tiles.
 constexpr int kCollWarps = 8;
 constexpr int kCollMaxChunkTiles = kCollWarps * 32;
-constexpr int kCollMinChunkTiles = kCollWarps;
+// (a bound of the tiles that hold that many candidates per warp)
+constexpr int kCollMaxRoom = 64 * kCollMaxChunkTiles;
+constexpr int kCollSpread = 304;
 constexpr int kCollTargetPerWarp = 256;
 constexpr int kMoveChunkTiles = 128;
 // Single-CTA path (small.cu): at most this many tiles per store and instance
@@ -341,6 +348,7 @@ struct DeviceRefs {
   unsigned int* seg_wstart;  // [n_seg + 1] summed tile weights before each segment
   unsigned int* coll_start;  // [n_inst + 1] first collision chunk of each instance
   unsigned int* coll_tiles;  // [n_inst] tiles per electron collision chunk
+  unsigned int* coll_room;   // [n_inst] the most its density of candidates allows
   unsigned int* move_start;  // [n_seg + 1] first repacking chunk of each segment
   ChunkStatus* coll_scan;    // [max collision chunks]
   ChunkStatus* move_scan;    // [max repacking chunks]
