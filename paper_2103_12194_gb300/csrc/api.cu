@@ -97,7 +97,8 @@ struct slpic_ctx {
   // with more warps deposit to global memory
   int smem_nodes_full = 0;
   int max_push_warps_smem = 0;
-  int collide_per_sm = 8;  // collision CTAs per SM
+  int collide_per_sm = 8;    // collision CTAs per SM (no more than are resident are launched)
+  int collide_resident = 1;  // those that an SM holds at once
   int small_limit = kSmallMaxTiles;  // single-CTA path: most tiles per store (0: off)
   // per instance: stepped since its field was last reset (phi is then formed
   // from the last deposit when read)
@@ -436,16 +437,17 @@ int commit(slpic_ctx* c) {
   }
   void* blk;
   const size_t nseg = 2 * (size_t)c->n_inst;
-  // ordered-scan records: at most one chunk per tile (kMoveChunkTiles tiles) of
-  // every store, plus one partial chunk per store
-  const size_t coll_chunks = total_tiles + nseg + 2;
+  // collision items: at most one per tile of every store; ordered-scan records:
+  // at most one chunk per kMoveChunkTiles tiles, plus one partial per store
+  const size_t coll_items = total_tiles + nseg + 2;
   const size_t move_chunks = total_tiles / kMoveChunkTiles + nseg + 2;
   size_t bytes = ((sizeof(InstDev) * c->n_inst + 255) & ~size_t(255)) +
                  ((sizeof(InstState) * c->n_inst + 255) & ~size_t(255)) +
                  ((sizeof(SpeciesState) * nseg + 255) & ~size_t(255)) +
                  ((sizeof(Transfer) * nseg + 255) & ~size_t(255)) + 256 +
                  6 * ((4 * (nseg + 1) + 255) & ~size_t(255)) + 256 +
-                 ((sizeof(ChunkStatus) * coll_chunks + 255) & ~size_t(255)) +
+                 ((4 * coll_items + 255) & ~size_t(255)) +
+                 ((sizeof(BirthBase) * c->n_inst + 255) & ~size_t(255)) +
                  ((sizeof(ChunkStatus) * move_chunks + 255) & ~size_t(255));
   if (int rc = dmalloc(c, &blk, bytes, "control")) return rc;
   CK(cudaMemset(blk, 0, bytes), "control");
@@ -462,7 +464,8 @@ int commit(slpic_ctx* c) {
   c->refs.move_start = carve<unsigned int>(p, nseg + 1);
   c->refs.coll_tiles = carve<unsigned int>(p, nseg + 1);
   c->refs.coll_room = carve<unsigned int>(p, nseg + 1);
-  c->refs.coll_scan = carve<ChunkStatus>(p, coll_chunks);
+  c->refs.item_births = carve<uint32_t>(p, coll_items);
+  c->refs.birth_base = carve<BirthBase>(p, c->n_inst);
   c->refs.move_scan = carve<ChunkStatus>(p, move_chunks);
   c->refs.inst = c->d_inst;
   c->refs.istate = c->d_istate;
@@ -473,15 +476,13 @@ int commit(slpic_ctx* c) {
                 cudaMemcpyHostToDevice),
      "control");
   {
-    // first step's electron collision chunks from the majorant probability:
-    // about P0 kTile candidates per full tile
-    std::vector<unsigned int> t(c->n_inst, (unsigned int)kCollMaxRoom);
+    // the first step's density of candidates from the majorant probability:
+    // about P0 kTile per full tile
+    std::vector<unsigned int> t(c->n_inst);
     for (int i = 0; i < c->n_inst; ++i) {
       const double P0 = c->fp64 ? c->h_inst[i].c64.P0 : (double)c->h_inst[i].c32.P0;
-      const double per_tile = P0 * kTile;
-      while (t[i] > (unsigned int)kCollWarps &&
-             t[i] / kCollWarps * per_tile > kCollTargetPerWarp)
-        t[i] >>= 1;
+      const double room = kCollTarget / std::max(P0 * kTile, 1e-9);
+      t[i] = (unsigned int)std::min(std::max(room, 1.0), (double)kCollMaxRoom);
     }
     CK(cudaMemcpy(c->refs.coll_room, t.data(), t.size() * 4, cudaMemcpyHostToDevice),
        "control");
@@ -518,7 +519,7 @@ int commit(slpic_ctx* c) {
       return cuda_fail(c, (cudaError_t)e2, "finish kernel configuration");
     c->refs.finish_net_nodes = net_nodes;
   }
-  if (int e2 = collide_config())
+  if (int e2 = collide_config(c->fp64, max_nodes, &c->collide_resident, &c->refs.coll_nodes))
     return cuda_fail(c, (cudaError_t)e2, "collision kernel configuration");
   int sms = 0;
   CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device), "attributes");
@@ -527,7 +528,7 @@ int commit(slpic_ctx* c) {
   c->blocks_per_sm = bps;
   c->push_grid = sms * bps;
   c->move_grid = sms * 2;
-  c->collide_grid = sms * c->collide_per_sm;
+  c->collide_grid = sms * std::min(c->collide_per_sm, c->collide_resident);
   for (int i = 0; i < c->n_inst; ++i) {
     if (int rc = upload_inst(c, i)) return rc;
     if (int rc = reset_field(c, i)) return rc;
@@ -696,7 +697,7 @@ int apply_shape(slpic_ctx* c, int warps, int coll_per_sm) {
   c->blocks_per_sm = bps;
   c->push_grid = c->sms * bps;
   c->collide_per_sm = coll_per_sm;
-  c->collide_grid = c->sms * coll_per_sm;
+  c->collide_grid = c->sms * std::min(coll_per_sm, c->collide_resident);
   if (int rc = replan(c)) return rc;
   return sync(c);
 }

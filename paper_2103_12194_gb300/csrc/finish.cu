@@ -1,6 +1,6 @@
 // End of a step.  k_finish (one CTA per instance) updates the marker counts
 // from the step's exact counters (the particle kernel compacted every tile,
-// k_collide appended every birth), decides whether a store is repacked,
+// k_collide counted every birth), decides whether a store is repacked,
 // publishes the step's deposit, solves the 1D Poisson equation for the next
 // step's field (its exact integer sums) and commits the step's tallies; the
 // last CTA plans the next step.  k_move evaluates the field from those sums
@@ -44,25 +44,22 @@ __device__ __forceinline__ void plan_totals(const DeviceRefs& r, int n_seg, unsi
   r.ctrl->n_tiles = start;
   r.ctrl->w_total = wstart;
   r.ctrl->n_seg = n_seg;
-  r.ctrl->n_coll_chunks = coll;
-  r.ctrl->coll_counter = 0;
+  r.ctrl->n_coll_items = coll;
   r.ctrl->n_move_chunks = move;
   r.ctrl->move_counter = 0;
   r.ctrl->epoch = (r.ctrl->epoch + 1u) & 0x3FFFFFFFu;
   r.ctrl->finish_done = 0;
 }
 
-// Tiles per electron collision chunk of an instance of n_tiles electron tiles:
-// `room` of them hold kCollTargetPerWarp candidates per warp.  Fewer where the
-// instance would not give its share of kCollSpread chunks, but not below an
-// eighth of room (a round of 32 candidates per warp) in float.
-__device__ __forceinline__ unsigned int chunk_tiles(unsigned long long room, uint32_t n_tiles,
-                                                    int n_inst, int fp64) {
+// Tiles per electron collision item of an instance of n_tiles electron tiles:
+// `room` of them hold kCollTarget candidates.  Fewer where the instance would
+// not give its share of kCollSpread items, but in float not below an eighth of
+// room (a round of 32 candidates).
+__device__ __forceinline__ unsigned int item_tiles(unsigned long long room, uint32_t n_tiles,
+                                                   int n_inst, int fp64) {
   const unsigned long long share = (unsigned long long)n_tiles * n_inst / kCollSpread;
   const unsigned long long most = min(room, max(share, fp64 ? 1ull : room / 8u));
-  unsigned int T = kCollMaxChunkTiles;
-  while (T > 1u && T > most) T >>= 1;
-  return T;
+  return (unsigned int)min(max(most, 1ull), (unsigned long long)kCollMaxTiles);
 }
 
 // The plan below by one warp (n_seg <= 32 kPlanPerLane), with shuffle scans
@@ -91,12 +88,10 @@ __device__ void plan_next_warp(const DeviceRefs& r) {
     const int i = lane * (kPlanPerLane / 2) + j;
     nc[j] = 0;
     if (i < r.n_inst) {
-      const long long T = chunk_tiles(r.coll_room[i], r.sstate[2 * i].n_tiles, r.n_inst,
-                                      r.fp64);
+      const long long T = item_tiles(r.coll_room[i], r.sstate[2 * i].n_tiles, r.n_inst, r.fp64);
       r.coll_tiles[i] = (unsigned int)T;
       nc[j] = ((long long)r.sstate[2 * i].n_tiles + T - 1) / T +
-              ((long long)r.sstate[2 * i + 1].n_tiles + kCollMaxChunkTiles - 1) /
-                  kCollMaxChunkTiles;
+              ((long long)r.sstate[2 * i + 1].n_tiles + kCollIonTiles - 1) / kCollIonTiles;
     }
     s_nc += nc[j];
   }
@@ -127,7 +122,7 @@ __device__ void plan_next_warp(const DeviceRefs& r) {
 }
 
 // Plan the next step from the tiles in use (all threads of one CTA):
-// particle-kernel tiles and their weights per segment, repacking chunks per segment and collision chunks per instance,
+// particle-kernel tiles and their weights per segment, repacking chunks per segment and collision items per instance,
 // as exclusive block scans in rounds of kFinThreads entries.
 __device__ void plan_next(const DeviceRefs& r, long long* s_buf) {
   __shared__ long long s_carry[4];
@@ -168,11 +163,10 @@ __device__ void plan_next(const DeviceRefs& r, long long* s_buf) {
     const int i = base + t;
     long long nc = 0;
     if (i < r.n_inst) {
-      const long long T = chunk_tiles(r.coll_room[i], r.sstate[2 * i].n_tiles, r.n_inst,
-                                      r.fp64);
+      const long long T = item_tiles(r.coll_room[i], r.sstate[2 * i].n_tiles, r.n_inst, r.fp64);
       r.coll_tiles[i] = (unsigned int)T;
       nc = ((long long)r.sstate[2 * i].n_tiles + T - 1) / T +
-           ((long long)r.sstate[2 * i + 1].n_tiles + kCollMaxChunkTiles - 1) / kCollMaxChunkTiles;
+           ((long long)r.sstate[2 * i + 1].n_tiles + kCollIonTiles - 1) / kCollIonTiles;
     }
     const long long i_nc = block_incl_scan<long long>(nc, s_buf);
     if (i < r.n_inst) r.coll_start[i] = (unsigned int)(s_carry[3] + i_nc - nc);
@@ -185,28 +179,98 @@ __device__ void plan_next(const DeviceRefs& r, long long* s_buf) {
                 (unsigned int)s_carry[2], (unsigned int)s_carry[3]);
 }
 
-}  // namespace
-
-// mode 0: finish a step (one CTA per instance; the last one plans the next
-// step); mode 1: plan only (one CTA).  Dynamic shared memory: net_nodes
-// int64 nodes for the net deposit (0: read it from global memory).
-__global__ void __launch_bounds__(kFinThreads) k_finish(DeviceRefs r, int mode, int net_nodes) {
-  extern __shared__ long long s_dyn[];
-  __shared__ long long s_i64[32];
-  __shared__ __int128 s_i128[32];
-  __shared__ unsigned long long s_acc[ACC_COUNT];
-  __shared__ int s_flag;
-  step_kernel_entry();
-  Control* ctrl = r.ctrl;
+// Append the step's births to the stores, by CTA b of nb: the births of its
+// share of the items, in item order (ionization electrons in (tile, slot)
+// order of their parents, emitted electrons after them), one thread each.
+// Every CTA sums the counts of the items before its own, so none waits.
+template <typename R>
+__device__ __noinline__ void place_births(const DeviceRefs& r, int b, int nb, uint32_t* s_pre,
+                                          long long* s_i64) {
+  const unsigned int n_items = r.ctrl->n_coll_items;
+  const unsigned int per = (n_items + nb - 1) / nb;
+  unsigned int i0 = (unsigned int)b * per;
+  const unsigned int i1 = min(i0 + per, n_items);
   const int t = threadIdx.x;
-  if (mode == 1) {
-    for (int sg = t; sg < 2 * r.n_inst; sg += kFinThreads) r.xfer[sg].compact = 0;
-    __syncthreads();
-    plan_next(r, s_i64);
-    return;
+  int inst = 0;
+  {
+    int lo = 0, hi = r.n_inst - 1;  // last instance with coll_start <= i0
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (r.coll_start[mid] <= i0) lo = mid;
+      else hi = mid - 1;
+    }
+    inst = lo;
   }
-  if (*((volatile int*)&ctrl->error)) return;
-  const int inst = blockIdx.x;
+  for (; i0 < i1; ++inst) {
+    const unsigned int first = r.coll_start[inst], end = min(i1, r.coll_start[inst + 1]);
+    if (end <= i0) continue;  // an instance without items
+    const InstDev& P = r.inst[inst];
+    const BirthBase B = r.birth_base[inst];
+    const uint32_t wt = r.coll_tiles[inst];
+    const uint32_t step = B.step;
+    // births of the instance before item i0
+    long long before;
+    {
+      long long n = 0;
+      for (unsigned int k = first + t; k < i0; k += kFinThreads) n += r.item_births[k];
+      const long long inc = block_incl_scan<long long>(n, s_i64);
+      if (t == kFinThreads - 1) s_i64[0] = inc;
+      __syncthreads();
+      before = s_i64[0];
+      __syncthreads();
+    }
+    const SpeciesDev& E = P.sp[kElectron];
+    const Markers<R> me{E.buf[B.cur[0]]}, mi{P.sp[kIon].buf[B.cur[1]]};
+    const uint32_t* list = reinterpret_cast<const uint32_t*>(E.buf[B.cur[0] ^ 1u]);
+    const unsigned int e_items = B.e_items;
+    for (; i0 < end; i0 += kFinThreads) {
+      // prefixes of up to kFinThreads items
+      const unsigned int m = min(end - i0, (unsigned int)kFinThreads);
+      const uint32_t c = (unsigned int)t < m ? r.item_births[i0 + t] : 0u;
+      const long long inc = block_incl_scan<long long>((long long)c, s_i64);
+      s_pre[t] = (uint32_t)(inc - c);
+      if (t == kFinThreads - 1) s_i64[0] = inc;
+      __syncthreads();
+      const uint32_t total = (uint32_t)s_i64[0];
+      for (uint32_t n = t; n < total; n += kFinThreads) {
+        // the item of birth n: the last one whose prefix is <= n
+        unsigned int lo = 0, hi = m - 1;
+        while (lo < hi) {
+          const unsigned int mid = (lo + hi + 1) >> 1;
+          if (s_pre[mid] <= n) lo = mid;
+          else hi = mid - 1;
+        }
+        const uint32_t q = n - s_pre[lo], rank = (uint32_t)before + n;
+        const unsigned int local = i0 + lo - first;
+        const Slot<R> pe = me[B.tail[0] + rank];
+        if (local < e_items) {
+          const CandRec<R> cr = get_cand<R>(E.crec, list[local * wt * kTile + q]);
+          born_pair<R>(P, pe, mi[B.tail[1] + rank], cr.cell, cr.off, cr.wj, cr.id, step, cr.vx,
+                       B.next_id[0] + rank, B.next_id[1] + rank);
+        } else {
+          // emitted at the cathode by an ion of the item's tiles
+          uint32_t k = (local - e_items) * kCollIonTiles, e = q, f;
+          while (e >= (f = P.sp[kIon].births[k])) {
+            e -= f;
+            ++k;
+          }
+          write_marker(pe, 0, (R)0, (R)0, (R)0, (R)0,
+                       reinterpret_cast<const R*>(E.stage_w)[(size_t)k * kTile + e],
+                       kGenBit | ((B.next_id[0] + rank) & kSerialMask));
+        }
+      }
+      before += total;
+      __syncthreads();
+    }
+    i0 = end;
+  }
+}
+
+// The end of a step of instance inst, by one CTA.
+__device__ __forceinline__ void finish_instance(const DeviceRefs& r, int inst, int net_nodes,
+                                                long long* s_dyn, long long* s_i64,
+                                                __int128* s_i128, unsigned long long* s_acc) {
+  const int t = threadIdx.x;
   const InstDev& P = r.inst[inst];
   InstState& is = r.istate[inst];
   unsigned long long* a = P.acc;
@@ -275,14 +339,12 @@ __global__ void __launch_bounds__(kFinThreads) k_finish(DeviceRefs r, int mode, 
     x.tail = tail;
     x.end = end;
     if (sp == kElectron) {
-      // tiles of an electron collision chunk of the next step: about
-      // kCollTargetPerWarp candidates per warp at this step's candidates per tile
+      // tiles that hold about kCollTarget candidates at this step's density
       const unsigned long long cand = s_acc[ACC_CAND];
       const unsigned long long room =
-          cand ? (unsigned long long)kCollTargetPerWarp * kCollWarps * s0.n_tiles / cand
+          cand ? (unsigned long long)kCollTarget * s0.n_tiles / cand
                : (unsigned long long)kCollMaxRoom;
-      r.coll_room[inst] = (unsigned int)min(max(room, (unsigned long long)kCollWarps),
-                                            (unsigned long long)kCollMaxRoom);
+      r.coll_room[inst] = (unsigned int)min(max(room, 1ull), (unsigned long long)kCollMaxRoom);
     }
     SpeciesState s1;
     s1.cur = x.dst;
@@ -332,6 +394,37 @@ __global__ void __launch_bounds__(kFinThreads) k_finish(DeviceRefs r, int mode, 
     is.step += 1u;
     is.n_steps_done += 1;
   }
+}
+
+}  // namespace
+
+// mode 0: finish a step (CTAs 0 .. n_inst - 1, one per instance; the others
+// place the births; the last one of all plans the next step); mode 1: plan only (one CTA).  Dynamic shared memory: net_nodes
+// int64 nodes for the net deposit (0: read it from global memory).
+__global__ void __launch_bounds__(kFinThreads) k_finish(DeviceRefs r, int mode, int net_nodes) {
+  extern __shared__ long long s_dyn[];
+  __shared__ long long s_i64[32];
+  __shared__ __int128 s_i128[32];
+  __shared__ unsigned long long s_acc[ACC_COUNT];
+  __shared__ uint32_t s_pre[kFinThreads];
+  __shared__ int s_flag;
+  step_kernel_entry();
+  Control* ctrl = r.ctrl;
+  const int t = threadIdx.x;
+  if (mode == 1) {
+    for (int sg = t; sg < 2 * r.n_inst; sg += kFinThreads) r.xfer[sg].compact = 0;
+    __syncthreads();
+    plan_next(r, s_i64);
+    return;
+  }
+  if (*((volatile int*)&ctrl->error)) return;
+  if ((int)blockIdx.x >= r.n_inst) {
+    const int b = blockIdx.x - r.n_inst, nb = gridDim.x - r.n_inst;
+    if (r.fp64) place_births<double>(r, b, nb, s_pre, s_i64);
+    else place_births<float>(r, b, nb, s_pre, s_i64);
+  } else {
+    finish_instance(r, blockIdx.x, net_nodes, s_dyn, s_i64, s_i128, s_acc);
+  }
 
   // ---- the last CTA plans the next step --------------------------------------
   __threadfence();
@@ -346,7 +439,6 @@ __global__ void __launch_bounds__(kFinThreads) k_finish(DeviceRefs r, int mode, 
     plan_next(r, s_i64);
   }
 }
-
 // The deposit of instance inst's live markers into its last-step grids
 // (zeroed by the caller): each marker adds fixed_charge(beta(|v|) w_j) at its
 // position, as the step deposits it.  A step's deposit is a function of the
@@ -442,7 +534,7 @@ int finish_config(int max_nodes, int* net_nodes) {
 }
 
 void launch_finish(const DeviceRefs& r, int mode, cudaStream_t s) {
-  const int grid = mode == 1 ? 1 : r.n_inst;
+  const int grid = mode == 1 ? 1 : r.n_inst + kBirthCtas;
   const int nodes = mode == 1 ? 0 : r.finish_net_nodes;
   launch_step_kernel(k_finish, grid, kFinThreads, (size_t)nodes * 8, s, r, mode, nodes);
 }

@@ -202,9 +202,8 @@ struct Transfer {
 };
 
 // A null-collision candidate as the particle kernel leaves it: the electron's
-// state after its push and its slot in the tile after compaction (the top bit
-// marks an ionization once it has collided; vx then holds the energy given to
-// the secondary).  One record fills a 32-byte sector in float, so the
+// state after its push and its slot in the tile after compaction (once it has
+// ionized, vx holds the energy given to the secondary).  One record fills a 32-byte sector in float, so the
 // collision kernel reads a candidate with one sector instead of one per field.
 template <typename R>
 struct CandRec;
@@ -222,7 +221,6 @@ struct alignas(16) CandRec<double> {
   uint32_t slot, pad;
 };
 static_assert(sizeof(CandRec<float>) == 32, "one sector per float record");
-constexpr uint32_t kIonizedMark = 0x80000000u;
 
 // Configuration of one species of one instance (constant during a run).
 struct SpeciesDev {
@@ -232,7 +230,9 @@ struct SpeciesDev {
                       // (at rest at x = 0), slot = ion tile * kTile + rank
   uint32_t* births;   // ions: [cap_tiles] electrons emitted by each tile in the step
   void* crec;         // electrons: [cap_tiles * kTile] CandRec<R>, the tile's
-                      // null-collision candidates in slot order
+                      // null-collision candidates in slot order (during a step
+                      // the buffer that is not in use holds, from an item's
+                      // first slot on, the numbers of its ionizations' records)
   uint32_t* n_cand;   // electrons: [cap_tiles] candidates per tile
   uint32_t cap_tiles;
   uint32_t pad;
@@ -295,8 +295,7 @@ struct Control {
   int error_inst;
   unsigned int spin_waits;   // polls that found data not yet there
   unsigned int spin_max;     // longest single wait, in polls
-  unsigned int coll_counter; // next collision chunk to hand out
-  unsigned int n_coll_chunks;
+  unsigned int n_coll_items;
   unsigned int move_counter; // next repacking chunk to hand out
   unsigned int n_move_chunks;
   unsigned int small_bar;    // single-CTA path: arrivals at its grid barriers
@@ -315,28 +314,33 @@ struct ChunkStatus {
   unsigned int pad;
 };
 
-// Collision chunks: kCollWarps warps of T / kCollWarps consecutive tiles
-// each (below kCollWarps tiles, one tile for each of the first T warps).
-// Electron chunks have T = coll_tiles[inst] tiles, a power of two up to
-// kCollMaxChunkTiles: small enough that a warp meets about kCollTargetPerWarp
-// candidates at the instance's last step's density (many collisions per step:
-// small chunks, more warps), and, down to a round of 32 candidates per warp
-// (in double, where the FP64 unit of each SM counts, down to one tile), that
-// the instance gives its share of kCollSpread chunks (two per SM: with few
-// tiles, fewer per CTA, so that every SM has some; 1e5 electrons of a 256-cell
-// gap: k_collide 36 -> 19 us, in double 487 -> 55 us).
-// Ion chunks (the electrons emitted at the cathode, rare) have
-// kCollMaxChunkTiles.  Repacking chunks: kMoveChunkTiles tiles.
-constexpr int kCollWarps = 8;
-constexpr int kCollMaxChunkTiles = kCollWarps * 32;
-// (a bound of the tiles that hold that many candidates per warp)
-constexpr int kCollMaxRoom = 64 * kCollMaxChunkTiles;
-constexpr int kCollSpread = 304;
-constexpr int kCollTargetPerWarp = 256;
+// Collision items, one warp each: consecutive tiles of one instance, electron
+// items of coll_tiles[inst] tiles and then ion items of kCollIonTiles (the
+// electrons emitted at the cathode, rare).  coll_tiles[inst] is at
+// most kCollMaxTiles: small enough that an item holds about kCollTarget
+// candidates at the instance's last step's density, and, down to a round of 32
+// candidates (in double, where the FP64 unit of each SM counts, down to one
+// tile), that the instance gives its share of kCollSpread items (16 per SM).
+constexpr int kCollMaxTiles = 32;
+constexpr int kCollIonTiles = 256;
+constexpr int kCollTarget = 128;
+constexpr int kCollSpread = 2432;
+// (a bound of the tiles that hold that many candidates)
+constexpr int kCollMaxRoom = 64 * kCollMaxTiles;
+// CTAs of k_finish beside the instances' own that place the births.
+constexpr int kBirthCtas = 64;
+// Repacking chunks: tiles each.
 constexpr int kMoveChunkTiles = 128;
 // Single-CTA path (small.cu): at most this many tiles per store and instance
 // when a step starts.
 constexpr int kSmallMaxTiles = 32;
+
+// Where a step's births go in the stores of one instance: buffers, first free
+// slots, next serial numbers, step and electron items, before the step's end
+// moves the state on.
+struct BirthBase {
+  uint32_t cur[2], tail[2], next_id[2], step, e_items;
+};
 
 struct DeviceRefs {
   InstDev* inst;          // [n_inst]
@@ -346,15 +350,17 @@ struct DeviceRefs {
   Control* ctrl;
   unsigned int* seg_start;   // [n_seg + 1] first tile of each segment
   unsigned int* seg_wstart;  // [n_seg + 1] summed tile weights before each segment
-  unsigned int* coll_start;  // [n_inst + 1] first collision chunk of each instance
-  unsigned int* coll_tiles;  // [n_inst] tiles per electron collision chunk
+  unsigned int* coll_start;  // [n_inst + 1] first collision item of each instance
+  unsigned int* coll_tiles;  // [n_inst] tiles per electron collision item
   unsigned int* coll_room;   // [n_inst] the most its density of candidates allows
   unsigned int* move_start;  // [n_seg + 1] first repacking chunk of each segment
-  ChunkStatus* coll_scan;    // [max collision chunks]
+  uint32_t* item_births;     // [max collision items] births of each item in the step
+  BirthBase* birth_base;     // [n_inst]
   ChunkStatus* move_scan;    // [max repacking chunks]
   int n_inst;
   int smem_nodes;         // deposit grid nodes in shared memory (0: global atomics)
   int push_warps;         // warps per particle-kernel CTA
+  int coll_nodes;         // collision kernel: deposit grid nodes in shared memory (0: none)
   int fp64;               // marker path in double precision (else float)
   int finish_net_nodes;   // k_finish keeps the net deposit of up to this many nodes in shared memory
 };
@@ -379,7 +385,9 @@ void launch_phi(const DeviceRefs& r, int inst, cudaStream_t s);
 void launch_deposit(const DeviceRefs& r, int inst, int n_tiles, cudaStream_t s);
 // Scatter the null-collision candidates queued by the particle kernel.
 void launch_collide(const DeviceRefs& r, int grid, cudaStream_t s);
-int collide_config();
+// Its resident CTAs per SM and the nodes of its shared charge grid (0: deposits
+// go to global memory) in a context of grids of up to max_nodes nodes.
+int collide_config(int fp64, int max_nodes, int* resident, int* nodes);
 // Seeding: n markers written contiguously from slot `base` of the current
 // buffer; mode 0/1/2 as SLPIC_SEED_*; for mode 3 (thermal) e0 carries the
 // thermal speed sqrt(k T / m).

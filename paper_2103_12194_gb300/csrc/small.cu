@@ -435,7 +435,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
             atomicCAS(&ctrl->error, 0, kErrCapacity);
           } else {
             const Slot<R> m = me[o];
-            born_pair<R, false>(P, me[pe], mi[pi], m.cell(), m.off(), m.wj(), m.id(), step,
+            born_pair<R>(P, me[pe], mi[pi], m.cell(), m.off(), m.wj(), m.id(), step,
                                 es[u], se.next_id + rank, si.next_id + rank);
           }
         }

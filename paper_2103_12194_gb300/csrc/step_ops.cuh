@@ -265,38 +265,62 @@ __device__ __forceinline__ void copy_marker(const Slot<R>& d, const Slot<R>& m) 
   write_marker(d, m.cell(), m.off(), m.vx(), m.vy(), m.vz(), m.wj(), m.id());
 }
 
-// Write the electron and Ar+ born by an ionization to their slots with their serial numbers, and (kDeposit) deposit
-// both.  The secondary gets energy es along an isotropic direction (block 1
-// of the primary's draws); the ion a gas-temperature Maxwellian (Box-Muller
-// on block 2).
-template <typename R, bool kDeposit = true>
-__device__ void born_pair(const InstDev& P, const Slot<R>& me, const Slot<R>& mi, int cell, R off, R wj, uint32_t id, uint32_t step, R es,
-                          uint32_t serial_e, uint32_t serial_i) {
+// Velocities of the electron and the Ar+ born by an ionization: the secondary
+// gets energy es along an isotropic direction (block 1 of the primary's
+// draws), the ion a gas-temperature Maxwellian (Box-Muller on block 2).
+template <typename R>
+__device__ __forceinline__ Velocity<R> born_electron(const InstDev& P, uint32_t id, uint32_t step,
+                                                     R es) {
   const StepConsts<R>& K = consts<R>(P);
-  const uint32_t gen = id & kGenBit;
   const uint4 r1 = philox4x32_10(make_uint4(id, step, P.ctr_inst * 2u, 1u), P.key0, P.key1);
-  R bx, by, bz;
+  Velocity<R> v;
   isotropic(r_sqrt(es * K.K_V[kElectron]), uniform01r<R>(r1.y), uniform01r<R>(r1.z), K.two_pi,
-            bx, by, bz);
-  write_marker(me, cell, off, bx, by, bz, wj, gen | (serial_e & kSerialMask));
-  if (kDeposit)
-    deposit(P.rho_acc[kElectron], cell, off,
-            fixed_charge(beta_of(r_sqrt(bx * bx + by * by + bz * bz), K.vlim[kElectron]) * wj,
-                         K.wscale));
+            v.vx, v.vy, v.vz);
+  return v;
+}
+template <typename R>
+__device__ __forceinline__ Velocity<R> born_ion(const InstDev& P, uint32_t id, uint32_t step) {
+  const StepConsts<R>& K = consts<R>(P);
   const uint4 r2 = philox4x32_10(make_uint4(id, step, P.ctr_inst * 2u, 2u), P.key0, P.key1);
   R g[4];
   uniform4<R>(r2, g);
   const R rr1 = r_sqrt((R)-2 * r_log(g[0]));
   const R rr2 = r_sqrt((R)-2 * r_log(g[2]));
   const R a1 = K.two_pi * g[1], a2 = K.two_pi * g[3];
-  const R ix = K.sigT_ion * (rr1 * r_cos(a1));
-  const R iy = K.sigT_ion * (rr1 * r_sin(a1));
-  const R iz = K.sigT_ion * (rr2 * r_cos(a2));
-  write_marker(mi, cell, off, ix, iy, iz, wj, gen | (serial_i & kSerialMask));
-  if (kDeposit)
-    deposit(P.rho_acc[kIon], cell, off,
-            fixed_charge(beta_of(r_sqrt(ix * ix + iy * iy + iz * iz), K.vlim[kIon]) * wj,
-                         K.wscale));
+  return {K.sigT_ion * (rr1 * r_cos(a1)), K.sigT_ion * (rr1 * r_sin(a1)),
+          K.sigT_ion * (rr2 * r_cos(a2))};
+}
+
+// Write the electron and Ar+ born by an ionization to their slots with their
+// serial numbers.
+template <typename R>
+__device__ void born_pair(const InstDev& P, const Slot<R>& me, const Slot<R>& mi, int cell, R off,
+                          R wj, uint32_t id, uint32_t step, R es, uint32_t serial_e,
+                          uint32_t serial_i) {
+  const uint32_t gen = id & kGenBit;
+  const Velocity<R> e = born_electron<R>(P, id, step, es);
+  write_marker(me, cell, off, e.vx, e.vy, e.vz, wj, gen | (serial_e & kSerialMask));
+  const Velocity<R> i = born_ion<R>(P, id, step);
+  write_marker(mi, cell, off, i.vx, i.vy, i.vz, wj, gen | (serial_i & kSerialMask));
+}
+
+// Deposit both at their parent's position (a species without a speed limit has
+// beta = 1, whatever its velocity).  Rare; kept out of line.
+template <typename R>
+__device__ __noinline__ void deposit_pair(const InstDev& P, int cell, R off, R wj, uint32_t id,
+                                          uint32_t step, R es) {
+  const StepConsts<R>& K = consts<R>(P);
+  R b[2] = {(R)1, (R)1};
+  if (K.vlim[kElectron] < (R)INFINITY) {
+    const Velocity<R> v = born_electron<R>(P, id, step, es);
+    b[0] = beta_of(r_sqrt(v.vx * v.vx + v.vy * v.vy + v.vz * v.vz), K.vlim[kElectron]);
+  }
+  if (K.vlim[kIon] < (R)INFINITY) {
+    const Velocity<R> v = born_ion<R>(P, id, step);
+    b[1] = beta_of(r_sqrt(v.vx * v.vx + v.vy * v.vy + v.vz * v.vz), K.vlim[kIon]);
+  }
+  for (int s = 0; s < 2; ++s)
+    deposit(P.rho_acc[s], cell, off, fixed_charge(b[s] * wj, K.wscale));
 }
 
 // Slot after the last live marker of a store (the particle kernel has

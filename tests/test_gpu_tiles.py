@@ -124,3 +124,61 @@ def test_markers_read_from_device_memory(slpic, start):  # noqa: F811
     for k in got:
         assert np.array_equal(got[k], view[k]), k
     sim.close()
+
+
+def deposit_of(m, spec, vlim):
+    """The fixed-point deposit of FP32 markers, as every step forms it."""
+    f = np.float32
+    v2 = m["vx"] * m["vx"] + m["vy"] * m["vy"] + m["vz"] * m["vz"]
+    with np.errstate(divide="ignore"):
+        beta = np.minimum(f(1), f(vlim) / np.sqrt(v2)) if math.isfinite(vlim) else f(1)
+    q = np.rint((beta * m["wj"]) * f(2.0 ** spec["charge_shift"])).astype(np.int64)
+    right = (q * (m["off"] * f(2.0 ** 24)).astype(np.int64)) >> 24
+    out = np.zeros(spec["n_cells"] + 1, np.int64)
+    np.add.at(out, m["cell"], q - right)
+    np.add.at(out, m["cell"] + 1, right)
+    return out
+
+
+@pytest.mark.parametrize("field_mode", [0, 1])
+@pytest.mark.parametrize("populations", [
+    [(40_000, 20_000)],                                        # one gap
+    [(0, 3000), (1, 0), (130, 1), (0, 0), (9000, 4000)],        # uneven ones: several per CTA
+    [(k * 37 + 1, 300) for k in range(60)],                    # more gaps than CTAs take singly
+])
+def test_collision_items_and_births(slpic, oracle_mod, populations, field_mode):  # noqa: F811
+    """One dense step of every process with emission: the births of each gap
+    in the order of their parents, with their serial numbers, whatever items
+    and CTAs they fall to, and the deposit of exactly the markers there are."""
+    sim = slpic.Simulation(len(populations))
+    specs, states = [], []
+    for k, (ne, ni) in enumerate(populations):
+        spec = inputs.gap_spec(n_cells=(64, 300, 1500)[k % 3], V=300.0, pd_torr_cm=20.0,
+                               gamma_se=0.5, field_mode=field_mode, charge_shift=24, seed=7 + k,
+                               instance=k)
+        specs.append(spec)
+        states.append(mixed_state(spec, ne, ni, seed=300 + k))
+        sim.configure(k, spec, capacity=(2 * ne + ni + 256, ne + ni + 256))
+    for k, (e, i) in enumerate(states):
+        sim.load(k, 0, e)
+        sim.load(k, 1, i)
+    sim.step(1)
+    born = emitted = 0
+    for k, spec in enumerate(specs):
+        ref = oracle_mod.Oracle(spec, precision=32)
+        ref.load(0, states[k][0])
+        ref.load(1, states[k][1])
+        ref.step(1)
+        h, g = ref.history()[-1], sim.history(k)[-1]
+        for key in ("n_live", "n_coll", "n_abs", "n_see", "n_candidates"):
+            assert np.array_equal(h[key], g[key]), (k, key)
+        born += int(h["n_coll"][2])
+        emitted += int(h["n_see"])
+        for s, vlim in ((0, spec["vlim_e"]), (1, spec["vlim_i"])):
+            m, r = sim.particles(k, s), ref.particles(s)
+            assert np.array_equal(m["id"], r["id"].astype(np.uint32)), (k, s)
+            assert np.array_equal(m["cell"], r["cell"]) and np.array_equal(
+                m["off"], r["off"].astype(np.float32)), (k, s)
+            assert np.array_equal(sim.charge(k, s), deposit_of(m, spec, vlim)), (k, s)
+    assert born > 0 and emitted > 0
+    sim.close()
