@@ -108,6 +108,27 @@ struct slpic_ctx {
   // the markers when read, or before they change)
   std::vector<char> dep_dirty;
   int blocks_per_sm = 0;
+  // Small transfers go through pinned memory, in the stream's order: `pin` is
+  // handed out from its start until the stream has been waited for (drain),
+  // which also delivers the reads.
+  struct Read {
+    void* to;
+    const char* from;
+    size_t bytes;
+  };
+  char* pin = nullptr;
+  size_t pin_size = 0, pin_used = 0;
+  std::vector<Read> reads;
+  // The instances' and stores' state as the host knows it; `known` while no
+  // step has run since it was read (a step captured into a caller's graph runs
+  // unseen: such a context always reads it again).
+  std::vector<char> state_raw;
+  std::vector<SpeciesState> hs;
+  std::vector<InstState> his;
+  std::vector<int64_t> tail;  // first free slot of each store (-1: not known)
+  Control hctrl{};
+  bool known = false, uncached = false;
+  bool plan_due = false;  // the stores have changed since the next step was planned
   // graph of kGraphSteps steps
   cudaGraphExec_t graph = nullptr;
   // profiling
@@ -149,9 +170,70 @@ int set_device(slpic_ctx* c) {
   return SLPIC_OK;
 }
 
-int device_error(slpic_ctx* c) {
-  Control h;
-  CK(cudaMemcpy(&h, c->d_ctrl, sizeof h, cudaMemcpyDeviceToHost), "read status");
+// Wait for the stream and deliver the reads queued on it.
+int drain(slpic_ctx* c) {
+  CK(cudaStreamSynchronize(c->stream), "stream synchronize");
+  for (const auto& r : c->reads) std::memcpy(r.to, r.from, r.bytes);
+  c->reads.clear();
+  c->pin_used = 0;
+  return SLPIC_OK;
+}
+
+// Room for `bytes` bytes of pinned memory until the next drain.
+int pin_room(slpic_ctx* c, size_t bytes, char** p) {
+  const size_t need = (bytes + 15) & ~size_t(15);
+  if (c->pin_used + need > c->pin_size) {
+    if (int rc = drain(c)) return rc;
+    if (need > c->pin_size) {
+      if (c->pin) CK(cudaFreeHost(c->pin), "pinned memory");
+      c->pin = nullptr;
+      c->pin_size = 0;
+      const size_t size = std::max(need, size_t(1) << 20);
+      CK(cudaHostAlloc((void**)&c->pin, size, cudaHostAllocDefault), "pinned memory");
+      c->pin_size = size;
+    }
+  }
+  *p = c->pin + c->pin_used;
+  c->pin_used += need;
+  return SLPIC_OK;
+}
+
+// Queue a copy to the device (the source may change at once) or from it (it
+// arrives with the next drain).
+int put(slpic_ctx* c, void* dev, const void* host, size_t bytes) {
+  char* p;
+  if (int rc = pin_room(c, bytes, &p)) return rc;
+  std::memcpy(p, host, bytes);
+  CK(cudaMemcpyAsync(dev, p, bytes, cudaMemcpyHostToDevice, c->stream), "copy to the device");
+  return SLPIC_OK;
+}
+int get(slpic_ctx* c, void* host, const void* dev, size_t bytes) {
+  char* p;
+  if (int rc = pin_room(c, bytes, &p)) return rc;
+  CK(cudaMemcpyAsync(p, dev, bytes, cudaMemcpyDeviceToHost, c->stream), "copy from the device");
+  c->reads.push_back({host, p, bytes});
+  return SLPIC_OK;
+}
+
+// The state of all instances and stores and the control block lie in one
+// stretch of device memory: queue a read of it, and take it over after the
+// drain.  Returns the device error it shows.
+size_t state_bytes(const slpic_ctx* c) {
+  return (size_t)((const char*)(c->d_ctrl + 1) - (const char*)c->d_istate);
+}
+int ask_state(slpic_ctx* c) {
+  c->state_raw.resize(state_bytes(c));
+  return get(c, c->state_raw.data(), c->d_istate, c->state_raw.size());
+}
+int take_state(slpic_ctx* c) {
+  const char* raw = c->state_raw.data();
+  auto at = [&](const void* dev) { return raw + ((const char*)dev - (const char*)c->d_istate); };
+  std::memcpy(c->his.data(), raw, sizeof(InstState) * c->his.size());
+  std::memcpy(c->hs.data(), at(c->d_sstate), sizeof(SpeciesState) * c->hs.size());
+  std::memcpy(&c->hctrl, at(c->d_ctrl), sizeof(Control));
+  std::fill(c->tail.begin(), c->tail.end(), -1);
+  const Control& h = c->hctrl;
+  c->known = h.error == kErrNone && !c->uncached;
   switch (h.error) {
     case kErrNone: return SLPIC_OK;
     case kErrCapacity:
@@ -166,11 +248,29 @@ int device_error(slpic_ctx* c) {
   }
 }
 
+// The state known on the host (hs, his), and the error latched on the device.
 int sync(slpic_ctx* c) {
   if (int rc = set_device(c)) return rc;
-  CK(cudaStreamSynchronize(c->stream), "stream synchronize");
-  if (!c->committed) return SLPIC_OK;
-  return device_error(c);
+  if (!c->committed) {
+    CK(cudaStreamSynchronize(c->stream), "stream synchronize");
+    return SLPIC_OK;
+  }
+  if (c->known) return SLPIC_OK;
+  if (int rc = ask_state(c)) return rc;
+  if (int rc = drain(c)) return rc;
+  return take_state(c);
+}
+
+// Read `bytes` bytes after everything queued, with the state if it is not
+// known: *err is the latched error, the return value a failure of the read.
+int read_with_state(slpic_ctx* c, void* host, const void* dev, size_t bytes, int* err) {
+  const bool ask = !c->known;
+  if (ask)
+    if (int rc = ask_state(c)) return rc;
+  if (int rc = get(c, host, dev, bytes)) return rc;
+  if (int rc = drain(c)) return rc;
+  *err = ask ? take_state(c) : SLPIC_OK;
+  return SLPIC_OK;
 }
 
 // The step's constants in the marker path's type R, each rounded once from
@@ -285,48 +385,44 @@ int dmalloc(slpic_ctx* c, void** p, size_t bytes, const char* what) {
 // Reset the vacuum field of instance i on the device: phi linear, E = -V/d.
 int reset_field(slpic_ctx* c, int i) {
   const InstDev& P = c->h_inst[i];
-  const int nn = P.n_cells + 1;
-  std::vector<double> phi(nn), E(nn, -P.V / P.d);
-  std::vector<float> E32(nn, (float)(-P.V / P.d));
-  for (int k = 0; k < nn; ++k) phi[k] = P.V * k / P.n_cells;
-  CK(cudaMemcpyAsync(P.phi, phi.data(), nn * 8, cudaMemcpyHostToDevice, c->stream), "field");
-  CK(cudaMemcpyAsync(P.E64, E.data(), nn * 8, cudaMemcpyHostToDevice, c->stream), "field");
-  CK(cudaMemcpyAsync(P.E32, E32.data(), nn * 4, cudaMemcpyHostToDevice, c->stream), "field");
-  CK(cudaStreamSynchronize(c->stream), "field");
+  launch_vacuum(P, -P.V / P.d, (float)(-P.V / P.d), c->stream);
+  CK(cudaGetLastError(), "field");
   if ((int)c->stepped.size() == c->n_inst) c->stepped[i] = 0;
   return SLPIC_OK;
 }
 
-int upload_inst(slpic_ctx* c, int i) {
-  CK(cudaMemcpyAsync(c->d_inst + i, &c->h_inst[i], sizeof(InstDev), cudaMemcpyHostToDevice,
-                     c->stream),
-     "upload instance");
-  CK(cudaStreamSynchronize(c->stream), "upload instance");
-  return SLPIC_OK;
+int upload_inst(slpic_ctx* c, int i) { return put(c, c->d_inst + i, &c->h_inst[i], sizeof(InstDev)); }
+
+int write_inst_state(slpic_ctx* c, int i) {
+  return put(c, c->d_istate + i, &c->his[i], sizeof(InstState));
 }
 
+// Set the state of a store to what the host now holds; `tail` is its first
+// free slot.  The next step is planned anew before it runs.
+int write_state(slpic_ctx* c, int inst, int sp, const SpeciesState& st, int64_t tail) {
+  c->hs[2 * inst + sp] = st;
+  c->tail[2 * inst + sp] = tail;
+  c->plan_due = true;
+  return put(c, c->d_sstate + inst * 2 + sp, &st, sizeof st);
+}
+
+// (the state is known)
 int zero_counters(slpic_ctx* c, int i) {
   const InstDev& P = c->h_inst[i];
-  CK(cudaMemsetAsync(P.acc, 0, ACC_COUNT * 8, c->stream), "reset");
-  CK(cudaMemsetAsync(P.total, 0, sizeof(TallyRec), c->stream), "reset");
-  CK(cudaMemsetAsync(P.ring, 0, sizeof(TallyRec) * P.ring_len, c->stream), "reset");
+  // both deposits, the Poisson sums (formed anew by every step), the step's
+  // accumulators, the history and the totals lie in one stretch
+  CK(cudaMemsetAsync(P.rho_acc[0], 0, (size_t)((char*)(P.total + 1) - (char*)P.rho_acc[0]),
+                     c->stream),
+     "reset");
   // step counter, step count and seeded weight restart; the live weight
   // describes the markers, which stay
-  InstState is;
-  CK(cudaMemcpyAsync(&is, c->d_istate + i, sizeof is, cudaMemcpyDeviceToHost, c->stream), "reset");
-  CK(cudaStreamSynchronize(c->stream), "reset");
+  InstState& is = c->his[i];
   is.step = 0;
   is.n_steps_done = 0;
   is.w_seed = 0;
   is.ion_steps = 0;
-  CK(cudaMemcpyAsync(c->d_istate + i, &is, sizeof is, cudaMemcpyHostToDevice, c->stream), "reset");
-  for (int s = 0; s < 2; ++s) {
-    CK(cudaMemsetAsync(P.rho_acc[s], 0, (P.n_cells + 1) * 8, c->stream), "reset");
-    CK(cudaMemsetAsync(P.rho_last[s], 0, (P.n_cells + 1) * 8, c->stream), "reset");
-  }
   if ((int)c->dep_dirty.size() == c->n_inst) c->dep_dirty[i] = 0;
-  CK(cudaStreamSynchronize(c->stream), "reset");
-  return SLPIC_OK;
+  return write_inst_state(c, i);
 }
 
 int commit(slpic_ctx* c) {
@@ -529,45 +625,32 @@ int commit(slpic_ctx* c) {
   c->push_grid = sms * bps;
   c->move_grid = sms * 2;
   c->collide_grid = sms * std::min(c->collide_per_sm, c->collide_resident);
+  c->hs.assign(nseg, SpeciesState{});
+  c->his.assign(c->n_inst, InstState{});
+  c->tail.assign(nseg, 0);
   for (int i = 0; i < c->n_inst; ++i) {
     if (int rc = upload_inst(c, i)) return rc;
     if (int rc = reset_field(c, i)) return rc;
     if (int rc = zero_counters(c, i)) return rc;
   }
   CK(cudaStreamCreateWithFlags(&c->capture_stream, cudaStreamNonBlocking), "stream");
+  if (int rc = drain(c)) return rc;
   c->committed = true;
-  launch_finish(c->refs, 1, c->stream);
-  CK(cudaGetLastError(), "plan");
-  CK(cudaStreamSynchronize(c->stream), "plan");
-  return SLPIC_OK;
-}
-
-int read_state(slpic_ctx* c, int inst, int sp, SpeciesState* out) {
-  CK(cudaMemcpy(out, c->d_sstate + inst * 2 + sp, sizeof *out, cudaMemcpyDeviceToHost),
-     "read state");
-  return SLPIC_OK;
-}
-
-int write_state(slpic_ctx* c, int inst, int sp, const SpeciesState& st) {
-  CK(cudaMemcpy(c->d_sstate + inst * 2 + sp, &st, sizeof st, cudaMemcpyHostToDevice),
-     "write state");
+  c->known = true;
+  c->plan_due = true;
   return SLPIC_OK;
 }
 
 // With an imposed field the step deposits nothing: form the last step's
 // deposit of instance i from its markers (a function of them) if it has
 // stepped since the deposit was last formed.  Called before the deposit is
-// read and before the markers change.
+// read and before the markers change, with the state known.
 int materialize_deposit(slpic_ctx* c, int i) {
   if (c->h_inst[i].field_mode == 1 || !c->dep_dirty[i]) return SLPIC_OK;
-  SpeciesState st[2];
-  CK(cudaMemcpyAsync(st, c->d_sstate + 2 * i, sizeof st, cudaMemcpyDeviceToHost, c->stream),
-     "deposit");
-  CK(cudaStreamSynchronize(c->stream), "deposit");
   const InstDev& P = c->h_inst[i];
   for (int s = 0; s < 2; ++s)
     CK(cudaMemsetAsync(P.rho_last[s], 0, (P.n_cells + 1) * 8, c->stream), "deposit");
-  launch_deposit(c->refs, i, (int)(st[0].n_tiles + st[1].n_tiles), c->stream);
+  launch_deposit(c->refs, i, (int)(c->hs[2 * i].n_tiles + c->hs[2 * i + 1].n_tiles), c->stream);
   CK(cudaGetLastError(), "deposit");
   c->dep_dirty[i] = 0;
   return SLPIC_OK;
@@ -579,9 +662,23 @@ void mark_stepped(slpic_ctx* c) {
     if (c->h_inst[i].field_mode != 1) c->dep_dirty[i] = 1;
 }
 
-int replan(slpic_ctx* c) {
+bool capturing(const slpic_ctx* c) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  return c->stream && cudaStreamIsCapturing(c->stream, &st) == cudaSuccess &&
+         st != cudaStreamCaptureStatusNone;
+}
+
+// Before steps are launched: the plan of the next one, if the stores have
+// changed since it was made (captured into a caller's graph, it is made by the
+// graph, and again by the next call), and the state no longer known.
+int begin_steps(slpic_ctx* c) {
+  const bool cap = capturing(c);
+  if (cap) c->uncached = true;
+  c->known = false;
+  if (!c->plan_due) return SLPIC_OK;
   launch_finish(c->refs, 1, c->stream);
   CK(cudaGetLastError(), "plan");
+  c->plan_due = cap;
   return SLPIC_OK;
 }
 
@@ -603,10 +700,7 @@ int run_small(slpic_ctx* c, int64_t n, int64_t* done,
   *done = 0;
   if (n <= 0 || c->small_limit <= 0 || c->profiling) return SLPIC_OK;
   if (int rc = sync(c)) return rc;
-  std::vector<SpeciesState> st(2 * (size_t)c->n_inst);
-  CK(cudaMemcpy(st.data(), c->d_sstate, sizeof(SpeciesState) * st.size(),
-                cudaMemcpyDeviceToHost),
-     "small path");
+  const std::vector<SpeciesState>& st = c->hs;
   const int64_t L = (int64_t)c->small_limit * kTile;
   int max_pn = 0;
   for (int i = 0; i < c->n_inst; ++i) {
@@ -635,14 +729,16 @@ int run_small(slpic_ctx* c, int64_t n, int64_t* done,
       return cuda_fail(c, (cudaError_t)e, "small path launch");
     launch_finish(c->refs, 1, c->stream);  // the batched path's next step
     CK(cudaGetLastError(), "small path");
-    CK(cudaStreamSynchronize(c->stream), "small path");
-    long long d = 0;
-    CK(cudaMemcpy(&d, &c->d_ctrl->small_done, sizeof d, cudaMemcpyDeviceToHost),
-       "small path");
+    c->known = false;
+    c->plan_due = false;
+    if (int rc = ask_state(c)) return rc;
+    if (int rc = drain(c)) return rc;
+    const int err = take_state(c);
+    const long long d = c->hctrl.small_done;
     *done += d;
     c->last_launches += 2;
     if (d > 0) mark_stepped(c);
-    if (int rc = device_error(c)) return rc;
+    if (err) return err;
     if (d < k) break;  // a store outgrew the path
   }
   return SLPIC_OK;
@@ -698,8 +794,8 @@ int apply_shape(slpic_ctx* c, int warps, int coll_per_sm) {
   c->push_grid = c->sms * bps;
   c->collide_per_sm = coll_per_sm;
   c->collide_grid = c->sms * std::min(coll_per_sm, c->collide_resident);
-  if (int rc = replan(c)) return rc;
-  return sync(c);
+  c->plan_due = true;
+  return SLPIC_OK;
 }
 
 // The seven marker arrays of a caller (cell, off, vx, vy, vz, w_j, id), in
@@ -789,6 +885,7 @@ int slpic_destroy(slpic_ctx* c) {
   drop_graph(c);
   for (auto& e : c->ev) cudaEventDestroy(e);
   for (void* p : c->allocs) cudaFree(p);
+  if (c->pin) cudaFreeHost(c->pin);
   if (c->capture_stream) cudaStreamDestroy(c->capture_stream);
   delete c;
   return SLPIC_OK;
@@ -796,6 +893,11 @@ int slpic_destroy(slpic_ctx* c) {
 
 int slpic_set_stream(slpic_ctx* c, void* stream) {
   if (!c) return SLPIC_ERR_INVALID_ARG;
+  if (c->committed && c->stream != (cudaStream_t)stream) {
+    // what is queued on the old stream comes before all that follows
+    if (int rc = set_device(c)) return rc;
+    if (int rc = drain(c)) return rc;
+  }
   c->stream = (cudaStream_t)stream;
   return SLPIC_OK;
 }
@@ -994,27 +1096,20 @@ int slpic_suggest_dt(double d, int n_cells, double V, double m_ion, int mode, do
 
 namespace {
 
-// Set the fills of tiles [first, ceil(end / kTile)) of a store whose slots
-// [first * kTile, end) are all live.
-int write_fills(slpic_ctx* c, const SpeciesDev& S, uint32_t cur, uint32_t first, uint32_t end) {
-  const uint32_t last = (end + kTile - 1) / kTile;
-  if (last <= first) return SLPIC_OK;
-  std::vector<uint32_t> f(last - first);
-  for (uint32_t k = first; k < last; ++k)
-    f[k - first] = std::min<uint32_t>(end - k * (uint32_t)kTile, (uint32_t)kTile);
-  CK(cudaMemcpy(S.fill[cur] + first, f.data(), f.size() * 4, cudaMemcpyHostToDevice), "fills");
-  return SLPIC_OK;
-}
-
-// First free slot after the last live marker of a store.
-int tail_slot(slpic_ctx* c, const SpeciesDev& S, const SpeciesState& st, uint32_t* out) {
-  if (st.n_tiles == 0) {
-    *out = 0;
-    return SLPIC_OK;
+// First free slot after the last live marker of a store (the state is known).
+int tail_slot(slpic_ctx* c, int inst, int sp, int64_t* out) {
+  const SpeciesState& st = c->hs[2 * inst + sp];
+  int64_t& tail = c->tail[2 * inst + sp];
+  if (tail < 0) {
+    uint32_t f = 0;
+    if (st.n_tiles) {
+      const SpeciesDev& S = c->h_inst[inst].sp[sp];
+      if (int rc = get(c, &f, S.fill[st.cur] + st.n_tiles - 1, 4)) return rc;
+      if (int rc = drain(c)) return rc;
+    }
+    tail = st.n_tiles ? (int64_t)(st.n_tiles - 1) * kTile + f : 0;
   }
-  uint32_t f = 0;
-  CK(cudaMemcpy(&f, S.fill[st.cur] + st.n_tiles - 1, 4, cudaMemcpyDeviceToHost), "fills");
-  *out = (st.n_tiles - 1) * (uint32_t)kTile + f;
+  *out = tail;
   return SLPIC_OK;
 }
 
@@ -1029,12 +1124,12 @@ extern "C" int slpic_seed(slpic_ctx* c, int inst, int species, int64_t n, int mo
   if (int rc = prepare(c)) return rc;
   if (int rc = sync(c)) return rc;
   if (int rc = materialize_deposit(c, inst)) return rc;
-  SpeciesState st;
-  if (int rc = read_state(c, inst, species, &st)) return rc;
+  SpeciesState st = c->hs[2 * inst + species];
   const InstDev& P = c->h_inst[inst];
   const SpeciesDev& S = P.sp[species];
-  uint32_t app = 0;
-  if (int rc = tail_slot(c, S, st, &app)) return rc;
+  int64_t tail = 0;
+  if (int rc = tail_slot(c, inst, species, &tail)) return rc;
+  const uint32_t app = (uint32_t)tail;
   if ((uint64_t)app + (uint64_t)n > (uint64_t)S.cap_tiles * kTile)
     return fail(c, SLPIC_ERR_CAPACITY, "seeding %lld markers exceeds the capacity", (long long)n);
   if ((uint64_t)st.next_id + (uint64_t)n > kSerialMask)
@@ -1052,23 +1147,17 @@ extern "C" int slpic_seed(slpic_ctx* c, int inst, int species, int64_t n, int mo
   const double lr = mode == 2 ? std::log(e_hi / e_lo) : 0.0;
   launch_seed(c->refs, inst, species, app, st.next_id, (uint32_t)n, mode, ekin, e_lo, lr, wj,
               c->stream);
+  launch_fills(S.fill[st.cur], app / kTile, app + (uint32_t)n, c->stream);
   CK(cudaGetLastError(), "seed");
-  CK(cudaStreamSynchronize(c->stream), "seed");
-  if (int rc = write_fills(c, S, st.cur, app / kTile, app + (uint32_t)n)) return rc;
   st.n_live += (uint32_t)n;
   st.next_id += (uint32_t)n;
   st.n_tiles = std::max(st.n_tiles, (app + (uint32_t)n + kTile - 1) / (uint32_t)kTile);
-  if (int rc = write_state(c, inst, species, st)) return rc;
-  {
-    InstState is;
-    CK(cudaMemcpy(&is, c->d_istate + inst, sizeof is, cudaMemcpyDeviceToHost), "seed");
-    const unsigned long long q = (unsigned long long)n * (unsigned long long)std::llrint(wq);
-    if (species == kElectron) is.w_seed += q;
-    is.w_live[species] += q;
-    CK(cudaMemcpy(c->d_istate + inst, &is, sizeof is, cudaMemcpyHostToDevice), "seed");
-  }
-  if (int rc = replan(c)) return rc;
-  return sync(c);
+  if (int rc = write_state(c, inst, species, st, app + n)) return rc;
+  InstState& is = c->his[inst];
+  const unsigned long long q = (unsigned long long)n * (unsigned long long)std::llrint(wq);
+  if (species == kElectron) is.w_seed += q;
+  is.w_live[species] += q;
+  return write_inst_state(c, inst);
 }
 
 namespace {
@@ -1116,8 +1205,7 @@ int load_common(slpic_ctx* c, int inst, int species, const Arrays& src, int64_t 
   const SpeciesDev& S = P.sp[species];
   if ((uint64_t)n > (uint64_t)S.cap_tiles * kTile)
     return fail(c, SLPIC_ERR_CAPACITY, "%lld markers exceed the capacity", (long long)n);
-  SpeciesState st;
-  if (int rc = read_state(c, inst, species, &st)) return rc;
+  SpeciesState st = c->hs[2 * inst + species];
   // arrays on the device are read where they are; host arrays (and whatever a
   // kernel must not read) are copied to the buffer that is not in use first,
   // by a copy that returns an error for what is no such memory
@@ -1133,40 +1221,35 @@ int load_common(slpic_ctx* c, int inst, int species, const Arrays& src, int64_t 
   }
   // validated on the device: a marker outside the gap would make the step
   // read and write outside the field and charge arrays
-  unsigned int* scratch = c->d_scratch;
-  unsigned int bad_init[4] = {0xFFFFFFFFu, 0u, 0u, 0u};
-  CK(cudaMemcpyAsync(scratch, bad_init, 16, cudaMemcpyHostToDevice, c->stream), "load");
-  launch_place(c->fp64, f, S.buf[st.cur], (uint32_t)n, P.n_cells, P.charge_shift, scratch,
-               reinterpret_cast<unsigned long long*>(scratch + 2), c->stream);
-  CK(cudaGetLastError(), "load");
-  unsigned int res[4];
-  CK(cudaMemcpyAsync(res, scratch, 16, cudaMemcpyDeviceToHost, c->stream), "load");
-  CK(cudaStreamSynchronize(c->stream), "load");
   st.n_live = 0;
   st.n_tiles = 0;
-  if (res[0] != 0xFFFFFFFFu) {
-    write_state(c, inst, species, st);
-    replan(c);
-    return fail(c, SLPIC_ERR_INVALID_ARG,
-                "marker %u outside the gap, not finite, or with a weight of 2^39 charge "
-                "units or more; the species was emptied", res[0]);
+  unsigned long long wsum = 0;
+  if (n > 0) {
+    unsigned int* scratch = c->d_scratch;
+    unsigned int res[4] = {0xFFFFFFFFu, 0u, 0u, 0u};
+    if (int rc = put(c, scratch, res, 16)) return rc;
+    launch_place(c->fp64, f, S.buf[st.cur], (uint32_t)n, P.n_cells, P.charge_shift, scratch,
+                 reinterpret_cast<unsigned long long*>(scratch + 2), c->stream);
+    launch_fills(S.fill[st.cur], 0, (uint32_t)n, c->stream);
+    CK(cudaGetLastError(), "load");
+    if (int rc = get(c, res, scratch, 16)) return rc;
+    if (int rc = drain(c)) return rc;
+    if (res[0] != 0xFFFFFFFFu) {
+      write_state(c, inst, species, st, 0);
+      return fail(c, SLPIC_ERR_INVALID_ARG,
+                  "marker %u outside the gap, not finite, or with a weight of 2^39 charge "
+                  "units or more; the species was emptied", res[0]);
+    }
+    std::memcpy(&wsum, res + 2, 8);
   }
-  if (int rc = write_fills(c, S, st.cur, 0, (uint32_t)n)) return rc;
   st.n_live = (uint32_t)n;
   st.n_tiles = (uint32_t)(((uint64_t)n + kTile - 1) / kTile);
   st.next_id = next_id;
-  if (int rc = write_state(c, inst, species, st)) return rc;
-  {
-    InstState is;
-    CK(cudaMemcpy(&is, c->d_istate + inst, sizeof is, cudaMemcpyDeviceToHost), "load");
-    unsigned long long wsum;
-    std::memcpy(&wsum, res + 2, 8);
-    if (species == kElectron) is.w_seed = wsum;
-    is.w_live[species] = wsum;
-    CK(cudaMemcpy(c->d_istate + inst, &is, sizeof is, cudaMemcpyHostToDevice), "load");
-  }
-  if (int rc = replan(c)) return rc;
-  return sync(c);
+  if (int rc = write_state(c, inst, species, st, n)) return rc;
+  InstState& is = c->his[inst];
+  if (species == kElectron) is.w_seed = wsum;
+  is.w_live[species] = wsum;
+  return write_inst_state(c, inst);
 }
 
 }  // namespace
@@ -1207,8 +1290,11 @@ int slpic_reset_counters(slpic_ctx* c, int inst) {
 int slpic_step(slpic_ctx* c, int64_t n) {
   if (!c || n < 0) return fail(c, SLPIC_ERR_INVALID_ARG, "bad step count");
   if (int rc = prepare(c)) return rc;
-  if (n > 0) mark_stepped(c);
   c->last_launches = 0;
+  if (n > 0) {
+    mark_stepped(c);
+    if (int rc = begin_steps(c)) return rc;
+  }
   if (c->profiling) {
     for (int64_t k = 0; k < n; ++k) {
       if (c->ev_used + 2 > c->ev.size()) {
@@ -1267,6 +1353,10 @@ int slpic_set_small_limit(slpic_ctx* c, int max_tiles) {
 
 int slpic_synchronize(slpic_ctx* c) {
   if (!c) return SLPIC_ERR_INVALID_ARG;
+  if (c->known) {
+    if (int rc = set_device(c)) return rc;
+    return drain(c);
+  }
   return sync(c);
 }
 
@@ -1274,30 +1364,32 @@ int slpic_clear_error(slpic_ctx* c) {
   if (!c) return SLPIC_ERR_INVALID_ARG;
   if (!c->committed) return SLPIC_OK;
   if (int rc = set_device(c)) return rc;
-  CK(cudaStreamSynchronize(c->stream), "clear");
-  CK(cudaMemset(&c->d_ctrl->error, 0, sizeof(int)), "clear");
+  CK(cudaMemsetAsync(&c->d_ctrl->error, 0, sizeof(int), c->stream), "clear");
   for (int i = 0; i < c->n_inst; ++i) {
     const InstDev& P = c->h_inst[i];
-    CK(cudaMemset(P.acc, 0, ACC_COUNT * 8), "clear");
-    for (int s = 0; s < 2; ++s) CK(cudaMemset(P.rho_acc[s], 0, (P.n_cells + 1) * 8), "clear");
+    CK(cudaMemsetAsync(P.acc, 0, ACC_COUNT * 8, c->stream), "clear");
+    for (int s = 0; s < 2; ++s)
+      CK(cudaMemsetAsync(P.rho_acc[s], 0, (P.n_cells + 1) * 8, c->stream), "clear");
   }
-  if (int rc = replan(c)) return rc;
-  CK(cudaStreamSynchronize(c->stream), "clear");
-  return SLPIC_OK;
+  c->known = false;
+  c->plan_due = true;
+  return drain(c);
 }
 
 int slpic_count(slpic_ctx* c, int inst, int species, int64_t* n) {
   if (!valid_inst(c, inst) || (species != 0 && species != 1) || !n)
     return fail(c, SLPIC_ERR_INVALID_ARG, "bad arguments");
   if (int rc = prepare(c)) return rc;
-  int rc = sync(c);
-  SpeciesState st;
-  if (int r2 = read_state(c, inst, species, &st)) return r2;
-  *n = st.n_live;
+  const int rc = sync(c);
+  *n = c->hs[2 * inst + species].n_live;
   return rc;
 }
 
 namespace {
+
+// Marker arrays up to this size are read through pinned memory, all seven with
+// one wait; larger ones straight into the caller's arrays.
+constexpr size_t kPinnedRead = size_t(1) << 20;
 
 int read_common(slpic_ctx* c, int inst, int species, const Arrays& host, int64_t capacity,
                 int64_t* n_out) {
@@ -1305,9 +1397,8 @@ int read_common(slpic_ctx* c, int inst, int species, const Arrays& host, int64_t
     return fail(c, SLPIC_ERR_INVALID_ARG, "bad arguments");
   if (int rc = precision_check(c, host.fp64)) return rc;
   if (int rc = prepare(c)) return rc;
-  int rc = sync(c);
-  SpeciesState st;
-  if (int r2 = read_state(c, inst, species, &st)) return r2;
+  const int rc = sync(c);
+  const SpeciesState st = c->hs[2 * inst + species];
   *n_out = st.n_live;
   if ((int64_t)st.n_live > capacity)
     return fail(c, SLPIC_ERR_INVALID_ARG, "host buffers hold %lld markers, %u live",
@@ -1315,31 +1406,30 @@ int read_common(slpic_ctx* c, int inst, int species, const Arrays& host, int64_t
   if (st.n_live > 0) {
     if (int r3 = arrays_check(c, host)) return r3;
     const SpeciesDev& S = c->h_inst[inst].sp[species];
-    // live markers before each tile, in the fills of the buffer that is not
-    // in use; the markers go through that buffer, in order
-    std::vector<uint32_t> pre(st.n_tiles);
-    CK(cudaMemcpy(pre.data(), S.fill[st.cur], st.n_tiles * 4, cudaMemcpyDeviceToHost), "read");
-    uint32_t before = 0;
-    for (uint32_t& p : pre) {
-      const uint32_t m = p;
-      p = before;
-      before += m;
-    }
-    CK(cudaMemcpyAsync(S.fill[st.cur ^ 1u], pre.data(), st.n_tiles * 4, cudaMemcpyHostToDevice,
-                       c->stream),
-       "read");
-    // (after a failed step the fills hold what that step left)
-    const size_t n = std::min<size_t>(before, st.n_live);
+    // the markers go through the buffer that is not in use, in store order;
+    // its fills hold the number of markers before each tile
+    uint32_t* const before = S.fill[st.cur ^ 1u];
     void* f[7];
-    carve_arrays(reinterpret_cast<char*>(S.buf[st.cur ^ 1u]), before, c->fp64 ? 8 : 4, f);
-    launch_gather(c->fp64, S.buf[st.cur], S.fill[st.cur], S.fill[st.cur ^ 1u], st.n_tiles, f,
-                  c->stream);
+    carve_arrays(reinterpret_cast<char*>(S.buf[st.cur ^ 1u]), st.n_live, c->fp64 ? 8 : 4, f);
+    launch_prefix(S.fill[st.cur], st.n_tiles, before, c->d_scratch, c->stream);
+    launch_gather(c->fp64, S.buf[st.cur], S.fill[st.cur], before, st.n_tiles, f, c->stream);
     CK(cudaGetLastError(), "read");
-    for (int k = 0; k < 7; ++k)
-      CK(cudaMemcpyAsync(host.f[k], f[k], field_bytes(c, k, n), cudaMemcpyDeviceToHost,
-                         c->stream),
-         "read");
-    CK(cudaStreamSynchronize(c->stream), "read");
+    // after a failed step the fills hold what that step left
+    uint32_t sum = st.n_live;
+    if (rc) {
+      if (int r3 = get(c, &sum, c->d_scratch, 4)) return r3;
+      if (int r3 = drain(c)) return r3;
+      sum = std::min(sum, st.n_live);
+    }
+    for (int k = 0; k < 7; ++k) {
+      const size_t b = field_bytes(c, k, sum);
+      if (b <= kPinnedRead) {
+        if (int r3 = get(c, host.f[k], f[k], b)) return r3;
+      } else {
+        CK(cudaMemcpyAsync(host.f[k], f[k], b, cudaMemcpyDeviceToHost, c->stream), "read");
+      }
+    }
+    if (int r3 = drain(c)) return r3;
   }
   return rc;
 }
@@ -1360,12 +1450,16 @@ int slpic_read_charge(slpic_ctx* c, int inst, int species, int64_t* host, int64_
   if (!valid_inst(c, inst) || (species != 0 && species != 1) || !host)
     return fail(c, SLPIC_ERR_INVALID_ARG, "bad arguments");
   if (int rc = prepare(c)) return rc;
-  int rc = sync(c);
   const InstDev& P = c->h_inst[inst];
+  int rc = SLPIC_OK;
+  const bool form = P.field_mode != 1 && c->dep_dirty[inst];
+  if (form || n != P.n_cells + 1) rc = sync(c);
   if (n != P.n_cells + 1) return fail(c, SLPIC_ERR_INVALID_ARG, "need n_cells + 1 values");
-  if (int r2 = materialize_deposit(c, inst)) return r2;
-  CK(cudaMemcpy(host, P.rho_last[species], n * 8, cudaMemcpyDeviceToHost), "read charge");
-  return rc;
+  if (form)
+    if (int r2 = materialize_deposit(c, inst)) return r2;
+  int err = SLPIC_OK;
+  if (int r2 = read_with_state(c, host, P.rho_last[species], n * 8, &err)) return r2;
+  return rc ? rc : err;
 }
 
 int slpic_read_density(slpic_ctx* c, int inst, int species, double* host, int64_t n) {
@@ -1388,28 +1482,30 @@ int slpic_read_density(slpic_ctx* c, int inst, int species, double* host, int64_
 int slpic_read_field(slpic_ctx* c, int inst, double* phi, double* E, int64_t n) {
   if (!valid_inst(c, inst) || !phi || !E) return fail(c, SLPIC_ERR_INVALID_ARG, "bad arguments");
   if (int rc = prepare(c)) return rc;
-  int rc = sync(c);
   const InstDev& P = c->h_inst[inst];
-  if (n != P.n_cells + 1) return fail(c, SLPIC_ERR_INVALID_ARG, "need n_cells + 1 values");
+  if (n != P.n_cells + 1) {
+    sync(c);
+    return fail(c, SLPIC_ERR_INVALID_ARG, "need n_cells + 1 values");
+  }
   // the step keeps only the node field; phi is formed from the last deposit
   // (in the frozen-field mode it stays the vacuum solution)
   if (P.field_mode == 1 && c->stepped[inst]) {
     launch_phi(c->refs, inst, c->stream);
     CK(cudaGetLastError(), "read field");
-    CK(cudaStreamSynchronize(c->stream), "read field");
   }
-  CK(cudaMemcpy(phi, P.phi, n * 8, cudaMemcpyDeviceToHost), "read field");
-  CK(cudaMemcpy(E, P.E64, n * 8, cudaMemcpyDeviceToHost), "read field");
-  return rc;
+  int err = SLPIC_OK;
+  if (int rc = get(c, phi, P.phi, n * 8)) return rc;
+  if (int rc = read_with_state(c, E, P.E64, n * 8, &err)) return rc;
+  return err;
 }
 
 int slpic_read_tallies(slpic_ctx* c, int inst, slpic_tallies* out) {
   static_assert(sizeof(slpic_tallies) == sizeof(TallyRec), "tally layout");
   if (!valid_inst(c, inst) || !out) return fail(c, SLPIC_ERR_INVALID_ARG, "bad arguments");
   if (int rc = prepare(c)) return rc;
-  int rc = sync(c);
-  CK(cudaMemcpy(out, c->h_inst[inst].total, sizeof *out, cudaMemcpyDeviceToHost), "read tallies");
-  return rc;
+  int err = SLPIC_OK;
+  if (int rc = read_with_state(c, out, c->h_inst[inst].total, sizeof *out, &err)) return rc;
+  return err;
 }
 
 int slpic_read_history(slpic_ctx* c, int inst, slpic_tallies* out, int64_t capacity,
@@ -1418,18 +1514,18 @@ int slpic_read_history(slpic_ctx* c, int inst, slpic_tallies* out, int64_t capac
     return fail(c, SLPIC_ERR_INVALID_ARG, "bad arguments");
   if (int rc = prepare(c)) return rc;
   int rc = sync(c);
-  InstState is;
-  CK(cudaMemcpy(&is, c->d_istate + inst, sizeof is, cudaMemcpyDeviceToHost), "history");
+  const InstState& is = c->his[inst];
   const InstDev& P = c->h_inst[inst];
   const long long have = std::min<long long>(is.n_steps_done, P.ring_len);
   const long long m = std::min<long long>(have, capacity);
-  std::vector<TallyRec> ring(P.ring_len);
-  CK(cudaMemcpy(ring.data(), P.ring, sizeof(TallyRec) * P.ring_len, cudaMemcpyDeviceToHost),
-     "history");
-  for (long long k = 0; k < m; ++k) {
-    const long long s = is.n_steps_done - m + k;
-    std::memcpy(out + k, &ring[s % P.ring_len], sizeof(TallyRec));
+  // the last m records: at most two stretches of the ring
+  for (long long k = 0; k < m;) {
+    const long long at = (is.n_steps_done - m + k) % P.ring_len;
+    const long long run = std::min(m - k, P.ring_len - at);
+    if (int r2 = get(c, out + k, P.ring + at, sizeof(TallyRec) * run)) return r2;
+    k += run;
   }
+  if (int r2 = drain(c)) return r2;
   *n_out = m;
   return rc;
 }
@@ -1455,10 +1551,8 @@ int slpic_read_gain(slpic_ctx* c, int inst, double* G) {
   if (!valid_inst(c, inst) || !G) return fail(c, SLPIC_ERR_INVALID_ARG, "bad arguments");
   slpic_tallies t;
   int rc = slpic_read_tallies(c, inst, &t);
-  InstState is;
-  CK(cudaMemcpy(&is, c->d_istate + inst, sizeof is, cudaMemcpyDeviceToHost), "gain");
   const InstDev& P = c->h_inst[inst];
-  const double seed = (double)is.w_seed / P.c64.wscale;
+  const double seed = (double)c->his[inst].w_seed / P.c64.wscale;
   *G = seed > 0 ? t.w_gain_gen0 / seed : 0.0;
   return rc;
 }
@@ -1755,11 +1849,7 @@ extern "C" int slpic_paschen_bisect(slpic_ctx* c, const slpic_paschen_spec* ps, 
       }
       done += k;
       if ((rc = sync(c))) break;
-      if (cudaMemcpy(st.data(), c->d_sstate, sizeof(SpeciesState) * st.size(),
-                     cudaMemcpyDeviceToHost) != cudaSuccess) {
-        rc = fail(c, SLPIC_ERR_CUDA, "paschen: reading the live counts");
-        break;
-      }
+      st = c->hs;
       bool live = false;
       k = ps->chunk_steps;
       for (int i = 0; i < n && !rc; ++i) {
@@ -1797,12 +1887,7 @@ extern "C" int slpic_paschen_bisect(slpic_ctx* c, const slpic_paschen_spec* ps, 
       }
       slpic_tallies t;
       if ((rc = slpic_read_tallies(c, i, &t))) break;
-      InstState is;
-      if (cudaMemcpy(&is, c->d_istate + i, sizeof is, cudaMemcpyDeviceToHost) != cudaSuccess) {
-        rc = fail(c, SLPIC_ERR_CUDA, "paschen: reading the seeded weight");
-        break;
-      }
-      const double w_seed = (double)is.w_seed / c->h_inst[i].c64.wscale;
+      const double w_seed = (double)c->his[i].w_seed / c->h_inst[i].c64.wscale;
       G[i] = w_seed > 0 ? t.w_gain_gen0 / w_seed : 0.0;
     }
     if (rc) break;
@@ -1906,12 +1991,12 @@ extern "C" int slpic_save(slpic_ctx* c, void* buf, size_t capacity, size_t* size
       CK(cudaGetLastError(), "save");
     }
     for (int s = 0; s < 2; ++s)
-      if (int rc = read_state(c, i, s, &st[2 * i + s])) return rc;
+      st[2 * i + s] = c->hs[2 * i + s];
     size_t b = 0;
     snap_inst_bytes(c, i, &st[2 * i], &b);
     total += b;
   }
-  CK(cudaStreamSynchronize(c->stream), "save");
+  if (int rc = drain(c)) return rc;
   *size_out = total;
   if (!buf) return SLPIC_OK;
   if (capacity < total)
@@ -1932,7 +2017,7 @@ extern "C" int slpic_save(slpic_ctx* c, void* buf, size_t capacity, size_t* size
     r.n_cells = P.n_cells;
     r.ring_len = P.ring_len;
     r.stepped = c->stepped[i];
-    CK(cudaMemcpy(&r.is, c->d_istate + i, sizeof r.is, cudaMemcpyDeviceToHost), "save");
+    r.is = c->his[i];
     CK(cudaMemcpy(&r.total, P.total, sizeof r.total, cudaMemcpyDeviceToHost), "save");
     for (int s = 0; s < 2; ++s) {
       r.n_live[s] = st[2 * i + s].n_live;
@@ -2026,6 +2111,8 @@ extern "C" int slpic_load(slpic_ctx* c, const void* buf, size_t size) {
     }
     // the counters, tallies, field and deposit as saved (the loads above
     // set the seeded and live weights from the markers)
+    if (int rc = drain(c)) return rc;
+    c->his[i] = r.is;
     CK(cudaMemcpy(c->d_istate + i, &r.is, sizeof r.is, cudaMemcpyHostToDevice), "load");
     CK(cudaMemcpy(P.total, &r.total, sizeof r.total, cudaMemcpyHostToDevice), "load");
     CK(cudaMemcpy(P.ring, ring, sizeof(TallyRec) * P.ring_len, cudaMemcpyHostToDevice), "load");
@@ -2037,8 +2124,8 @@ extern "C" int slpic_load(slpic_ctx* c, const void* buf, size_t size) {
     c->stepped[i] = (char)r.stepped;
     c->dep_dirty[i] = 0;
   }
-  if (int rc = replan(c)) return rc;
-  return sync(c);
+  c->plan_due = true;
+  return SLPIC_OK;
 }
 
 extern "C" int slpic_set_spin_limit(slpic_ctx* c, uint32_t polls) {
@@ -2114,11 +2201,8 @@ extern "C" int slpic_ion_trend(slpic_ctx* c, int64_t steps_per_window, int n_win
   std::vector<char> stopped(n, 0);
   auto read_states = [&]() -> int {
     if (int rc = sync(c)) return rc;
-    if (cudaMemcpy(st.data(), c->d_sstate, sizeof(SpeciesState) * st.size(),
-                   cudaMemcpyDeviceToHost) != cudaSuccess ||
-        cudaMemcpy(is.data(), c->d_istate, sizeof(InstState) * is.size(),
-                   cudaMemcpyDeviceToHost) != cudaSuccess)
-      return fail(c, SLPIC_ERR_CUDA, "ion trend: reading the live counts");
+    st = c->hs;
+    is = c->his;
     return SLPIC_OK;
   };
   if (int rc = read_states()) return rc;

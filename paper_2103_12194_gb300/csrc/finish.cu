@@ -513,6 +513,52 @@ void launch_phi(const DeviceRefs& r, int inst, cudaStream_t s) {
   k_phi<<<1, kFinThreads, 0, s>>>(r, inst);
 }
 
+__global__ void __launch_bounds__(256) k_vacuum(double* phi, double* E64, float* E32, int N,
+                                                double V, double E, float Ef) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k > N) return;
+  phi[k] = V * k / N;
+  E64[k] = E;
+  E32[k] = Ef;
+}
+
+void launch_vacuum(const InstDev& P, double E, float E32, cudaStream_t s) {
+  k_vacuum<<<P.n_cells / 256 + 1, 256, 0, s>>>(P.phi, P.E64, P.E32, P.n_cells, P.V, E, E32);
+}
+
+__global__ void __launch_bounds__(256) k_fills(uint32_t* fill, uint32_t first, uint32_t last,
+                                               uint32_t end) {
+  const uint32_t k = first + blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < last) fill[k] = min(end - k * (uint32_t)kTile, (uint32_t)kTile);
+}
+
+void launch_fills(uint32_t* fill, uint32_t first, uint32_t end, cudaStream_t s) {
+  const uint32_t last = end / kTile + (end % kTile != 0);
+  if (last > first) k_fills<<<(last - first + 255) / 256, 256, 0, s>>>(fill, first, last, end);
+}
+
+// Exclusive prefix of the fills by one CTA (when markers are read).
+__global__ void __launch_bounds__(kFinThreads) k_prefix(const uint32_t* fill, uint32_t n,
+                                                        uint32_t* prefix, uint32_t* total) {
+  __shared__ long long s_i64[32];
+  const uint32_t chunk = (n + kFinThreads - 1) / kFinThreads;
+  const uint32_t k0 = min(threadIdx.x * chunk, n), k1 = min(k0 + chunk, n);
+  long long loc = 0;
+  for (uint32_t k = k0; k < k1; ++k) loc += fill[k];
+  const long long inc = block_incl_scan<long long>(loc, s_i64);
+  long long run = inc - loc;
+  for (uint32_t k = k0; k < k1; ++k) {
+    prefix[k] = (uint32_t)run;
+    run += fill[k];
+  }
+  if (threadIdx.x == kFinThreads - 1) *total = (uint32_t)inc;
+}
+
+void launch_prefix(const uint32_t* fill, uint32_t n_tiles, uint32_t* prefix, uint32_t* total,
+                   cudaStream_t s) {
+  k_prefix<<<1, kFinThreads, 0, s>>>(fill, n_tiles, prefix, total);
+}
+
 // Dynamic shared memory of k_finish: the net deposit of the largest grid,
 // when it fits (DeviceRefs::finish_net_nodes, from finish_config).
 int finish_config(int max_nodes, int* net_nodes) {

@@ -379,6 +379,14 @@ int finish_config(int max_nodes, int* net_nodes);
 void launch_move(const DeviceRefs& r, int grid, cudaStream_t s);
 // Node potential of instance inst from its last deposit (Poisson mode).
 void launch_phi(const DeviceRefs& r, int inst, cudaStream_t s);
+// The vacuum field of an instance: phi = V k / N, E on every node.
+void launch_vacuum(const InstDev& P, double E, float E32, cudaStream_t s);
+// Fills of tiles [first, ceil(end / kTile)) of a store whose slots from
+// first * kTile to end are all live.
+void launch_fills(uint32_t* fill, uint32_t first, uint32_t end, cudaStream_t s);
+// Markers before each of n_tiles tiles, and (*total) in all of them.
+void launch_prefix(const uint32_t* fill, uint32_t n_tiles, uint32_t* prefix, uint32_t* total,
+                   cudaStream_t s);
 // Deposit of instance inst's live markers (n_tiles tiles of both species)
 // added to its last-step grids; used with an imposed field, where the step
 // itself deposits nothing.
