@@ -449,7 +449,7 @@ int commit(slpic_ctx* c) {
     if (c->fp64) bytes += (tab_n * sizeof(TabNode64) + 255) & ~size_t(255);
     bytes += ((nn * 4 + 255) & ~size_t(255));
     bytes += 2 * ((nn * 8 + 255) & ~size_t(255));
-    bytes += 5 * ((nn * 8 + 255) & ~size_t(255)) + 256;
+    bytes += 4 * ((nn * 8 + 255) & ~size_t(255)) + (nn / kFieldNodes + 1) * 24 + 512;
     bytes += 256 + ((sizeof(TallyRec) * kRingLen + 255) & ~size_t(255)) + 256;
     void* blk;
     if (int rc = dmalloc(c, &blk, bytes, "instance arrays")) return rc;
@@ -466,8 +466,8 @@ int commit(slpic_ctx* c) {
     P.rho_acc[1] = carve<unsigned long long>(p, nn);
     P.rho_last[0] = carve<long long>(p, nn);
     P.rho_last[1] = carve<long long>(p, nn);
-    P.pois_I = carve<long long>(p, nn);
-    P.pois_D1 = carve<double>(p, 1);
+    P.pois_W = carve<__int128>(p, nn / kFieldNodes + 1);
+    P.pois_S = carve<long long>(p, nn / kFieldNodes + 1);
     P.acc = carve<unsigned long long>(p, ACC_COUNT);
     P.ring = carve<TallyRec>(p, kRingLen);
     P.total = carve<TallyRec>(p, 1);
@@ -541,7 +541,7 @@ int commit(slpic_ctx* c) {
                  ((sizeof(InstState) * c->n_inst + 255) & ~size_t(255)) +
                  ((sizeof(SpeciesState) * nseg + 255) & ~size_t(255)) +
                  ((sizeof(Transfer) * nseg + 255) & ~size_t(255)) + 256 +
-                 6 * ((4 * (nseg + 1) + 255) & ~size_t(255)) + 256 +
+                 8 * ((4 * (nseg + 1) + 255) & ~size_t(255)) + 256 +
                  ((4 * coll_items + 255) & ~size_t(255)) +
                  ((sizeof(BirthBase) * c->n_inst + 255) & ~size_t(255)) +
                  ((sizeof(ChunkStatus) * move_chunks + 255) & ~size_t(255));
@@ -560,6 +560,15 @@ int commit(slpic_ctx* c) {
   c->refs.move_start = carve<unsigned int>(p, nseg + 1);
   c->refs.coll_tiles = carve<unsigned int>(p, nseg + 1);
   c->refs.coll_room = carve<unsigned int>(p, nseg + 1);
+  c->refs.birth_start = carve<unsigned int>(p, nseg + 1);
+  c->refs.field_start = carve<int>(p, nseg + 1);
+  {
+    std::vector<int> f(c->n_inst + 1, 0);
+    for (int i = 0; i < c->n_inst; ++i) f[i + 1] = f[i] + c->hi[i].n_cells / kFieldNodes + 1;
+    CK(cudaMemcpy(c->refs.field_start, f.data(), f.size() * 4, cudaMemcpyHostToDevice),
+       "control");
+    c->refs.n_field = f[c->n_inst];
+  }
   c->refs.item_births = carve<uint32_t>(p, coll_items);
   c->refs.birth_base = carve<BirthBase>(p, c->n_inst);
   c->refs.move_scan = carve<ChunkStatus>(p, move_chunks);
@@ -608,12 +617,6 @@ int commit(slpic_ctx* c) {
     if (int e2 = push_config(c->fp64, 0, &gw, &gbps))
       return cuda_fail(c, (cudaError_t)e2, "particle kernel configuration");
     if (gbps > 0 && gw > warps) max_warps = gw;
-  }
-  {
-    int net_nodes = 0;
-    if (int e2 = finish_config(max_nodes, &net_nodes))
-      return cuda_fail(c, (cudaError_t)e2, "finish kernel configuration");
-    c->refs.finish_net_nodes = net_nodes;
   }
   if (int e2 = collide_config(c->fp64, max_nodes, &c->collide_resident, &c->refs.coll_nodes))
     return cuda_fail(c, (cudaError_t)e2, "collision kernel configuration");

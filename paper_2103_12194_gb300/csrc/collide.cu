@@ -99,6 +99,9 @@ __global__ void __launch_bounds__(coll_warps<R>() * 32, sizeof(R) == 4 ? 1 : 3)
   Control* ctrl = r.ctrl;
   if (*((volatile int*)&ctrl->error)) return;
   const unsigned int n_items = ctrl->n_coll_items;
+  // (k_finish plans the next step while the births are still placed)
+  if (blockIdx.x == 0)
+    for (int i = threadIdx.x; i <= r.n_inst; i += blockDim.x) r.birth_start[i] = r.coll_start[i];
   const unsigned int i0 = (unsigned int)((unsigned long long)blockIdx.x * n_items / gridDim.x);
   const unsigned int i1 =
       (unsigned int)((unsigned long long)(blockIdx.x + 1) * n_items / gridDim.x);
@@ -336,6 +339,7 @@ __global__ void __launch_bounds__(coll_warps<R>() * 32, sizeof(R) == 4 ? 1 : 3)
             b.next_id[1] = si.next_id;
             b.step = step;
             b.e_items = e_items;
+            b.tiles = wt;
             r.birth_base[inst] = b;
             if (b.tail[0] + P.acc[ACC_SEE] > (unsigned long long)E.cap_tiles * kTile)
               atomicCAS(&ctrl->error, 0, kErrCapacity);

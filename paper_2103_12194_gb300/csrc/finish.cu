@@ -1,13 +1,13 @@
-// End of a step.  k_finish (one CTA per instance) updates the marker counts
-// from the step's exact counters (the particle kernel compacted every tile,
-// k_collide counted every birth), decides whether a store is repacked,
-// publishes the step's deposit, solves the 1D Poisson equation for the next
-// step's field (its exact integer sums) and commits the step's tallies; the
-// last CTA plans the next step.  k_move evaluates the field from those sums
-// over the whole grid and repacks the stores that became sparse.  With an imposed
-// field the step deposits nothing and k_deposit forms the deposit from the
-// markers when it is read.  Also: seeding, load validation and the Philox
-// self-check kernel.
+// End of a step.  k_finish updates the marker counts of every instance from
+// the step's exact counters (the particle kernel compacted every tile,
+// k_collide counted every birth), decides whether a store is repacked, commits
+// the step's tallies and plans the next step; beside this it publishes the
+// step's deposit with the sums of its net charge, block by block, and appends
+// the step's births to the stores.  k_move evaluates the field of the 1D
+// Poisson equation from those sums and repacks the stores that became sparse.
+// With an imposed field the step deposits nothing and k_deposit forms the
+// deposit from the markers when it is read.  Also: seeding, loading and reading
+// markers and the Philox self-check kernel.
 #include <algorithm>
 
 #include "device_common.cuh"
@@ -49,6 +49,90 @@ __device__ __forceinline__ void plan_totals(const DeviceRefs& r, int n_seg, unsi
   r.ctrl->move_counter = 0;
   r.ctrl->epoch = (r.ctrl->epoch + 1u) & 0x3FFFFFFFu;
   r.ctrl->finish_done = 0;
+}
+
+// Instance of block u of the nodes of all instances.
+__device__ __forceinline__ int field_inst(const DeviceRefs& r, int u) {
+  int lo = 0, hi = r.n_inst - 1;  // last instance with field_start <= u
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (r.field_start[mid] <= u) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
+// Block `block` of the node field of instance P's last Poisson solve, by the
+// kMoveThreads threads of a CTA.
+//   (phi[k+1] - 2 phi[k] + phi[k-1]) = -C net_k, k = 1 .. N-1.  With D_k =
+// phi[k] - phi[k-1]: D_k = D_1 - C I_k, I_k = sum_{0<j<k} net_j, and phi[N] = V
+// fixes D_1 = (V + C J_N) / N, J_N = sum_{0<i<=N} I_i = sum_{0<j<N} (N - j) net_j.
+// The node field is the centred difference of phi, written with these exact
+// integer sums: E_k = -(D_k + D_{k+1}) / (2 dx) = -(2 D_1 - C (I_k + I_{k+1}))
+// / (2 dx), one-sided at the electrodes.  k_finish has left every block's
+// sums; phi is formed on demand (k_phi) when it is read.
+struct FieldShared {
+  long long S;     // net charge of the blocks before
+  double D1;
+  long long w[kMoveThreads / 32];
+};
+__device__ __forceinline__ void poisson_field(const InstDev& P, int block, FieldShared& sh) {
+  constexpr int kPer = kFieldNodes / kMoveThreads;
+  static_assert(kPer == 4, "two 16-byte loads of each deposit");
+  const int N = P.n_cells, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int k0 = block * kFieldNodes + t * kPer;
+  long long net[kPer] = {0, 0, 0, 0};
+#pragma unroll
+  for (int j = 0; j < kPer; ++j) {
+    const int k = k0 + j;
+    if (k > 0 && k < N) net[j] = P.rho_last[kIon][k] - P.rho_last[kElectron][k];
+  }
+  if (warp == 0) {
+    const int nb = N / kFieldNodes + 1;
+    long long S = 0;
+    __int128 W = 0;
+    for (int b = lane; b < nb; b += 32) {
+      if (b < block) S += P.pois_S[b];
+      W += P.pois_W[b];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      S += __shfl_xor_sync(0xFFFFFFFFu, S, o);
+      const unsigned long long wl = __shfl_xor_sync(0xFFFFFFFFu, (unsigned long long)W, o);
+      const long long wh = __shfl_xor_sync(0xFFFFFFFFu, (long long)(W >> 64), o);
+      W += (__int128)(((unsigned __int128)(unsigned long long)wh << 64) | wl);
+    }
+    // one thread forms D_1 (FP64 is scarce on this part) and shares it
+    if (lane == 0) {
+      sh.S = S;
+      sh.D1 = (P.V + P.pois_C * (double)W) / (double)N;
+    }
+  }
+  const long long loc = net[0] + net[1] + net[2] + net[3];
+  const long long inc = warp_incl_scan(loc, lane);
+  if (lane == 31) sh.w[warp] = inc;
+  __syncthreads();
+  long long I = sh.S + inc - loc;  // I_{k0}
+#pragma unroll
+  for (int w = 0; w < kMoveThreads / 32; ++w)
+    if (w < warp) I += sh.w[w];
+  const double D1 = sh.D1, C = P.pois_C;
+  const double inv2dx = 1.0 / (2.0 * P.dx);
+  const double twoD1 = D1 + D1;
+#pragma unroll
+  for (int j = 0; j < kPer; ++j) {
+    const int k = k0 + j;
+    if (k > N) break;
+    const long long I1 = I + net[j];
+    double e;
+    if (k == 0) e = -D1 / P.dx;  // I_1 = 0: D_1
+    else if (k < N) e = -(twoD1 - C * (double)(I + I1)) * inv2dx;
+    else e = -(D1 - C * (double)I) / P.dx;
+    P.E64[k] = e;
+    P.E32[k] = (float)e;
+    I = I1;
+  }
+  __syncthreads();  // sh is free for the next block
 }
 
 // Tiles per electron collision item of an instance of n_tiles electron tiles:
@@ -186,7 +270,7 @@ __device__ void plan_next(const DeviceRefs& r, long long* s_buf) {
 template <typename R>
 __device__ __noinline__ void place_births(const DeviceRefs& r, int b, int nb, uint32_t* s_pre,
                                           long long* s_i64) {
-  const unsigned int n_items = r.ctrl->n_coll_items;
+  const unsigned int n_items = r.birth_start[r.n_inst];
   const unsigned int per = (n_items + nb - 1) / nb;
   unsigned int i0 = (unsigned int)b * per;
   const unsigned int i1 = min(i0 + per, n_items);
@@ -196,17 +280,17 @@ __device__ __noinline__ void place_births(const DeviceRefs& r, int b, int nb, ui
     int lo = 0, hi = r.n_inst - 1;  // last instance with coll_start <= i0
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
-      if (r.coll_start[mid] <= i0) lo = mid;
+      if (r.birth_start[mid] <= i0) lo = mid;
       else hi = mid - 1;
     }
     inst = lo;
   }
   for (; i0 < i1; ++inst) {
-    const unsigned int first = r.coll_start[inst], end = min(i1, r.coll_start[inst + 1]);
+    const unsigned int first = r.birth_start[inst], end = min(i1, r.birth_start[inst + 1]);
     if (end <= i0) continue;  // an instance without items
     const InstDev& P = r.inst[inst];
     const BirthBase B = r.birth_base[inst];
-    const uint32_t wt = r.coll_tiles[inst];
+    const uint32_t wt = B.tiles;
     const uint32_t step = B.step;
     // births of the instance before item i0
     long long before;
@@ -266,62 +350,69 @@ __device__ __noinline__ void place_births(const DeviceRefs& r, int b, int nb, ui
   }
 }
 
-// The end of a step of instance inst, by one CTA.
-__device__ __forceinline__ void finish_instance(const DeviceRefs& r, int inst, int net_nodes,
-                                                long long* s_dyn, long long* s_i64,
-                                                __int128* s_i128, unsigned long long* s_acc) {
+// What the state CTA of an instance keeps in shared memory.
+struct StateShared {
+  unsigned long long acc[ACC_COUNT];
+  InstState is;
+  SpeciesState st[2];
+  Transfer x[2];
+};
+
+// The plan of a single instance, by one thread, from what its state CTA holds.
+__device__ __forceinline__ void plan_single(const DeviceRefs& r, const StateShared& sh,
+                                            unsigned int room) {
+  unsigned int ns = 0, w = 0, mv = 0;
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    r.seg_start[s] = ns;
+    r.seg_wstart[s] = w;
+    r.move_start[s] = mv;
+    ns += sh.st[s].n_tiles;
+    w += sh.st[s].n_tiles * (s ? kWeightIon : kWeightElectron);
+    if (sh.x[s].compact) mv += (sh.x[s].n_tiles_old + kMoveChunkTiles - 1) / kMoveChunkTiles;
+  }
+  const unsigned int T = item_tiles(room, sh.st[0].n_tiles, 1, r.fp64);
+  r.coll_tiles[0] = T;
+  r.coll_start[0] = 0u;
+  plan_totals(r, 2, ns, w, mv,
+              (sh.st[0].n_tiles + T - 1) / T +
+                  (sh.st[1].n_tiles + kCollIonTiles - 1) / kCollIonTiles);
+}
+
+// The end of a step of instance inst: counts, fills, tallies.  A chain of
+// global round trips, so every load that can be is issued at the start.
+// Returns the tiles that hold about kCollTarget candidates.
+__device__ __forceinline__ unsigned int finish_state(const DeviceRefs& r, int inst,
+                                                     StateShared& sh) {
   const int t = threadIdx.x;
   const InstDev& P = r.inst[inst];
-  InstState& is = r.istate[inst];
   unsigned long long* a = P.acc;
-  const int N = P.n_cells, nn = N + 1;
-  long long* s_net = nn <= net_nodes ? s_dyn : nullptr;
-
-  // ---- accumulators and the step's deposit, all threads at once -------------
-  // deposit -> rho_last (and the net charge to shared memory); clear both
+  const long long total = t < kTallySlots ? reinterpret_cast<long long*>(P.total)[t] : 0ll;
   if (t < ACC_COUNT) {
-    s_acc[t] = a[t];
+    sh.acc[t] = a[t];
     a[t] = 0ull;
   }
-  // (with an imposed field nothing was deposited: the deposit is formed from
-  // the markers when it is read)
-  // (four nodes per thread at a time: their loads are issued before any store)
-  for (int k0 = t; k0 < nn && P.field_mode == 1; k0 += 4 * kFinThreads) {
-    long long qe[4], qi[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int k = k0 + u * kFinThreads;
-      qe[u] = k < nn ? (long long)P.rho_acc[kElectron][k] : 0ll;
-      qi[u] = k < nn ? (long long)P.rho_acc[kIon][k] : 0ll;
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int k = k0 + u * kFinThreads;
-      if (k >= nn) break;
-      P.rho_last[kElectron][k] = qe[u];
-      P.rho_last[kIon][k] = qi[u];
-      P.rho_acc[kElectron][k] = 0ull;
-      P.rho_acc[kIon][k] = 0ull;
-      if (s_net) s_net[k] = qi[u] - qe[u];
-    }
+  if (t == 32) sh.is = r.istate[inst];
+  uint32_t tail = 0;
+  if (t < 2) {
+    const SpeciesState st = r.sstate[inst * 2 + t];
+    sh.st[t] = st;
+    tail = tail_slot(P.sp[t], st);
   }
   __syncthreads();
 
   // ---- marker counts and where the stores end (one thread per species) -------
   // survivors = live - absorbed; births (ionizations: an electron and an ion
-  // each; emitted electrons) were appended after the last live marker
+  // each; emitted electrons) are appended after the last live marker
+  unsigned int room = 0;
   if (t < 2) {
     const int sp = t;
-    const uint32_t n_ionz = (uint32_t)s_acc[ACC_COLL2], n_see = (uint32_t)s_acc[ACC_SEE];
-    SpeciesState& st = r.sstate[inst * 2 + sp];
-    const SpeciesDev& S = P.sp[sp];
-    Transfer& x = r.xfer[inst * 2 + sp];
-    const uint32_t absorbed = (uint32_t)(s_acc[ACC_NABS + 2 * sp] + s_acc[ACC_NABS + 2 * sp + 1]);
+    const uint32_t n_ionz = (uint32_t)sh.acc[ACC_COLL2], n_see = (uint32_t)sh.acc[ACC_SEE];
+    const uint32_t absorbed =
+        (uint32_t)(sh.acc[ACC_NABS + 2 * sp] + sh.acc[ACC_NABS + 2 * sp + 1]);
     const uint32_t nb = sp ? n_ionz : n_ionz + n_see;
-    const SpeciesState s0 = st;
+    const SpeciesState s0 = sh.st[sp];
     const uint32_t surv = s0.n_live - absorbed;
-    const uint32_t tail =
-        s0.n_tiles ? (s0.n_tiles - 1) * (uint32_t)kTile + S.fill[s0.cur][s0.n_tiles - 1] : 0u;
     const uint32_t end = tail + nb;
     const uint32_t n_new = surv + nb;
     const uint32_t nt = (end + kTile - 1) / kTile;
@@ -331,6 +422,7 @@ __device__ __forceinline__ void finish_instance(const DeviceRefs& r, int inst, i
     // half the rate in its last steps)
     const uint32_t compact =
         (nt > 2 && (unsigned long long)n_new * 16 < (unsigned long long)nt * kTile * 15) ? 1u : 0u;
+    Transfer x;
     x.compact = compact;
     x.src = s0.cur;
     x.dst = compact ? s0.cur ^ 1u : s0.cur;
@@ -338,74 +430,84 @@ __device__ __forceinline__ void finish_instance(const DeviceRefs& r, int inst, i
     x.n_new = n_new;
     x.tail = tail;
     x.end = end;
-    if (sp == kElectron) {
-      // tiles that hold about kCollTarget candidates at this step's density
-      const unsigned long long cand = s_acc[ACC_CAND];
-      const unsigned long long room =
-          cand ? (unsigned long long)kCollTarget * s0.n_tiles / cand
-               : (unsigned long long)kCollMaxRoom;
-      r.coll_room[inst] = (unsigned int)min(max(room, 1ull), (unsigned long long)kCollMaxRoom);
-    }
+    x.pad = 0u;
     SpeciesState s1;
     s1.cur = x.dst;
     s1.n_live = n_new;
     s1.next_id = s0.next_id + nb;
     s1.n_tiles = compact ? (n_new + kTile - 1) / kTile : nt;
-    st = s1;
+    sh.x[sp] = x;
+    sh.st[sp] = s1;
+    r.xfer[inst * 2 + sp] = x;
+    r.sstate[inst * 2 + sp] = s1;
+    if (sp == kElectron) {
+      // tiles that hold about kCollTarget candidates at this step's density
+      const unsigned long long cand = sh.acc[ACC_CAND];
+      const unsigned long long fit =
+          cand ? (unsigned long long)kCollTarget * s0.n_tiles / cand
+               : (unsigned long long)kCollMaxRoom;
+      room = (unsigned int)min(max(fit, 1ull), (unsigned long long)kCollMaxRoom);
+      r.coll_room[inst] = room;
+    }
   }
   __syncthreads();
   // fills of the tail tile and the new tiles: their slots below `end` are live
   // (k_move reads them when it repacks the store)
   for (int sp = 0; sp < 2; ++sp) {
-    const SpeciesDev& S = P.sp[sp];
-    const Transfer& x = r.xfer[inst * 2 + sp];
+    const Transfer& x = sh.x[sp];
     if (x.end == x.tail) continue;
+    uint32_t* const fill = P.sp[sp].fill[x.src];
     for (uint32_t k = x.tail / kTile + t; k < x.n_tiles_old; k += kFinThreads)
-      S.fill[x.src][k] = min(x.end - k * (uint32_t)kTile, (uint32_t)kTile);
+      fill[k] = min(x.end - k * (uint32_t)kTile, (uint32_t)kTile);
   }
-
-  // ---- Poisson: (phi[k+1] - 2 phi[k] + phi[k-1]) = -C net_k, k = 1..N-1 ----
-  // With D_k = phi[k] - phi[k-1]: D_k = D_1 - C I_k, I_k = sum_{0<j<k} net_j,
-  // and phi[N] = V fixes D_1 = (V + C J_N) / N, J_N = sum_{0<i<=N} I_i.
-  // The node field is the centred difference of phi, written with the exact
-  // integer sums: E_k = -(D_k + D_{k+1}) / (2 dx) = -(2 D_1 - C (I_k + I_{k+1}))
-  // / (2 dx), one-sided at the electrodes.  This CTA leaves I_k and D_1; k_move,
-  // which follows every step on many SMs, evaluates E in FP64 (poisson_field),
-  // and phi is formed on demand (k_phi) when it is read.
-  if (P.field_mode == 1) {
-    const int chunk = (N + kFinThreads - 1) / kFinThreads;  // over k = 1..N
-    const int k0 = 1 + t * chunk;
-    long long I0;
-    const double D1 = poisson_d1(P, s_net, k0, chunk, s_i64, s_i128, &I0);
-    long long Ik = I0;
-    for (int k = k0; k < k0 + chunk && k <= N; ++k) {
-      P.pois_I[k] = Ik;
-      if (k <= N - 1) Ik += net_at(P, s_net, k);
-    }
-    if (t == 0) *P.pois_D1 = D1;
-  }
-
   // ---- tallies: one thread per 8-byte slot of the record ---------------------
   if (t < kTallySlots)
-    commit_tally_slot(P, t, s_acc, is.step, is.n_steps_done, r.sstate[inst * 2].n_live,
-                      r.sstate[inst * 2 + 1].n_live, is.w_live, &is.ion_steps);
+    commit_tally_slot(P, t, sh.acc, sh.is.step, sh.is.n_steps_done, sh.st[0].n_live,
+                      sh.st[1].n_live, sh.is.w_live, &sh.is.ion_steps, total);
   __syncthreads();
-  if (t == 0) {
-    is.step += 1u;
-    is.n_steps_done += 1;
+  if (t == 32) {
+    sh.is.step += 1u;
+    sh.is.n_steps_done += 1;
+    r.istate[inst] = sh.is;
+  }
+  return room;
+}
+
+// One block of kFieldNodes nodes of an instance: the step's deposit becomes
+// the last step's, and the block leaves its sums of the net charge net_j
+// (0 < j < N) for the field: S = sum net_j and W = sum (N - j) net_j.
+__device__ __forceinline__ void finish_nodes(const InstDev& P, int block, long long* s_i64,
+                                             __int128* s_i128) {
+  const int k = block * kFieldNodes + (int)threadIdx.x, N = P.n_cells;
+  long long net = 0;
+  if (k <= N) {
+    const long long qe = (long long)P.rho_acc[kElectron][k], qi = (long long)P.rho_acc[kIon][k];
+    P.rho_last[kElectron][k] = qe;
+    P.rho_last[kIon][k] = qi;
+    P.rho_acc[kElectron][k] = 0ull;
+    P.rho_acc[kIon][k] = 0ull;
+    if (k > 0 && k < N) net = qi - qe;
+  }
+  const long long S = block_incl_scan<long long>(net, s_i64);
+  const __int128 W = block_incl_scan<__int128>((__int128)net * (N - k), s_i128);
+  if (threadIdx.x == kFinThreads - 1) {
+    P.pois_S[block] = S;
+    P.pois_W[block] = W;
   }
 }
 
 }  // namespace
 
-// mode 0: finish a step (CTAs 0 .. n_inst - 1, one per instance; the others
-// place the births; the last one of all plans the next step); mode 1: plan only (one CTA).  Dynamic shared memory: net_nodes
-// int64 nodes for the net deposit (0: read it from global memory).
-__global__ void __launch_bounds__(kFinThreads) k_finish(DeviceRefs r, int mode, int net_nodes) {
-  extern __shared__ long long s_dyn[];
+// mode 0: finish a step.  CTAs 0 .. n_inst - 1, one per instance, update its
+// state (the last one plans the next step); the next n_field take the blocks of
+// nodes of all instances in turn; the last kBirthCtas place the births.  No CTA
+// waits for another, and the longest chain is that of an instance's state: 12
+// us a step at 256 cells with the whole deposit and the Poisson sums in that
+// CTA, 16 at 4096 and 39 at 21832.  mode 1: plan only (one CTA).
+__global__ void __launch_bounds__(kFinThreads) k_finish(DeviceRefs r, int mode, int n_field) {
   __shared__ long long s_i64[32];
   __shared__ __int128 s_i128[32];
-  __shared__ unsigned long long s_acc[ACC_COUNT];
+  __shared__ StateShared sh;
   __shared__ uint32_t s_pre[kFinThreads];
   __shared__ int s_flag;
   step_kernel_entry();
@@ -418,20 +520,35 @@ __global__ void __launch_bounds__(kFinThreads) k_finish(DeviceRefs r, int mode, 
     return;
   }
   if (*((volatile int*)&ctrl->error)) return;
-  if ((int)blockIdx.x >= r.n_inst) {
-    const int b = blockIdx.x - r.n_inst, nb = gridDim.x - r.n_inst;
-    if (r.fp64) place_births<double>(r, b, nb, s_pre, s_i64);
-    else place_births<float>(r, b, nb, s_pre, s_i64);
-  } else {
-    finish_instance(r, blockIdx.x, net_nodes, s_dyn, s_i64, s_i128, s_acc);
+  int b = blockIdx.x;
+  if (b >= r.n_inst) {
+    b -= r.n_inst;
+    if (b < n_field) {
+      for (int u = b; u < r.field_start[r.n_inst]; u += n_field) {
+        const int inst = field_inst(r, u);
+        const InstDev& P = r.inst[inst];
+        // (with an imposed field nothing was deposited: the deposit is formed
+        // from the markers when it is read)
+        if (P.field_mode == 1) finish_nodes(P, u - r.field_start[inst], s_i64, s_i128);
+      }
+    } else if (r.fp64) {
+      place_births<double>(r, b - n_field, kBirthCtas, s_pre, s_i64);
+    } else {
+      place_births<float>(r, b - n_field, kBirthCtas, s_pre, s_i64);
+    }
+    return;
   }
-
-  // ---- the last CTA plans the next step --------------------------------------
+  const unsigned int room = finish_state(r, b, sh);
+  if (r.n_inst == 1) {
+    if (t == 0) plan_single(r, sh, room);
+    return;
+  }
+  // ---- the last instance plans the next step ---------------------------------
   __threadfence();
   __syncthreads();
   if (t == 0) {
     const unsigned int ticket = atomicAdd(&ctrl->finish_done, 1u);
-    s_flag = ticket == gridDim.x - 1 ? 1 : 0;
+    s_flag = ticket == (unsigned int)r.n_inst - 1u ? 1 : 0;
   }
   __syncthreads();
   if (s_flag) {
@@ -439,6 +556,7 @@ __global__ void __launch_bounds__(kFinThreads) k_finish(DeviceRefs r, int mode, 
     plan_next(r, s_i64);
   }
 }
+
 // The deposit of instance inst's live markers into its last-step grids
 // (zeroed by the caller): each marker adds fixed_charge(beta(|v|) w_j) at its
 // position, as the step deposits it.  A step's deposit is a function of the
@@ -559,30 +677,10 @@ void launch_prefix(const uint32_t* fill, uint32_t n_tiles, uint32_t* prefix, uin
   k_prefix<<<1, kFinThreads, 0, s>>>(fill, n_tiles, prefix, total);
 }
 
-// Dynamic shared memory of k_finish: the net deposit of the largest grid,
-// when it fits (DeviceRefs::finish_net_nodes, from finish_config).
-int finish_config(int max_nodes, int* net_nodes) {
-  int dev = 0, optin = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return (int)e;
-  e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (e != cudaSuccess) return (int)e;
-  const int room = (optin - 8 * 1024) / 8;  // static shared memory stays below 8 KB
-  *net_nodes = max_nodes <= room ? max_nodes : 0;
-  // the limit is the most a CTA can have, so that one context's
-  // configuration never lowers it under another's
-  cudaFuncAttributes fa;
-  e = cudaFuncGetAttributes(&fa, k_finish);
-  if (e != cudaSuccess) return (int)e;
-  e = cudaFuncSetAttribute(k_finish, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           optin - (int)fa.sharedSizeBytes);
-  return (int)e;
-}
-
 void launch_finish(const DeviceRefs& r, int mode, cudaStream_t s) {
-  const int grid = mode == 1 ? 1 : r.n_inst + kBirthCtas;
-  const int nodes = mode == 1 ? 0 : r.finish_net_nodes;
-  launch_step_kernel(k_finish, grid, kFinThreads, (size_t)nodes * 8, s, r, mode, nodes);
+  const int n_field = std::min(r.n_field, kFieldCtas);
+  const int grid = mode == 1 ? 1 : r.n_inst + n_field + kBirthCtas;
+  launch_step_kernel(k_finish, grid, kFinThreads, 0, s, r, mode, n_field);
 }
 
 // ---------------------------------------------------------------------------
@@ -597,21 +695,15 @@ __global__ void __launch_bounds__(kMoveThreads) k_move(DeviceRefs r) {
   __shared__ uint32_t s_fill[kMoveChunkTiles];
   __shared__ uint32_t s_pre[kMoveChunkTiles];
   __shared__ unsigned int s_chunk;
+  __shared__ FieldShared s_field;
   constexpr int kPerLaneTiles = kMoveChunkTiles / 32;
   step_kernel_entry();
   Control* ctrl = r.ctrl;
   if (*((volatile int*)&ctrl->error)) return;
-  // the field of the step's Poisson solves: CTA b takes part b / n_inst of
-  // instance b % n_inst (every instance gets gridDim / n_inst CTAs, at least
-  // one), node by node
-  {
-    const int n_inst = r.n_inst;
-    const int parts = max(1, (int)gridDim.x / n_inst);
-    for (int b = blockIdx.x; b < n_inst * parts; b += gridDim.x) {
-      const InstDev& P = r.inst[b % n_inst];
-      if (P.field_mode == 1)
-        poisson_field(P, (b / n_inst) * blockDim.x + threadIdx.x, parts * blockDim.x);
-    }
+  // the field of the step's Poisson solves, a block of nodes at a time
+  for (int u = blockIdx.x; u < r.n_field; u += gridDim.x) {
+    const int inst = field_inst(r, u);
+    if (r.inst[inst].field_mode == 1) poisson_field(r.inst[inst], u - r.field_start[inst], s_field);
   }
   const unsigned int n_chunks = ctrl->n_move_chunks;
   if (n_chunks == 0) return;

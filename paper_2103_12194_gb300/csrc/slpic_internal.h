@@ -262,8 +262,8 @@ struct InstDev {
   float* E32;                   // node field used by the FP32 push
   double* phi;                  // node potential
   double* E64;                  // node field
-  long long* pois_I;            // [nn] I_k = sum_{0<j<k} net_j of the last solve
-  double* pois_D1;              // [1] D_1 of the last solve
+  long long* pois_S;            // per block of kFieldNodes nodes: net charge of the last step
+  __int128* pois_W;             // and its sum weighted by N - node
   unsigned long long* rho_acc[2];  // fixed-point deposit of the current step
   long long* rho_last[2];          // deposit of the last finished step
   unsigned long long* acc;         // ACC_COUNT per-step accumulators
@@ -327,8 +327,11 @@ constexpr int kCollTarget = 128;
 constexpr int kCollSpread = 2432;
 // (a bound of the tiles that hold that many candidates)
 constexpr int kCollMaxRoom = 64 * kCollMaxTiles;
-// CTAs of k_finish beside the instances' own that place the births.
+// CTAs of k_finish beside the instances' own: those that place the births, and
+// at most so many for the blocks of nodes.
 constexpr int kBirthCtas = 64;
+constexpr int kFieldCtas = 80;
+constexpr int kFieldNodes = 1024;
 // Repacking chunks: tiles each.
 constexpr int kMoveChunkTiles = 128;
 // Single-CTA path (small.cu): at most this many tiles per store and instance
@@ -336,10 +339,10 @@ constexpr int kMoveChunkTiles = 128;
 constexpr int kSmallMaxTiles = 32;
 
 // Where a step's births go in the stores of one instance: buffers, first free
-// slots, next serial numbers, step and electron items, before the step's end
-// moves the state on.
+// slots, next serial numbers, step, electron items and their tiles, before the
+// step's end moves the state and the plan on.
 struct BirthBase {
-  uint32_t cur[2], tail[2], next_id[2], step, e_items;
+  uint32_t cur[2], tail[2], next_id[2], step, e_items, tiles;
 };
 
 struct DeviceRefs {
@@ -356,13 +359,15 @@ struct DeviceRefs {
   unsigned int* move_start;  // [n_seg + 1] first repacking chunk of each segment
   uint32_t* item_births;     // [max collision items] births of each item in the step
   BirthBase* birth_base;     // [n_inst]
+  unsigned int* birth_start; // [n_inst + 1] coll_start of the step whose births are placed
+  int* field_start;          // [n_inst + 1] first block of nodes of each instance
   ChunkStatus* move_scan;    // [max repacking chunks]
   int n_inst;
   int smem_nodes;         // deposit grid nodes in shared memory (0: global atomics)
   int push_warps;         // warps per particle-kernel CTA
   int coll_nodes;         // collision kernel: deposit grid nodes in shared memory (0: none)
   int fp64;               // marker path in double precision (else float)
-  int finish_net_nodes;   // k_finish keeps the net deposit of up to this many nodes in shared memory
+  int n_field;            // blocks of kFieldNodes nodes of all instances
 };
 
 // Launchers (defined in the .cu files).
@@ -374,8 +379,6 @@ int push_config(int fp64, int smem_nodes, int* warps, int* blocks_per_sm);
 int push_blocks_per_sm(int fp64, int warps, int smem_nodes, int* blocks_per_sm);
 // mode 0: finish a step and plan the next; mode 1: plan only (one CTA).
 void launch_finish(const DeviceRefs& r, int mode, cudaStream_t s);
-// Shared-memory room of k_finish for the largest grid (0: read from global).
-int finish_config(int max_nodes, int* net_nodes);
 void launch_move(const DeviceRefs& r, int grid, cudaStream_t s);
 // Node potential of instance inst from its last deposit (Poisson mode).
 void launch_phi(const DeviceRefs& r, int inst, cudaStream_t s);

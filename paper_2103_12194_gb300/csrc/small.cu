@@ -555,7 +555,8 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
     // ---- tallies ---------------------------------------------------------------
     if (t < kTallySlots)
       commit_tally_slot(P, t, sh.acc, sh.step, sh.n_steps_done, sh.st[0].n_live,
-                        sh.st[1].n_live, sh.w_live, &sh.ion_steps);
+                        sh.st[1].n_live, sh.w_live, &sh.ion_steps,
+                        reinterpret_cast<const long long*>(P.total)[t]);
     __syncthreads();
     if (t < ACC_COUNT) sh.acc[t] = 0ull;
     if (t == 0) {

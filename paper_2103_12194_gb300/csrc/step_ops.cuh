@@ -432,30 +432,6 @@ __device__ double poisson_d1(const InstDev& P, const long long* s_net, int k0, i
   return D1;
 }
 
-// The node field of instance P's last Poisson solve from its exact integer
-// sums (k_finish leaves I_k and D_1): the centred difference of phi,
-// E_k = -(2 D_1 - C (I_k + I_{k+1})) / (2 dx), one-sided at the electrodes,
-// for the nodes k = k0, k0 + stride, ...
-__device__ __forceinline__ void poisson_field(const InstDev& P, int k0, int stride) {
-  const int N = P.n_cells;
-  const double D1 = *P.pois_D1;
-  const double C = P.pois_C;
-  const double inv2dx = 1.0 / (2.0 * P.dx);
-  const double twoD1 = D1 + D1;
-  for (int k = k0; k <= N; k += stride) {
-    double e;
-    if (k == 0) {
-      e = -D1 / P.dx;  // I_1 = 0: D_1
-    } else if (k <= N - 1) {
-      e = -(twoD1 - C * (double)(P.pois_I[k] + P.pois_I[k + 1])) * inv2dx;
-    } else {
-      e = -(D1 - C * (double)P.pois_I[k]) / P.dx;  // k = N
-    }
-    P.E64[k] = e;
-    P.E32[k] = (float)e;
-  }
-}
-
 // Record of one step (TallyRec) from its accumulators q: thread t < kTallySlots
 // writes 8-byte slot t to the history ring and the totals.  Slot layout: 0
 // step, 1-2 n_live, 3-4 w_live, 5-7 n_coll, 8 n_candidates, 9-12 n_abs, 13-16
@@ -463,7 +439,8 @@ __device__ __forceinline__ void poisson_field(const InstDev& P, int k0, int stri
 // n_clamp, 23 n_majorant, 24 marker_steps, 25 w_gain_gen0; slots 0-4 are
 // states (replaced in the totals), the others sums.  n_live_* are the counts
 // after the step; w_live (fixed point, per species) is updated by its changes,
-// and ion_steps gains the step's live ions.
+// and ion_steps gains the step's live ions.  total: the slot's bits in the
+// totals before the step.
 constexpr int kTallySlots = (int)(sizeof(TallyRec) / 8);
 static_assert(kTallySlots == 26, "TallyRec layout");
 
@@ -471,7 +448,7 @@ __device__ __forceinline__ void commit_tally_slot(const InstDev& P, int t,
                                                   const unsigned long long* q, uint32_t step,
                                                   long long n_steps_done, uint32_t n_live_e,
                                                   uint32_t n_live_i, unsigned long long* w_live,
-                                                  long long* ion_steps) {
+                                                  long long* ion_steps, long long total) {
   const double unit = 1.0 / P.c64.wscale;
   long long iv = 0;
   double dv = 0.0;
@@ -519,12 +496,10 @@ __device__ __forceinline__ void commit_tally_slot(const InstDev& P, int t,
   long long* tot = reinterpret_cast<long long*>(P.total);
   if (is_double) {
     reinterpret_cast<double*>(ring)[t] = dv;
-    if (t <= 4) reinterpret_cast<double*>(tot)[t] = dv;
-    else reinterpret_cast<double*>(tot)[t] += dv;
+    reinterpret_cast<double*>(tot)[t] = t <= 4 ? dv : __longlong_as_double(total) + dv;
   } else {
     ring[t] = iv;
-    if (t <= 4) tot[t] = iv;
-    else tot[t] += iv;
+    tot[t] = t <= 4 ? iv : total + iv;
   }
 }
 
