@@ -625,7 +625,7 @@ int commit(slpic_ctx* c) {
   c->sms = sms;
   c->max_push_warps = max_warps;
   c->blocks_per_sm = bps;
-  c->push_grid = sms * bps;
+  c->push_grid = c->refs.push_grid = sms * bps;
   c->move_grid = sms * 2;
   c->collide_grid = sms * std::min(c->collide_per_sm, c->collide_resident);
   c->hs.assign(nseg, SpeciesState{});
@@ -794,7 +794,7 @@ int apply_shape(slpic_ctx* c, int warps, int coll_per_sm) {
   c->refs.smem_nodes = nodes;
   c->refs.push_warps = warps;
   c->blocks_per_sm = bps;
-  c->push_grid = c->sms * bps;
+  c->push_grid = c->refs.push_grid = c->sms * bps;
   c->collide_per_sm = coll_per_sm;
   c->collide_grid = c->sms * std::min(coll_per_sm, c->collide_resident);
   c->plan_due = true;

@@ -146,6 +146,16 @@ __device__ __forceinline__ unsigned int item_tiles(unsigned long long room, uint
   return (unsigned int)min(max(most, 1ull), (unsigned long long)kCollMaxTiles);
 }
 
+// Weight of starting a segment, in the particle kernel's split of `total`
+// weights over its CTAs: a barrier, a flush of the charge grid and an empty
+// pipeline, about as long as 16 electron tiles of a CTA.  (A CTA whose range
+// held ten small gaps took far longer than the others: k_push on 32 uneven gaps
+// 242 us, 201 with this; 24 or 96 instead of 48 run the same.)  No more than a CTA's share, which populations
+// of few tiles are spread over.
+__device__ __forceinline__ long long seg_cost(const DeviceRefs& r, long long total) {
+  return min((long long)kSegCost, total / r.push_grid);
+}
+
 // The plan below by one warp (n_seg <= 32 kPlanPerLane), with shuffle scans
 // and no block barrier.
 __device__ void plan_next_warp(const DeviceRefs& r) {
@@ -179,7 +189,19 @@ __device__ void plan_next_warp(const DeviceRefs& r) {
     }
     s_nc += nc[j];
   }
-  const long long i_ns = warp_incl_scan(s_ns, lane), i_w = warp_incl_scan(s_w, lane);
+  const long long i_ns = warp_incl_scan(s_ns, lane);
+  long long i_w = warp_incl_scan(s_w, lane);
+  // and the cost of every segment that is not empty
+  const long long cost = seg_cost(r, __shfl_sync(0xFFFFFFFFu, i_w, 31));
+  long long s_c = 0;
+#pragma unroll
+  for (int j = 0; j < kPlanPerLane; ++j) {
+    const long long c = ns[j] ? cost : 0;
+    w[j] += c;
+    s_c += c;
+  }
+  s_w += s_c;
+  i_w += warp_incl_scan(s_c, lane);
   const long long i_mv = warp_incl_scan(s_mv, lane), i_nc = warp_incl_scan(s_nc, lane);
   long long e_ns = i_ns - s_ns, e_w = i_w - s_w, e_mv = i_mv - s_mv, e_nc = i_nc - s_nc;
 #pragma unroll
@@ -200,30 +222,44 @@ __device__ void plan_next_warp(const DeviceRefs& r) {
     if (i < r.n_inst) r.coll_start[i] = (unsigned int)e_nc;
     e_nc += nc[j];
   }
-  if (lane == 31)
+  if (lane == 31) {
+    r.ctrl->seg_cost = (unsigned int)cost;
     plan_totals(r, n_seg, (unsigned int)i_ns, (unsigned int)i_w, (unsigned int)i_mv,
                 (unsigned int)i_nc);
+  }
 }
 
 // Plan the next step from the tiles in use (all threads of one CTA):
 // particle-kernel tiles and their weights per segment, repacking chunks per segment and collision items per instance,
 // as exclusive block scans in rounds of kFinThreads entries.
 __device__ void plan_next(const DeviceRefs& r, long long* s_buf) {
-  __shared__ long long s_carry[4];
+  __shared__ long long s_carry[5];
   const int n_seg = r.n_inst * 2;
   if (n_seg <= 32 * kPlanPerLane) {
     if (threadIdx.x < 32) plan_next_warp(r);
     return;
   }
   const int t = threadIdx.x;
-  if (t < 4) s_carry[t] = 0;
+  if (t < 5) s_carry[t] = 0;
   __syncthreads();
+  // the summed weights of the tiles give the cost of a segment
+  for (int base = 0; base < n_seg; base += kFinThreads) {
+    const int sg = base + t;
+    const long long w = sg < n_seg ? (long long)r.sstate[sg].n_tiles *
+                                         ((sg & 1) ? kWeightIon : kWeightElectron)
+                                   : 0;
+    const long long i_w = block_incl_scan<long long>(w, s_buf);
+    if (t == kFinThreads - 1) s_carry[4] += i_w;
+  }
+  __syncthreads();
+  const long long cost = seg_cost(r, s_carry[4]);
+  if (t == 0) r.ctrl->seg_cost = (unsigned int)cost;
   for (int base = 0; base < n_seg; base += kFinThreads) {
     const int sg = base + t;
     long long ns = 0, w = 0, mv = 0;
     if (sg < n_seg) {
       ns = r.sstate[sg].n_tiles;
-      w = ns * ((sg & 1) ? kWeightIon : kWeightElectron);
+      w = ns * ((sg & 1) ? kWeightIon : kWeightElectron) + (ns ? cost : 0);
       const Transfer& x = r.xfer[sg];
       if (x.compact) mv = ((long long)x.n_tiles_old + kMoveChunkTiles - 1) / kMoveChunkTiles;
     }
@@ -371,6 +407,7 @@ __device__ __forceinline__ void plan_single(const DeviceRefs& r, const StateShar
     w += sh.st[s].n_tiles * (s ? kWeightIon : kWeightElectron);
     if (sh.x[s].compact) mv += (sh.x[s].n_tiles_old + kMoveChunkTiles - 1) / kMoveChunkTiles;
   }
+  r.ctrl->seg_cost = 0u;
   const unsigned int T = item_tiles(room, sh.st[0].n_tiles, 1, r.fp64);
   r.coll_tiles[0] = T;
   r.coll_start[0] = 0u;

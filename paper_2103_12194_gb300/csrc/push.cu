@@ -105,7 +105,9 @@ __device__ __forceinline__ unsigned int first_tile(const DeviceRefs& r, unsigned
     else hi = mid - 1;
   }
   const unsigned int w = (lo & 1) ? kWeightIon : kWeightElectron;
-  const unsigned int q = r.seg_start[lo] + (target - r.seg_wstart[lo] + w - 1) / w;
+  // (a segment's weight begins with the cost of starting it)
+  const unsigned int at = target - r.seg_wstart[lo], cost = r.ctrl->seg_cost;
+  const unsigned int q = r.seg_start[lo] + (at > cost ? at - cost + w - 1 : 0u) / w;
   return min(q, r.seg_start[lo + 1]);
 }
 

@@ -45,6 +45,7 @@ __host__ __device__ constexpr size_t tile_bytes_read(bool all, bool w) {
 // 18 % slower on a grid of 21832 cells, whose ions wait for global atomics.)
 constexpr unsigned int kWeightElectron = 3;
 constexpr unsigned int kWeightIon = 2;
+constexpr unsigned int kSegCost = 48;
 
 // Device error word values (copied to the host status codes).
 constexpr int kErrNone = 0;
@@ -289,6 +290,7 @@ struct Control {
   unsigned int epoch;        // step epoch of the look-back records
   unsigned int n_tiles;      // particle-kernel tiles this step
   unsigned int w_total;      // their summed weights
+  unsigned int seg_cost;     // of which for starting a segment that is not empty
   unsigned int n_seg;        // segments = instances * 2
   unsigned int finish_done;  // CTAs of the finish kernel that completed
   int error;                 // first device error (kErr*)
@@ -365,6 +367,7 @@ struct DeviceRefs {
   int n_inst;
   int smem_nodes;         // deposit grid nodes in shared memory (0: global atomics)
   int push_warps;         // warps per particle-kernel CTA
+  int push_grid;          // its CTAs
   int coll_nodes;         // collision kernel: deposit grid nodes in shared memory (0: none)
   int fp64;               // marker path in double precision (else float)
   int n_field;            // blocks of kFieldNodes nodes of all instances
