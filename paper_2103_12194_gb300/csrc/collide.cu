@@ -167,8 +167,8 @@ __global__ void __launch_bounds__(coll_warps<R>() * 32, sizeof(R) == 4 ? 1 : 3)
       m.vz() = nv.vz;
       if (dep)
         deposit(rho_e, cell, off,
-                fixed_charge(beta_of(r_sqrt(nv.vx * nv.vx + nv.vy * nv.vy + nv.vz * nv.vz),
-                                     vlim) * wj, wscale));
+                fixed_charge(beta_any(nv.vx * nv.vx + nv.vy * nv.vy + nv.vz * nv.vz, vlim) * wj,
+                             wscale));
     };
     uint32_t e_head = 0, e_tail = 0, n_head = 0, n_tail = 0;
     // scatter the n <= 32 oldest elastic (inelastic) entries, lane l the l-th
@@ -191,11 +191,8 @@ __global__ void __launch_bounds__(coll_warps<R>() * 32, sizeof(R) == 4 ? 1 : 3)
         u3 = Q.e_u3[i];
       }
       __syncwarp();  // the entries are read before the next round refills them
-      if (on) {
-        const R v1 = r_sqrt(vx * vx + vy * vy + vz * vz);
-        finish_one(slot, cell, off, wj,
-                   scatter_elastic<R>(K, kv, vx, vy, vz, v1, eps, u2, u3));
-      }
+      if (on)
+        finish_one(slot, cell, off, wj, scatter_elastic_any(K, kv, vx, vy, vz, eps, u2, u3));
       e_head += n;
     };
     auto drain_inelastic = [&](uint32_t n) {
@@ -274,11 +271,11 @@ __global__ void __launch_bounds__(coll_warps<R>() * 32, sizeof(R) == 4 ? 1 : 3)
         R u[4] = {0, 0, 0, 0}, eps = 0;
         if (on) {
           const R s1 = cr.vx * cr.vx + cr.vy * cr.vy + cr.vz * cr.vz;
-          const R v1 = r_sqrt(s1);
+          const R v1 = sqrt_any(s1);
           const uint4 rr = philox4x32_10(make_uint4(cr.id, step, ctr2, 0u), key0, key1);
           proc = choose_process<R>(P, vlim, v1, s1, rr, acc, u, eps, kx);
           if (proc == 3 && dep)  // null: the velocity is kept
-            deposit(rho_e, cr.cell, cr.off, fixed_charge(beta_of(v1, vlim) * cr.wj, wscale));
+            deposit(rho_e, cr.cell, cr.off, fixed_charge(beta_any(s1, vlim) * cr.wj, wscale));
         }
         const uint32_t be = __ballot_sync(0xFFFFFFFFu, proc == 0);
         const uint32_t bn = __ballot_sync(0xFFFFFFFFu, proc == 1 || proc == 2);

@@ -500,7 +500,7 @@ __device__ __forceinline__ unsigned int finish_state(const DeviceRefs& r, int in
   // ---- tallies: one thread per 8-byte slot of the record ---------------------
   if (t < kTallySlots)
     commit_tally_slot(P, t, sh.acc, sh.is.step, sh.is.n_steps_done, sh.st[0].n_live,
-                      sh.st[1].n_live, sh.is.w_live, &sh.is.ion_steps, total);
+                      sh.st[1].n_live, sh.is.w_live, &sh.is.ion_steps, 1.0 / P.c64.wscale, total);
   __syncthreads();
   if (t == 32) {
     sh.is.step += 1u;

@@ -150,30 +150,6 @@ __device__ __forceinline__ void load_tile(unsigned char* stage, const unsigned c
   bulk_load(stage, tile, bytes, bar);
 }
 
-// Kick and beta of a pass: in float on the branch-free path, in double slot
-// by slot.
-template <typename R>
-__device__ __forceinline__ void limited_kick_beta(R (&vx)[kPerHalf], const R (&vy)[kPerHalf],
-                                                  const R (&vz)[kPerHalf],
-                                                  const R (&a)[kPerHalf],
-                                                  const bool (&live)[kPerHalf], R vlim,
-                                                  R (&beta)[kPerHalf]) {
-  if constexpr (sizeof(R) == 4) {
-    kick_beta_mid<kPerHalf>(vx, vy, vz, a, live, vlim, beta);
-  } else {
-#pragma unroll
-    for (int j = 0; j < kPerHalf; ++j) {
-      R x1[1] = {vx[j]};
-      const R y1[1] = {vy[j]}, z1[1] = {vz[j]}, a1[1] = {a[j]};
-      limited_kick_n<R, 1>(x1, y1, z1, a1, vlim);
-      vx[j] = x1[0];
-    }
-#pragma unroll
-    for (int j = 0; j < kPerHalf; ++j)
-      beta[j] = beta_of(r_sqrt(vx[j] * vx[j] + vy[j] * vy[j] + vz[j] * vz[j]), vlim);
-  }
-}
-
 }  // namespace
 
 template <typename R>
@@ -327,7 +303,7 @@ __global__ void __launch_bounds__(kPushMaxWarps * 32, 1) k_push(DeviceRefs r) {
         // Eq. slpicEOMv across and above it) and drift (beta of the post-kick
         // speed); an unlimited species has beta = 1
         if (limited) {
-          limited_kick_beta<R>(vx, vy, vz, a, live, vlim, b1);
+          limited_kick_beta<R, kPerHalf>(vx, vy, vz, a, live, vlim, b1);
         } else {
 #pragma unroll
           for (int j = 0; j < kPerHalf; ++j) {

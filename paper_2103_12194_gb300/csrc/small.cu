@@ -39,6 +39,7 @@ constexpr int kSmallWarps = kSmallThreads / 32;
 constexpr int kSmallFillCap = 4 * kSmallMaxTiles;
 constexpr int kSmallCandRows = kSmallMaxTiles * kTile / kSmallThreads;
 static_assert(kSmallMaxTiles <= 32, "one lane per tile in the prefix scans");
+static_assert(ACC_COUNT <= 32 && kTallySlots <= 32, "the tallies by one warp");
 static_assert(kSmallCandRows * kSmallThreads == kSmallMaxTiles * kTile, "candidate rows");
 static_assert(kSmallCandRows <= 8, "16-bit row counters in one 128-bit scan value");
 
@@ -46,10 +47,10 @@ struct SmallShared {
   unsigned long long acc[ACC_COUNT];
   uint32_t fill[2][kSmallFillCap];
   uint32_t cnt[2][kSmallMaxTiles];  // per tile: candidates (electrons), emissions (ions)
-  uint32_t pre[2][kSmallFillCap];   // exclusive prefixes (counts; fills when repacking)
-  uint32_t tot[2];
+  uint32_t pre[kSmallFillCap];      // exclusive prefixes of the fills when repacking
+  uint32_t wpre[kSmallWarps][2][kSmallMaxTiles];  // of the counts, one copy per warp
   SpeciesState st[2];
-  uint32_t tail[2], end[2], n_new[2], nt[2], nb[2], compact[2];
+  uint32_t tail[2], end[2], n_new[2], nt[2], compact[2];
   uint32_t step;
   long long n_steps_done;
   unsigned long long w_live[2];
@@ -57,6 +58,7 @@ struct SmallShared {
   long long i64[32];
   __int128 i128[32];
   int stop;
+  int err;  // this CTA's device error
 };
 
 // Last tile j < n whose exclusive prefix pre[j] is at or below e (that tile
@@ -173,16 +175,26 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
   }
   const R* Eglob = node_field<R>(P);
 
+  // this thread's slot of the running totals
+  const double unit = 1.0 / P.c64.wscale;
+  long long total = t < kTallySlots ? reinterpret_cast<const long long*>(P.total)[t] : 0ll;
+  const bool single = gridDim.x == 1;
+  if (t == 0) sh.err = *((volatile int*)&ctrl->error);
+
   long long done = 0;
   for (;;) {
-    // ---- another step? all CTAs decide together ------------------------------
+    // ---- another step? a single CTA from what it holds, several together ----
     __syncthreads();
-    if (t == 0) {
+    if (single) {
+      if (done >= n_steps || (int)sh.st[0].n_tiles > max_tiles ||
+          (int)sh.st[1].n_tiles > max_tiles || sh.err)
+        break;
+    } else if (t == 0) {
       int stop = done >= n_steps ? 2 : 0;
       if (!stop && ((int)sh.st[0].n_tiles > max_tiles || (int)sh.st[1].n_tiles > max_tiles ||
                     *((volatile int*)&ctrl->error)))
         stop = 1;
-      if (stop != 2 && gridDim.x > 1) {
+      if (stop != 2) {
         // grid barrier b = done: arrive, then wait (bounded) for every CTA
         if (stop) atomicOr(&ctrl->small_stop, 1);
         __threadfence();
@@ -208,8 +220,10 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
       }
       sh.stop = stop;
     }
-    __syncthreads();
-    if (sh.stop) break;
+    if (!single) {
+      __syncthreads();
+      if (sh.stop) break;
+    }
     const uint32_t step = sh.step;
 
     // ---- 1. push: one warp per tile ---------------------------------------------
@@ -239,7 +253,8 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
           wj[j] = live[j] ? m.wj() : (R)0;
           id[j] = live[j] ? m.id() : 0u;
         }
-        const R qmdt = K.qmdt[sp], vlim = K.vlim[sp], dtdx = K.dtdx, P0 = K.P0;
+        const R qmdt = K.qmdt[sp], vlim = K.vlim[sp], dtdx = K.dtdx;
+        const uint32_t cand_thr = K.cand_thr;
         const uint32_t Nc = (uint32_t)N;
         const bool electrons = sp == kElectron;
         const bool limited = vlim < (R)INFINITY;
@@ -257,10 +272,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
           a[j] = qmdt * (E0 + off[j] * (E1 - E0));
         }
         if (limited) {
-          limited_kick_n<R, kPerLane>(vx, vy, vz, a, vlim);
-#pragma unroll
-          for (int j = 0; j < kPerLane; ++j)
-            b1[j] = beta_of(r_sqrt(vx[j] * vx[j] + vy[j] * vy[j] + vz[j] * vz[j]), vlim);
+          limited_kick_beta<R, kPerLane>(vx, vy, vz, a, live, vlim, b1);
         } else {
 #pragma unroll
           for (int j = 0; j < kPerLane; ++j) {
@@ -298,7 +310,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
 #pragma unroll
           for (int j = 0; j < kPerLane; ++j) {
             const uint2 rr = philox2x32_10(make_uint2(id[j], step), key2);
-            event[j] = alive[j] && uniform01r<R>(rr.x) < P0;
+            event[j] = alive[j] && (rr.x >> 9) < cand_thr;
           }
         }
         uint32_t b_alive[kPerLane], b_event[kPerLane];
@@ -352,11 +364,22 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
     __syncthreads();
 
     // ---- 2. collisions and births ---------------------------------------------
-    if (warp < 2) {
-      const uint32_t tot = warp_prefix(sh.cnt[warp], (int)sh.st[warp].n_tiles, sh.pre[warp]);
-      if (lane == 0) sh.tot[warp] = tot;
+    // (every warp forms the prefixes of the tiles' events for itself)
+    uint32_t tot[2];
+    for (int sp = 0; sp < 2; ++sp) {
+      const uint32_t v = lane < (int)sh.st[sp].n_tiles ? sh.cnt[sp][lane] : 0u;
+      uint32_t inc = v;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+        if (lane >= o) inc += y;
+      }
+      sh.wpre[warp][sp][lane] = inc - v;
+      tot[sp] = __shfl_sync(0xFFFFFFFFu, inc, 31);
     }
-    __syncthreads();
+    __syncwarp();
+    const uint32_t* const pre_e = sh.wpre[warp][0];
+    const uint32_t* const pre_i = sh.wpre[warp][1];
     const SpeciesState se = sh.st[0], si = sh.st[1];
     const Markers<R> me{E.buf[se.cur]};
     const Markers<R> mi{I.buf[si.cur]};
@@ -364,7 +387,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
     const uint32_t app_i = si.n_tiles ? (si.n_tiles - 1) * (uint32_t)kTile + sh.fill[1][si.n_tiles - 1] : 0u;
     const uint32_t cap_e = E.cap_tiles * (uint32_t)kTile, cap_i = I.cap_tiles * (uint32_t)kTile;
     {
-      const uint32_t C = sh.tot[0];
+      const uint32_t C = tot[0];
       const R kv = K.K_V[kElectron], vlim = K.vlim[kElectron];
       uint32_t slot[kSmallCandRows];
       R es[kSmallCandRows];
@@ -376,8 +399,8 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
         slot[u] = 0u;
         es[u] = (R)0;
         if (c >= C) continue;
-        const int j = tile_of_event(sh.pre[0], (int)se.n_tiles, c);
-        const uint32_t q = c - sh.pre[0][j];
+        const int j = tile_of_event(pre_e, (int)se.n_tiles, c);
+        const uint32_t q = c - pre_e[j];
         const size_t base = (size_t)j * kTile;
         const CandRec<R> cr = get_cand<R>(E.crec, base + q);
         const size_t o = base + cr.slot;
@@ -415,7 +438,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
       // so row u precedes row u + 1 and inside a row the threads are in order
       // (the scan is skipped in the many steps without an ionization)
       unsigned __int128 incl = 0, rows = 0;
-      if (__syncthreads_or(flags != 0)) {
+      if (C && __syncthreads_or(flags != 0)) {
         incl = (unsigned __int128)block_incl_scan<__int128, kSmallThreads>((__int128)flags,
                                                                            sh.i128);
         if (t == kSmallThreads - 1) sh.i128[0] = (__int128)incl;  // row totals
@@ -433,6 +456,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
           const uint32_t o = slot[u];
           if (pe >= cap_e || pi >= cap_i) {
             atomicCAS(&ctrl->error, 0, kErrCapacity);
+            sh.err = kErrCapacity;
           } else {
             const Slot<R> m = me[o];
             born_pair<R>(P, me[pe], mi[pi], m.cell(), m.off(), m.wj(), m.id(), step,
@@ -444,13 +468,14 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
       // electrons emitted at the cathode, after every ionization electron
       const uint32_t n_ionz = before;
       const R* sw = reinterpret_cast<const R*>(E.stage_w);
-      for (uint32_t e = t; e < sh.tot[1]; e += kSmallThreads) {
-        const int j = tile_of_event(sh.pre[1], (int)si.n_tiles, e);
-        const size_t o = (size_t)j * kTile + (e - sh.pre[1][j]);
+      for (uint32_t e = t; e < tot[1]; e += kSmallThreads) {
+        const int j = tile_of_event(pre_i, (int)si.n_tiles, e);
+        const size_t o = (size_t)j * kTile + (e - pre_i[j]);
         const uint32_t rank = n_ionz + e;
         const uint32_t pe = app_e + rank;
         if (pe >= cap_e) {
           atomicCAS(&ctrl->error, 0, kErrCapacity);
+          sh.err = kErrCapacity;
           continue;
         }
         write_marker(me[pe], 0, (R)0, (R)0, (R)0, (R)0, sw[o],
@@ -458,7 +483,8 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
       }
     }
     __syncthreads();
-    if (*((volatile int*)&ctrl->error)) break;  // the step is not committed
+    // (the step is not committed then)
+    if (single ? sh.err : *((volatile int*)&ctrl->error)) break;
 
     // ---- 3. counts, fills and where the stores end ---------------------------
     if (t < 2) {
@@ -477,10 +503,15 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
       sh.end[sp] = end;
       sh.n_new[sp] = n_new;
       sh.nt[sp] = nt;
-      sh.nb[sp] = nb;
       // repack when under three quarters of the slots in use are live
-      sh.compact[sp] =
-          (nt > 2 && (unsigned long long)n_new * 4 < (unsigned long long)nt * kTile * 3) ? 1u : 0u;
+      const bool compact =
+          nt > 2 && (unsigned long long)n_new * 4 < (unsigned long long)nt * kTile * 3;
+      sh.compact[sp] = compact ? 1u : 0u;
+      SpeciesState s1 = s0;
+      s1.n_live = n_new;
+      s1.next_id += nb;
+      if (!compact) s1.n_tiles = nt;  // (the rest after the repacking)
+      sh.st[sp] = s1;
     }
     __syncthreads();
     for (int sp = 0; sp < 2; ++sp) {
@@ -488,33 +519,32 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
       for (uint32_t k = sh.tail[sp] / kTile + t; k < sh.nt[sp]; k += kSmallThreads)
         sh.fill[sp][k] = min(sh.end[sp] - k * (uint32_t)kTile, (uint32_t)kTile);
     }
-    __syncthreads();
     // ---- repacking of a sparse store into its other buffer, in order --------
-    for (int sp = 0; sp < 2; ++sp) {
-      if (!sh.compact[sp]) continue;
-      if (warp == 0) warp_prefix(sh.fill[sp], (int)sh.nt[sp], sh.pre[sp]);
+    if (sh.compact[0] | sh.compact[1]) {
       __syncthreads();
-      const SpeciesDev& S = P.sp[sp];
-      const Markers<R> src{S.buf[sh.st[sp].cur]}, dst{S.buf[sh.st[sp].cur ^ 1u]};
-      for (uint32_t k = warp; k < sh.nt[sp]; k += kSmallWarps) {
-        const uint32_t n = sh.fill[sp][k];
-        const uint32_t to = sh.pre[sp][k];
-        for (uint32_t i = lane; i < n; i += 32) copy_marker(dst[to + i], src.at(k, i));
+      for (int sp = 0; sp < 2; ++sp) {
+        if (!sh.compact[sp]) continue;
+        if (warp == 0) warp_prefix(sh.fill[sp], (int)sh.nt[sp], sh.pre);
+        __syncthreads();
+        const SpeciesDev& S = P.sp[sp];
+        const Markers<R> src{S.buf[sh.st[sp].cur]}, dst{S.buf[sh.st[sp].cur ^ 1u]};
+        for (uint32_t k = warp; k < sh.nt[sp]; k += kSmallWarps) {
+          const uint32_t n = sh.fill[sp][k];
+          const uint32_t to = sh.pre[k];
+          for (uint32_t i = lane; i < n; i += 32) copy_marker(dst[to + i], src.at(k, i));
+        }
+        __syncthreads();
+        const uint32_t nt_new = (sh.n_new[sp] + kTile - 1) / kTile;
+        for (uint32_t k = t; k < nt_new; k += kSmallThreads)
+          sh.fill[sp][k] = min(sh.n_new[sp] - k * (uint32_t)kTile, (uint32_t)kTile);
+        __syncthreads();
       }
-      __syncthreads();
-      const uint32_t nt_new = (sh.n_new[sp] + kTile - 1) / kTile;
-      for (uint32_t k = t; k < nt_new; k += kSmallThreads)
-        sh.fill[sp][k] = min(sh.n_new[sp] - k * (uint32_t)kTile, (uint32_t)kTile);
-      __syncthreads();
+      if (t < 2 && sh.compact[t]) {
+        sh.st[t].cur ^= 1u;
+        sh.st[t].n_tiles = (sh.n_new[t] + kTile - 1) / kTile;
+      }
     }
-    if (t < 2) {
-      SpeciesState& s = sh.st[t];
-      if (sh.compact[t]) s.cur ^= 1u;
-      s.n_tiles = sh.compact[t] ? (sh.n_new[t] + kTile - 1) / kTile : sh.nt[t];
-      s.n_live = sh.n_new[t];
-      s.next_id += sh.nb[t];
-    }
-    __syncthreads();
+    if (poisson) __syncthreads();
 
     // ---- deposit and field (field mode 1) ------------------------------------
     if (poisson) {
@@ -552,16 +582,17 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
       for (int k = t; k < nn; k += kSmallThreads) s_rho0[k] = 0ull;
     }
 
-    // ---- tallies ---------------------------------------------------------------
-    if (t < kTallySlots)
-      commit_tally_slot(P, t, sh.acc, sh.step, sh.n_steps_done, sh.st[0].n_live,
-                        sh.st[1].n_live, sh.w_live, &sh.ion_steps,
-                        reinterpret_cast<const long long*>(P.total)[t]);
-    __syncthreads();
-    if (t < ACC_COUNT) sh.acc[t] = 0ull;
-    if (t == 0) {
-      sh.step += 1u;
-      sh.n_steps_done += 1;
+    // ---- tallies, by the first warp (the others wait at the next step) --------
+    if (warp == 0) {
+      if (t < kTallySlots)
+        total = commit_tally_slot(P, t, sh.acc, sh.step, sh.n_steps_done, sh.st[0].n_live,
+                                  sh.st[1].n_live, sh.w_live, &sh.ion_steps, unit, total);
+      __syncwarp();
+      if (t < ACC_COUNT) sh.acc[t] = 0ull;
+      if (t == 0) {
+        sh.step += 1u;
+        sh.n_steps_done += 1;
+      }
     }
     ++done;
   }

@@ -157,8 +157,10 @@ __device__ __forceinline__ int choose_process(const InstDev& P, R vlim, R v1, R 
   // the first process whose cumulative rate exceeds the draw: elastic,
   // excitation level 1..n_exc, ionization; none: a null collision
   const int n_proc = P.n_exc + 2;
-  int k = 0;
-  while (k < n_proc && !(rsel < c * xs[k])) ++k;
+  int k = n_proc;
+#pragma unroll
+  for (int i = kMaxProc - 1; i >= 0; --i)
+    if (i < n_proc && rsel < c * xs[i]) k = i;
   k_out = k;
   return k == n_proc ? 3 : (k == 0 ? 0 : (k <= P.n_exc ? 1 : 2));
 }
@@ -187,6 +189,73 @@ __device__ __forceinline__ Velocity<R> scatter_elastic(const StepConsts<R>& K, R
   rotate(ux, uy, uz, cc, sc, cp, sn);
   const R vn = r_sqrt(e_new * kv);
   return {vn * ux, vn * uy, vn * uz};
+}
+
+// The same out of line, from the velocity alone.
+template <typename R>
+__device__ __noinline__ Velocity<R> scatter_elastic_ieee(const StepConsts<R>& K, R kv, R vx, R vy,
+                                                         R vz, R eps, R u2, R u3) {
+  return scatter_elastic<R>(K, kv, vx, vy, vz, r_sqrt(vx * vx + vy * vy + vz * vz), eps, u2, u3);
+}
+
+// scatter_elastic for a warp's drain: in float the same operations with the
+// branch-free roots and quotients, one reciprocal for the quotients that share
+// a divisor (they are a third of the scattering's instructions).  Their
+// arguments stay in range while the speed is in [2^-10, 2^29], the energy in
+// [2^-30, 2^30] and every component is zero or above 2^-24 of the speed; other
+// lanes take the IEEE forms.
+__device__ __forceinline__ Velocity<double> scatter_elastic_any(const StepConsts<double>& K,
+                                                                double kv, double vx, double vy,
+                                                                double vz, double eps, double u2,
+                                                                double u3) {
+  return scatter_elastic<double>(K, kv, vx, vy, vz, r_sqrt(vx * vx + vy * vy + vz * vz), eps, u2,
+                                 u3);
+}
+__device__ __forceinline__ Velocity<float> scatter_elastic_any(const StepConsts<float>& K,
+                                                               float kv, float vx, float vy,
+                                                               float vz, float eps, float u2,
+                                                               float u3) {
+  const float v1 = sqrt_mid(vx * vx + vy * vy + vz * vz);
+  const float least = v1 * 5.9604644775390625e-08f;
+  auto fits = [&](float x) { return fabsf(x) >= least || x == 0.0f; };
+  if (!(v1 >= 0.0009765625f && v1 <= 536870912.0f && eps >= 9.313225746154785e-10f &&
+        eps <= 1073741824.0f && fits(vx) && fits(vy) && fits(vz)))
+    return scatter_elastic_ieee<float>(K, kv, vx, vy, vz, eps, u2, u3);
+  // a / b from the reciprocal y of b (div_mid)
+  auto over = [](float a, float b, float y) {
+    const float q = a * y;
+    return __fmaf_rn(__fmaf_rn(-b, q, a), y, q);
+  };
+  const float L = log1pf(eps);
+  const float em = expm1f(u2 * L);
+  const float ep = -expm1f(-(1.0f - u2) * L);
+  const float ye = rcp_mid(eps);
+  const float omc = fminf(2.0f, fmaxf(0.0f, over(em + em, eps, ye)));
+  const float opc = fminf(2.0f, fmaxf(0.0f, over((1.0f + eps) * (ep + ep), eps, ye)));
+  const float cc = omc <= 1.0f ? 1.0f - omc : opc - 1.0f;
+  const float sc = sqrt_mid0(omc * opc);
+  const float ph = K.two_pi * u3;
+  const float cp = cosf(ph), sp = sinf(ph);
+  const float e_new = eps * (1.0f - K.R2 * omc);
+  const float yv = rcp_mid(v1);
+  const float ux = over(vx, v1, yv), uy = over(vy, v1, yv), uz = over(vz, v1, yv);
+  // rotate()'s two frames, the x and z axes changing places
+  const bool z_frame = !(fabsf(ux) <= 0.99f);
+  const float a = z_frame ? uz : ux;
+  const float w = sqrt_mid((1.0f - a) * (1.0f + a));
+  const float yw = rcp_mid(w);
+  float nx, ny, nz;
+  if (!z_frame) {
+    nx = ux * cc + sc * (cp * w);
+    ny = uy * cc + sc * over(uz * sp - ux * (uy * cp), w, yw);
+    nz = uz * cc - sc * over(uy * sp + ux * (uz * cp), w, yw);
+  } else {
+    nx = ux * cc + sc * over(uy * sp - uz * (ux * cp), w, yw);
+    ny = uy * cc - sc * over(ux * sp + uz * (uy * cp), w, yw);
+    nz = uz * cc + sc * (cp * w);
+  }
+  const float vn = sqrt_mid(e_new * kv);
+  return {vn * nx, vn * ny, vn * nz};
 }
 
 // Excitation of level k: the threshold removed, an isotropic direction.
@@ -440,16 +509,14 @@ __device__ double poisson_d1(const InstDev& P, const long long* s_net, int k0, i
 // states (replaced in the totals), the others sums.  n_live_* are the counts
 // after the step; w_live (fixed point, per species) is updated by its changes,
 // and ion_steps gains the step's live ions.  total: the slot's bits in the
-// totals before the step.
+// totals before the step; the new ones are returned.  unit: 2^-charge_shift.
 constexpr int kTallySlots = (int)(sizeof(TallyRec) / 8);
 static_assert(kTallySlots == 26, "TallyRec layout");
 
-__device__ __forceinline__ void commit_tally_slot(const InstDev& P, int t,
-                                                  const unsigned long long* q, uint32_t step,
-                                                  long long n_steps_done, uint32_t n_live_e,
-                                                  uint32_t n_live_i, unsigned long long* w_live,
-                                                  long long* ion_steps, long long total) {
-  const double unit = 1.0 / P.c64.wscale;
+__device__ __forceinline__ long long commit_tally_slot(
+    const InstDev& P, int t, const unsigned long long* q, uint32_t step, long long n_steps_done,
+    uint32_t n_live_e, uint32_t n_live_i, unsigned long long* w_live, long long* ion_steps,
+    double unit, long long total) {
   long long iv = 0;
   double dv = 0.0;
   bool is_double = false;
@@ -495,12 +562,14 @@ __device__ __forceinline__ void commit_tally_slot(const InstDev& P, int t,
   long long* ring = reinterpret_cast<long long*>(P.ring + n_steps_done % P.ring_len);
   long long* tot = reinterpret_cast<long long*>(P.total);
   if (is_double) {
-    reinterpret_cast<double*>(ring)[t] = dv;
-    reinterpret_cast<double*>(tot)[t] = t <= 4 ? dv : __longlong_as_double(total) + dv;
+    iv = __double_as_longlong(dv);
+    total = t <= 4 ? iv : __double_as_longlong(__longlong_as_double(total) + dv);
   } else {
-    ring[t] = iv;
-    tot[t] = t <= 4 ? iv : total + iv;
+    total = t <= 4 ? iv : total + iv;
   }
+  ring[t] = iv;
+  tot[t] = total;
+  return total;
 }
 
 }  // namespace

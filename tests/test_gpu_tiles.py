@@ -97,13 +97,14 @@ def test_kicks_outside_the_branch_free_range(slpic, oracle_mod, vlim, kick):  # 
 
 def test_branch_free_operations_equal_the_ieee_ones(slpic, tmp_path):  # noqa: F811
     """sqrt_mid and rcp_mid on every float of their range, div_mid on 2^32
-    pairs (tests/rounding_check.cu)."""
+    pairs, the elastic scattering and beta on 2^28 draws
+    (tests/rounding_check.cu)."""
     from paper_2103_12194_gb300 import build
     exe = str(tmp_path / "rounding_check")
     subprocess.check_call([build.nvcc()] + build.common_flags() +
                           ["-I", build.CSRC, os.path.join(HERE, "rounding_check.cu"), "-o", exe])
     out = subprocess.run([exe], capture_output=True, text=True, timeout=120)
-    assert out.returncode == 0 and out.stdout.split()[:3] == ["0", "0", "0"], out.stdout
+    assert out.returncode == 0 and out.stdout.split()[:5] == ["0"] * 5, out.stdout
 
 
 @pytest.mark.parametrize("start", [0, 1, 3])
