@@ -618,6 +618,8 @@ int commit(slpic_ctx* c) {
       return cuda_fail(c, (cudaError_t)e2, "particle kernel configuration");
     if (gbps > 0 && gw > warps) max_warps = gw;
   }
+  if (int e2 = deposit_config(c->fp64))
+    return cuda_fail(c, (cudaError_t)e2, "deposit kernel configuration");
   if (int e2 = collide_config(c->fp64, max_nodes, &c->collide_resident, &c->refs.coll_nodes))
     return cuda_fail(c, (cudaError_t)e2, "collision kernel configuration");
   int sms = 0;
@@ -653,7 +655,8 @@ int materialize_deposit(slpic_ctx* c, int i) {
   const InstDev& P = c->h_inst[i];
   for (int s = 0; s < 2; ++s)
     CK(cudaMemsetAsync(P.rho_last[s], 0, (P.n_cells + 1) * 8, c->stream), "deposit");
-  launch_deposit(c->refs, i, (int)(c->hs[2 * i].n_tiles + c->hs[2 * i + 1].n_tiles), c->stream);
+  launch_deposit(c->refs, i, (int)(c->hs[2 * i].n_tiles + c->hs[2 * i + 1].n_tiles), P.n_cells + 1,
+                 c->sms, c->stream);
   CK(cudaGetLastError(), "deposit");
   c->dep_dirty[i] = 0;
   return SLPIC_OK;
@@ -1493,7 +1496,7 @@ int slpic_read_field(slpic_ctx* c, int inst, double* phi, double* E, int64_t n) 
   // the step keeps only the node field; phi is formed from the last deposit
   // (in the frozen-field mode it stays the vacuum solution)
   if (P.field_mode == 1 && c->stepped[inst]) {
-    launch_phi(c->refs, inst, c->stream);
+    launch_phi(c->refs, inst, P.n_cells, c->stream);
     CK(cudaGetLastError(), "read field");
   }
   int err = SLPIC_OK;
@@ -1990,7 +1993,7 @@ extern "C" int slpic_save(slpic_ctx* c, void* buf, size_t capacity, size_t* size
     // the deposit and phi as a read would form them
     if (int rc = materialize_deposit(c, i)) return rc;
     if (c->h_inst[i].field_mode == 1 && c->stepped[i]) {
-      launch_phi(c->refs, i, c->stream);
+      launch_phi(c->refs, i, c->h_inst[i].n_cells, c->stream);
       CK(cudaGetLastError(), "save");
     }
     for (int s = 0; s < 2; ++s)

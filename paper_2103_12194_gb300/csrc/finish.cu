@@ -51,6 +51,22 @@ __device__ __forceinline__ void plan_totals(const DeviceRefs& r, int n_seg, unsi
   r.ctrl->finish_done = 0;
 }
 
+// Sum over the lanes of a warp.
+__device__ __forceinline__ long long warp_sum(long long v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+  return v;
+}
+__device__ __forceinline__ __int128 warp_sum(__int128 v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long l = __shfl_xor_sync(0xFFFFFFFFu, (unsigned long long)v, o);
+    const long long h = __shfl_xor_sync(0xFFFFFFFFu, (long long)(v >> 64), o);
+    v += (__int128)(((unsigned __int128)(unsigned long long)h << 64) | l);
+  }
+  return v;
+}
+
 // Instance of block u of the nodes of all instances.
 __device__ __forceinline__ int field_inst(const DeviceRefs& r, int u) {
   int lo = 0, hi = r.n_inst - 1;  // last instance with field_start <= u
@@ -95,13 +111,8 @@ __device__ __forceinline__ void poisson_field(const InstDev& P, int block, Field
       if (b < block) S += P.pois_S[b];
       W += P.pois_W[b];
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      S += __shfl_xor_sync(0xFFFFFFFFu, S, o);
-      const unsigned long long wl = __shfl_xor_sync(0xFFFFFFFFu, (unsigned long long)W, o);
-      const long long wh = __shfl_xor_sync(0xFFFFFFFFu, (long long)(W >> 64), o);
-      W += (__int128)(((unsigned __int128)(unsigned long long)wh << 64) | wl);
-    }
+    S = warp_sum(S);
+    W = warp_sum(W);
     // one thread forms D_1 (FP64 is scarce on this part) and shares it
     if (lane == 0) {
       sh.S = S;
@@ -510,6 +521,17 @@ __device__ __forceinline__ unsigned int finish_state(const DeviceRefs& r, int in
   return room;
 }
 
+// A block's sums of the net charge and of it weighted, from its nodes' values.
+__device__ __forceinline__ void block_sums(const InstDev& P, int block, long long net, int weight,
+                                           long long* s_i64, __int128* s_i128) {
+  const long long S = block_incl_scan<long long>(net, s_i64);
+  const __int128 W = block_incl_scan<__int128>((__int128)net * weight, s_i128);
+  if (threadIdx.x == kFinThreads - 1) {
+    P.pois_S[block] = S;
+    P.pois_W[block] = W;
+  }
+}
+
 // One block of kFieldNodes nodes of an instance: the step's deposit becomes
 // the last step's, and the block leaves its sums of the net charge net_j
 // (0 < j < N) for the field: S = sum net_j and W = sum (N - j) net_j.
@@ -525,12 +547,7 @@ __device__ __forceinline__ void finish_nodes(const InstDev& P, int block, long l
     P.rho_acc[kIon][k] = 0ull;
     if (k > 0 && k < N) net = qi - qe;
   }
-  const long long S = block_incl_scan<long long>(net, s_i64);
-  const __int128 W = block_incl_scan<__int128>((__int128)net * (N - k), s_i128);
-  if (threadIdx.x == kFinThreads - 1) {
-    P.pois_S[block] = S;
-    P.pois_W[block] = W;
-  }
+  block_sums(P, block, net, N - k, s_i64, s_i128);
 }
 
 }  // namespace
@@ -598,74 +615,135 @@ __global__ void __launch_bounds__(kFinThreads) k_finish(DeviceRefs r, int mode, 
 // (zeroed by the caller): each marker adds fixed_charge(beta(|v|) w_j) at its
 // position, as the step deposits it.  A step's deposit is a function of the
 // markers after it, so with an imposed field it is formed here, when read,
-// instead of during every step.  One warp per tile, tiles of both species in
-// a grid-stride loop.
+// instead of during every step.  CTA b takes its share of the tiles of each
+// species, one warp per tile, into a copy of the grid in shared memory when
+// its markers outnumber the nodes (smem != 0): with every marker's two adds
+// going to the same few lines of global memory 8e6 markers on 4097 nodes took
+// 280 us, 55 with the copies.
+constexpr int kDepositThreads = 512;
 template <typename R>
-__global__ void __launch_bounds__(256) k_deposit(DeviceRefs r, int inst) {
+__global__ void __launch_bounds__(kDepositThreads) k_deposit(DeviceRefs r, int inst, int smem) {
+  extern __shared__ unsigned long long s_rho[];
   const InstDev& P = r.inst[inst];
   const StepConsts<R>& K = consts<R>(P);
-  const int lane = threadIdx.x & 31;
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int n_warps = (gridDim.x * blockDim.x) >> 5;
-  const SpeciesState se = r.sstate[inst * 2], si = r.sstate[inst * 2 + 1];
-  const uint32_t ne = se.n_tiles, n_items = se.n_tiles + si.n_tiles;
-  for (uint32_t it = warp; it < n_items; it += n_warps) {
-    const int sp = it < ne ? 0 : 1;
-    const uint32_t k = it < ne ? it : it - ne;
-    const SpeciesState& st = sp ? si : se;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nn = P.n_cells + 1;
+  for (int sp = 0; sp < 2; ++sp) {
+    const SpeciesState st = r.sstate[inst * 2 + sp];
+    const uint32_t k0 = (uint32_t)((unsigned long long)blockIdx.x * st.n_tiles / gridDim.x);
+    const uint32_t k1 = (uint32_t)((unsigned long long)(blockIdx.x + 1) * st.n_tiles / gridDim.x);
+    if (k0 == k1) continue;
     const Markers<R> mk{P.sp[sp].buf[st.cur]};
+    const uint32_t* const fill = P.sp[sp].fill[st.cur];
     const R vlim = K.vlim[sp];
     const bool limited = vlim < (R)INFINITY;
-    unsigned long long* rho = reinterpret_cast<unsigned long long*>(P.rho_last[sp]);
-    const uint32_t n = P.sp[sp].fill[st.cur][k];
-    for (uint32_t i = lane; i < n; i += 32) {
-      const Slot<R> m = mk.at(k, i);
-      const R vx = m.vx(), vy = m.vy(), vz = m.vz();
-      const R b = limited ? beta_of(r_sqrt(vx * vx + vy * vy + vz * vz), vlim) : (R)1;
-      deposit(rho, m.cell(), m.off(), fixed_charge(b * m.wj(), K.wscale));
+    unsigned long long* const g = reinterpret_cast<unsigned long long*>(P.rho_last[sp]);
+    unsigned long long* const rho = smem ? s_rho : g;
+    if (smem) {
+      for (int k = threadIdx.x; k < nn; k += kDepositThreads) s_rho[k] = 0ull;
+      __syncthreads();
+    }
+    for (uint32_t k = k0 + warp; k < k1; k += kDepositThreads / 32) {
+      const uint32_t n = fill[k];
+      for (uint32_t i = lane; i < n; i += 32) {
+        const Slot<R> m = mk.at(k, i);
+        R b = (R)1;
+        if (limited) {
+          const R vx = m.vx(), vy = m.vy(), vz = m.vz();
+          b = beta_any(vx * vx + vy * vy + vz * vz, vlim);
+        }
+        deposit(rho, m.cell(), m.off(), fixed_charge(b * m.wj(), K.wscale));
+      }
+    }
+    if (smem) {
+      __syncthreads();
+      for (int k = threadIdx.x; k < nn; k += kDepositThreads)
+        if (s_rho[k]) atomicAdd(g + k, s_rho[k]);
+      __syncthreads();
     }
   }
 }
 
-void launch_deposit(const DeviceRefs& r, int inst, int n_tiles, cudaStream_t s) {
-  const int grid = std::max(1, std::min((n_tiles + 7) / 8, 4096));
-  if (r.fp64) k_deposit<double><<<grid, 256, 0, s>>>(r, inst);
-  else k_deposit<float><<<grid, 256, 0, s>>>(r, inst);
+template <typename R>
+static void launch_deposit_t(const DeviceRefs& r, int inst, int n_tiles, int n_nodes, int sms,
+                             cudaStream_t s) {
+  const int most = sms * 2;
+  const int grid = std::max(1, std::min((n_tiles + 15) / 16, most));
+  // two CTAs per SM hold a copy each while it fits
+  const size_t bytes = (size_t)n_nodes * 8;
+  const bool smem = bytes <= kDepositSmem && (long long)n_tiles * kTile / grid >= n_nodes;
+  k_deposit<R><<<grid, kDepositThreads, smem ? bytes : 0, s>>>(r, inst, smem ? 1 : 0);
 }
 
-// phi_k = k D_1 - C J_k, J_k = sum_{0<i<=k} I_i, from the last step's deposit
-// (one CTA; read only when the field is read).
-__global__ void __launch_bounds__(kFinThreads) k_phi(DeviceRefs r, int inst) {
+void launch_deposit(const DeviceRefs& r, int inst, int n_tiles, int n_nodes, int sms,
+                    cudaStream_t s) {
+  if (r.fp64) launch_deposit_t<double>(r, inst, n_tiles, n_nodes, sms, s);
+  else launch_deposit_t<float>(r, inst, n_tiles, n_nodes, sms, s);
+}
+
+int deposit_config(int fp64) {
+  return (int)(fp64 ? cudaFuncSetAttribute(k_deposit<double>,
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)kDepositSmem)
+                    : cudaFuncSetAttribute(k_deposit<float>,
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)kDepositSmem));
+}
+
+// The potential of instance inst from its last deposit (read only when the
+// field is read), block by block like the field: the blocks' sums first, then
+// phi_k = k D_1 - C J_k, J_k = sum_{0<i<=k} I_i, with J at a block's first node
+// k_b = sum (k_b - j) net_j = sum over the blocks before of W - (N - k_b) S.
+// (By one CTA over the whole grid 4096 cells took 14 us and 21832 69.)
+__global__ void __launch_bounds__(kFinThreads) k_phi_sums(DeviceRefs r, int inst) {
   __shared__ long long s_i64[32];
   __shared__ __int128 s_i128[32];
   const InstDev& P = r.inst[inst];
-  const int N = P.n_cells;
-  const int chunk = (N + kFinThreads - 1) / kFinThreads;
-  const int k0 = 1 + threadIdx.x * chunk;
-  long long Ik;
-  const double D1 = poisson_d1(P, nullptr, k0, chunk, s_i64, s_i128, &Ik);
-  const double C = P.pois_C;
-  // J at the chunk start: exclusive scan of the chunks' sums of I
-  __int128 locJ = 0;
-  {
-    long long I = Ik;
-    for (int k = k0; k < k0 + chunk && k <= N; ++k) {
-      locJ += (__int128)I;
-      if (k <= N - 1) I += P.rho_last[kIon][k] - P.rho_last[kElectron][k];
-    }
-  }
-  const __int128 incJ = block_incl_scan<__int128>(locJ, s_i128);
-  __int128 J = incJ - locJ;
-  for (int k = k0; k < k0 + chunk && k <= N; ++k) {
-    J += (__int128)Ik;
-    if (k <= N - 1) Ik += P.rho_last[kIon][k] - P.rho_last[kElectron][k];
-    P.phi[k] = k == N ? P.V : (double)k * D1 - C * (double)J;
-  }
-  if (threadIdx.x == 0) P.phi[0] = 0.0;
+  const int k = blockIdx.x * kFieldNodes + (int)threadIdx.x, N = P.n_cells;
+  const long long net = k > 0 && k < N ? P.rho_last[kIon][k] - P.rho_last[kElectron][k] : 0ll;
+  block_sums(P, blockIdx.x, net, N - k, s_i64, s_i128);
 }
 
-void launch_phi(const DeviceRefs& r, int inst, cudaStream_t s) {
-  k_phi<<<1, kFinThreads, 0, s>>>(r, inst);
+__global__ void __launch_bounds__(kFinThreads) k_phi(DeviceRefs r, int inst) {
+  __shared__ long long s_i64[32];
+  __shared__ __int128 s_i128[32];
+  __shared__ __int128 s_J;
+  __shared__ long long s_S;
+  __shared__ double s_D1;
+  const InstDev& P = r.inst[inst];
+  const int kb = blockIdx.x * kFieldNodes, k = kb + (int)threadIdx.x, N = P.n_cells;
+  const long long net = k > 0 && k < N ? P.rho_last[kIon][k] - P.rho_last[kElectron][k] : 0ll;
+  if (threadIdx.x < 32) {
+    const int nb = N / kFieldNodes + 1;
+    long long S = 0;
+    __int128 W = 0, J = 0;
+    for (int b = threadIdx.x; b < nb; b += 32) {
+      if (b < (int)blockIdx.x) {
+        S += P.pois_S[b];
+        J += P.pois_W[b] - (__int128)P.pois_S[b] * (N - kb);
+      }
+      W += P.pois_W[b];
+    }
+    S = warp_sum(S);
+    J = warp_sum(J);
+    W = warp_sum(W);
+    if (threadIdx.x == 0) {
+      s_S = S;
+      s_J = J;
+      s_D1 = (P.V + P.pois_C * (double)W) / (double)N;
+    }
+  }
+  const long long inc = block_incl_scan<long long>(net, s_i64);  // (ends with a barrier)
+  const long long I = s_S + inc - net;                           // I_k
+  // J_k = J_kb + sum_{kb<i<=k} I_i
+  const __int128 J = s_J + block_incl_scan<__int128>(threadIdx.x ? (__int128)I : (__int128)0, s_i128);
+  if (k > N) return;
+  P.phi[k] = k == 0 ? 0.0 : k == N ? P.V : (double)k * s_D1 - P.pois_C * (double)J;
+}
+
+void launch_phi(const DeviceRefs& r, int inst, int n_cells, cudaStream_t s) {
+  const int blocks = n_cells / kFieldNodes + 1;
+  k_phi_sums<<<blocks, kFinThreads, 0, s>>>(r, inst);
+  k_phi<<<blocks, kFinThreads, 0, s>>>(r, inst);
 }
 
 __global__ void __launch_bounds__(256) k_vacuum(double* phi, double* E64, float* E32, int N,
@@ -890,15 +968,18 @@ void launch_seed(const DeviceRefs& r, int inst, int species, uint32_t base, uint
 // Copy a caller's markers into a tiled store and check them (cell in [0, N),
 // offset in [0, 1), finite velocities, non-negative weight below 2^39 charge
 // units); records the smallest bad index in *bad and the fixed-point sum of
-// the weights in *wsum.  One pass: each marker is read and written once.
+// the weights in *wsum.  One pass: each marker is read and written once, and a
+// CTA adds its weights once (an add per warp to the one sum took 4e6 markers
+// from 40 to 97 us).
 template <typename R>
 __global__ void __launch_bounds__(256) k_place(SoAT<R> src, Markers<R> dst, uint32_t n, int N,
                                                int shift, unsigned int* bad,
                                                unsigned long long* wsum) {
   const R wscale = (R)ldexp(1.0, shift);  // 2^shift, exact
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  __shared__ unsigned long long s_w[8];
   unsigned long long w = 0;
-  if (i < n) {
+  const uint32_t stride = gridDim.x * blockDim.x;
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
     const R o = src.f[0][i], x = src.f[1][i], y = src.f[2][i], z = src.f[3][i], wj = src.f[4][i];
     const int c = src.cell[i];
     // the fixed-point weight must stay below 2^39 units so that the 24-bit
@@ -906,11 +987,16 @@ __global__ void __launch_bounds__(256) k_place(SoAT<R> src, Markers<R> dst, uint
     const bool ok = c >= 0 && c < N && o >= (R)0 && o < (R)1 && isfinite(x) && isfinite(y) &&
                     isfinite(z) && wj >= (R)0 && wj * wscale < (R)549755813888.0;
     if (!ok) atomicMin(bad, i);
-    else w = (unsigned long long)fixed_charge(wj, wscale);
+    else w += (unsigned long long)fixed_charge(wj, wscale);
     write_marker(dst[i], c, o, x, y, z, wj, src.id[i]);
   }
   for (int o = 16; o > 0; o >>= 1) w += __shfl_down_sync(0xFFFFFFFFu, w, o);
-  if ((threadIdx.x & 31) == 0 && w) atomicAdd(wsum, w);
+  if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = w;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int k = 1; k < 8; ++k) w += s_w[k];
+    if (w) atomicAdd(wsum, w);
+  }
 }
 
 template <typename R>
@@ -920,7 +1006,7 @@ static void place(const void* const src[7], unsigned char* buf, uint32_t n, int 
   a.cell = static_cast<const int32_t*>(src[0]);
   for (int k = 0; k < 5; ++k) a.f[k] = static_cast<const R*>(src[1 + k]);
   a.id = static_cast<const uint32_t*>(src[6]);
-  k_place<R><<<(n + 255) / 256, 256, 0, s>>>(a, Markers<R>{buf}, n, N, shift, bad, wsum);
+  k_place<R><<<std::min((n + 255) / 256, 4096u), 256, 0, s>>>(a, Markers<R>{buf}, n, N, shift, bad, wsum);
 }
 
 void launch_place(int fp64, const void* const src[7], unsigned char* buf, uint32_t n, int N,

@@ -384,7 +384,7 @@ int push_blocks_per_sm(int fp64, int warps, int smem_nodes, int* blocks_per_sm);
 void launch_finish(const DeviceRefs& r, int mode, cudaStream_t s);
 void launch_move(const DeviceRefs& r, int grid, cudaStream_t s);
 // Node potential of instance inst from its last deposit (Poisson mode).
-void launch_phi(const DeviceRefs& r, int inst, cudaStream_t s);
+void launch_phi(const DeviceRefs& r, int inst, int n_cells, cudaStream_t s);
 // The vacuum field of an instance: phi = V k / N, E on every node.
 void launch_vacuum(const InstDev& P, double E, float E32, cudaStream_t s);
 // Fills of tiles [first, ceil(end / kTile)) of a store whose slots from
@@ -395,8 +395,11 @@ void launch_prefix(const uint32_t* fill, uint32_t n_tiles, uint32_t* prefix, uin
                    cudaStream_t s);
 // Deposit of instance inst's live markers (n_tiles tiles of both species)
 // added to its last-step grids; used with an imposed field, where the step
-// itself deposits nothing.
-void launch_deposit(const DeviceRefs& r, int inst, int n_tiles, cudaStream_t s);
+// itself deposits nothing.  kDepositSmem: shared memory of a CTA's charge grid.
+constexpr size_t kDepositSmem = 100 * 1024;
+void launch_deposit(const DeviceRefs& r, int inst, int n_tiles, int n_nodes, int sms,
+                    cudaStream_t s);
+int deposit_config(int fp64);
 // Scatter the null-collision candidates queued by the particle kernel.
 void launch_collide(const DeviceRefs& r, int grid, cudaStream_t s);
 // Its resident CTAs per SM and the nodes of its shared charge grid (0: deposits
