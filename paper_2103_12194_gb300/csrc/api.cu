@@ -107,6 +107,8 @@ struct slpic_ctx {
   // was formed (the step deposits nothing then; the deposit is formed from
   // the markers when read, or before they change)
   std::vector<char> dep_dirty;
+  // the step it was formed after (steps a caller replays are seen by it)
+  std::vector<uint32_t> dep_step;
   int blocks_per_sm = 0;
   // Small transfers go through pinned memory, in the stream's order: `pin` is
   // handed out from its start until the stream has been waited for (drain),
@@ -119,6 +121,9 @@ struct slpic_ctx {
   char* pin = nullptr;
   size_t pin_size = 0, pin_used = 0;
   std::vector<Read> reads;
+  // Recorded after the last upload; `loose` while that may not have arrived.
+  cudaEvent_t loose_ev = nullptr;
+  bool loose = false;
   // The instances' and stores' state as the host knows it; `known` while no
   // step has run since it was read (a step captured into a caller's graph runs
   // unseen: such a context always reads it again).
@@ -154,6 +159,7 @@ int fail(slpic_ctx* c, int code, const char* fmt, ...) {
 }
 
 int cuda_fail(slpic_ctx* c, cudaError_t e, const char* what) {
+  cudaGetLastError();  // reported here, not by the next call
   return fail(c, SLPIC_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
@@ -170,13 +176,46 @@ int set_device(slpic_ctx* c) {
   return SLPIC_OK;
 }
 
-// Wait for the stream and deliver the reads queued on it.
+bool capturing(const slpic_ctx* c) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  return c->stream && cudaStreamIsCapturing(c->stream, &st) == cudaSuccess &&
+         st != cudaStreamCaptureStatusNone;
+}
+
+// Wait for the stream and deliver the reads queued on it (fails while the
+// stream is being captured; the reads are then dropped).
 int drain(slpic_ctx* c) {
-  CK(cudaStreamSynchronize(c->stream), "stream synchronize");
-  for (const auto& r : c->reads) std::memcpy(r.to, r.from, r.bytes);
+  const cudaError_t e = cudaStreamSynchronize(c->stream);
+  if (e == cudaSuccess) {
+    for (const auto& r : c->reads) std::memcpy(r.to, r.from, r.bytes);
+    c->pin_used = 0;
+    c->loose = false;
+  }
   c->reads.clear();
-  c->pin_used = 0;
+  if (e == cudaSuccess) return SLPIC_OK;
+  return cuda_fail(c, e, "stream synchronize");
+}
+
+// Wait for the uploads alone: not by the stream, which may be the caller's to
+// destroy or in capture by now.
+int settle(slpic_ctx* c) {
+  if (!c->loose) return SLPIC_OK;
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  CK(cudaThreadExchangeStreamCaptureMode(&mode), "uploads");
+  const cudaError_t e = cudaEventSynchronize(c->loose_ev);
+  CK(cudaThreadExchangeStreamCaptureMode(&mode), "uploads");
+  if (e != cudaSuccess) return cuda_fail(c, e, "uploads");
+  c->loose = false;
   return SLPIC_OK;
+}
+
+// Note that the stream holds uploads the host has not waited for.  Steps that
+// a caller captured may run on any stream: they find every upload arrived.
+int uploaded(slpic_ctx* c) {
+  if (!c->loose_ev) CK(cudaEventCreateWithFlags(&c->loose_ev, cudaEventDisableTiming), "event");
+  CK(cudaEventRecord(c->loose_ev, c->stream), "event");
+  c->loose = true;
+  return c->uncached ? settle(c) : SLPIC_OK;
 }
 
 // Room for `bytes` bytes of pinned memory until the next drain.
@@ -202,15 +241,19 @@ int pin_room(slpic_ctx* c, size_t bytes, char** p) {
 // arrives with the next drain).
 int put(slpic_ctx* c, void* dev, const void* host, size_t bytes) {
   char* p;
+  if (capturing(c)) return drain(c);
   if (int rc = pin_room(c, bytes, &p)) return rc;
   std::memcpy(p, host, bytes);
   CK(cudaMemcpyAsync(dev, p, bytes, cudaMemcpyHostToDevice, c->stream), "copy to the device");
-  return SLPIC_OK;
+  return uploaded(c);
 }
 int get(slpic_ctx* c, void* host, const void* dev, size_t bytes) {
   char* p;
   if (int rc = pin_room(c, bytes, &p)) return rc;
-  CK(cudaMemcpyAsync(p, dev, bytes, cudaMemcpyDeviceToHost, c->stream), "copy from the device");
+  if (cudaError_t e = cudaMemcpyAsync(p, dev, bytes, cudaMemcpyDeviceToHost, c->stream)) {
+    c->reads.clear();  // their call ends here
+    return cuda_fail(c, e, "copy from the device");
+  }
   c->reads.push_back({host, p, bytes});
   return SLPIC_OK;
 }
@@ -255,6 +298,7 @@ int sync(slpic_ctx* c) {
     CK(cudaStreamSynchronize(c->stream), "stream synchronize");
     return SLPIC_OK;
   }
+  if (capturing(c)) return drain(c);
   if (c->known) return SLPIC_OK;
   if (int rc = ask_state(c)) return rc;
   if (int rc = drain(c)) return rc;
@@ -264,6 +308,7 @@ int sync(slpic_ctx* c) {
 // Read `bytes` bytes after everything queued, with the state if it is not
 // known: *err is the latched error, the return value a failure of the read.
 int read_with_state(slpic_ctx* c, void* host, const void* dev, size_t bytes, int* err) {
+  if (capturing(c)) return drain(c);
   const bool ask = !c->known;
   if (ask)
     if (int rc = ask_state(c)) return rc;
@@ -388,7 +433,7 @@ int reset_field(slpic_ctx* c, int i) {
   launch_vacuum(P, -P.V / P.d, (float)(-P.V / P.d), c->stream);
   CK(cudaGetLastError(), "field");
   if ((int)c->stepped.size() == c->n_inst) c->stepped[i] = 0;
-  return SLPIC_OK;
+  return uploaded(c);
 }
 
 int upload_inst(slpic_ctx* c, int i) { return put(c, c->d_inst + i, &c->h_inst[i], sizeof(InstDev)); }
@@ -421,7 +466,8 @@ int zero_counters(slpic_ctx* c, int i) {
   is.n_steps_done = 0;
   is.w_seed = 0;
   is.ion_steps = 0;
-  if ((int)c->dep_dirty.size() == c->n_inst) c->dep_dirty[i] = 0;
+  c->dep_dirty[i] = 0;
+  c->dep_step[i] = 0;
   return write_inst_state(c, i);
 }
 
@@ -651,7 +697,8 @@ int commit(slpic_ctx* c) {
 // stepped since the deposit was last formed.  Called before the deposit is
 // read and before the markers change, with the state known.
 int materialize_deposit(slpic_ctx* c, int i) {
-  if (c->h_inst[i].field_mode == 1 || !c->dep_dirty[i]) return SLPIC_OK;
+  const bool replayed = c->uncached && c->his[i].step != c->dep_step[i];
+  if (c->h_inst[i].field_mode == 1 || !(c->dep_dirty[i] || replayed)) return SLPIC_OK;
   const InstDev& P = c->h_inst[i];
   for (int s = 0; s < 2; ++s)
     CK(cudaMemsetAsync(P.rho_last[s], 0, (P.n_cells + 1) * 8, c->stream), "deposit");
@@ -659,6 +706,7 @@ int materialize_deposit(slpic_ctx* c, int i) {
                  c->sms, c->stream);
   CK(cudaGetLastError(), "deposit");
   c->dep_dirty[i] = 0;
+  c->dep_step[i] = c->his[i].step;
   return SLPIC_OK;
 }
 
@@ -668,18 +716,15 @@ void mark_stepped(slpic_ctx* c) {
     if (c->h_inst[i].field_mode != 1) c->dep_dirty[i] = 1;
 }
 
-bool capturing(const slpic_ctx* c) {
-  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  return c->stream && cudaStreamIsCapturing(c->stream, &st) == cudaSuccess &&
-         st != cudaStreamCaptureStatusNone;
-}
-
 // Before steps are launched: the plan of the next one, if the stores have
 // changed since it was made (captured into a caller's graph, it is made by the
 // graph, and again by the next call), and the state no longer known.
 int begin_steps(slpic_ctx* c) {
   const bool cap = capturing(c);
-  if (cap) c->uncached = true;
+  if (cap) {
+    c->uncached = true;
+    if (int rc = settle(c)) return rc;
+  }
   c->known = false;
   if (!c->plan_due) return SLPIC_OK;
   launch_finish(c->refs, 1, c->stream);
@@ -775,8 +820,9 @@ int build_graph(slpic_ctx* c) {
   return SLPIC_OK;
 }
 
-// Launch shape of the step: warps per particle-kernel CTA (the super-tile
-// size, so the next step is replanned) and collision CTAs per SM.  Results do
+// Launch shape of the step: warps per particle-kernel CTA (the plan's shares
+// depend on the grid, so the next step is replanned) and collision CTAs per
+// SM, no more than are resident at once.  Results do
 // not depend on it: tiles are independent, deposits are integer sums and
 // births are ordered by (tile, slot).
 int apply_shape(slpic_ctx* c, int warps, int coll_per_sm) {
@@ -880,6 +926,7 @@ int slpic_create(slpic_ctx** out, int device, int n_instances) {
   c->hi.resize(n_instances);
   c->stepped.assign(n_instances, 0);
   c->dep_dirty.assign(n_instances, 0);
+  c->dep_step.assign(n_instances, 0);
   *out = c;
   return SLPIC_OK;
 }
@@ -892,6 +939,7 @@ int slpic_destroy(slpic_ctx* c) {
   for (auto& e : c->ev) cudaEventDestroy(e);
   for (void* p : c->allocs) cudaFree(p);
   if (c->pin) cudaFreeHost(c->pin);
+  if (c->loose_ev) cudaEventDestroy(c->loose_ev);
   if (c->capture_stream) cudaStreamDestroy(c->capture_stream);
   delete c;
   return SLPIC_OK;
@@ -899,10 +947,11 @@ int slpic_destroy(slpic_ctx* c) {
 
 int slpic_set_stream(slpic_ctx* c, void* stream) {
   if (!c) return SLPIC_ERR_INVALID_ARG;
+  // uploads queued on the old stream come before all that follows
   if (c->committed && c->stream != (cudaStream_t)stream) {
-    // what is queued on the old stream comes before all that follows
     if (int rc = set_device(c)) return rc;
-    if (int rc = drain(c)) return rc;
+    if (int rc = settle(c)) return rc;
+    c->pin_used = 0;
   }
   c->stream = (cudaStream_t)stream;
   return SLPIC_OK;
@@ -1458,7 +1507,7 @@ int slpic_read_charge(slpic_ctx* c, int inst, int species, int64_t* host, int64_
   if (int rc = prepare(c)) return rc;
   const InstDev& P = c->h_inst[inst];
   int rc = SLPIC_OK;
-  const bool form = P.field_mode != 1 && c->dep_dirty[inst];
+  const bool form = P.field_mode != 1 && (c->dep_dirty[inst] || c->uncached);
   if (form || n != P.n_cells + 1) rc = sync(c);
   if (n != P.n_cells + 1) return fail(c, SLPIC_ERR_INVALID_ARG, "need n_cells + 1 values");
   if (form)
@@ -2129,6 +2178,7 @@ extern "C" int slpic_load(slpic_ctx* c, const void* buf, size_t size) {
       CK(cudaMemcpy(P.rho_last[s], rho[s], nn * 8, cudaMemcpyHostToDevice), "load");
     c->stepped[i] = (char)r.stepped;
     c->dep_dirty[i] = 0;
+    c->dep_step[i] = r.is.step;
   }
   c->plan_due = true;
   return SLPIC_OK;

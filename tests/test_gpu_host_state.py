@@ -1,6 +1,8 @@
 """What the host knows of a context's state: it must not go stale when steps
 run in a graph that the caller captured, when markers are appended with and
 without steps in between, or when the stream changes."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -81,3 +83,66 @@ def test_appending_with_and_without_steps(slpic, field_mode):  # noqa: F811
     same(one, two)
     one.close()
     two.close()
+
+
+@pytest.mark.parametrize("call", ["set_voltage", "seed", "count", "tallies", "field", "charge",
+                                  "reset_counters", "history"])
+def test_refused_while_captured(slpic, call):  # noqa: F811
+    """Calls that answer on the host, or change what the host holds, are
+    refused while their stream is captured, also when the state is known; the
+    context is as before after it."""
+    import torch
+    cuda = ctypes.CDLL("libcuda.so.1")
+    stream = torch.cuda.Stream()
+    sim, plain = make(slpic, 1, stream), make(slpic, 1)
+    for s in (sim, plain):
+        s.step(3)
+        s.count(0, 0)  # the state is known from here
+    args = {"set_voltage": (0, 300.0), "seed": (0, 0, 5, slpic.SEED_REST),
+            "count": (0, 0), "charge": (0, 0)}
+    graph, handle = ctypes.c_void_p(), ctypes.c_void_p(stream.cuda_stream)
+    assert cuda.cuStreamBeginCapture_v2(handle, 1) == 0  # this thread's calls alone
+    try:
+        with pytest.raises(slpic.SlpicError):
+            getattr(sim, call)(*args.get(call, (0,)))
+    finally:
+        assert cuda.cuStreamEndCapture(handle, ctypes.byref(graph)) != 0  # invalidated
+    for s in (sim, plain):
+        s.set_voltage(0, 300.0)
+        s.step(2)
+    same(sim, plain)
+    sim.close()
+    plain.close()
+
+
+def test_uploads_arrive_before_steps_on_other_streams(slpic):  # noqa: F811
+    """Steps captured on the context's stream and replayed on another one find
+    what the calls before them have set, those before the capture too; a stream
+    that is destroyed may be replaced."""
+    import torch
+    cuda = ctypes.CDLL("libcuda.so.1")
+    own = ctypes.c_void_p()
+    sim, plain = make(slpic, 0), make(slpic, 0)
+    sim.synchronize()
+    assert cuda.cuStreamCreate(ctypes.byref(own), 1) == 0
+    sim.set_stream(own.value)
+    for s in (sim, plain):
+        s.set_voltage(0, 280.0)
+    assert cuda.cuStreamSynchronize(own) == 0 and cuda.cuStreamDestroy_v2(own) == 0
+    stream, other = torch.cuda.Stream(), torch.cuda.Stream()
+    sim.set_stream(stream)
+    graph = torch.cuda.CUDAGraph()
+    for s in (sim, plain):
+        s.seed(0, 0, 300, slpic.SEED_REST)
+    with torch.cuda.graph(graph, stream=stream, capture_error_mode="thread_local"):
+        sim.step(1)
+    with torch.cuda.stream(other):
+        for V in (250.0, 350.0, 150.0):
+            sim.set_voltage(0, V)
+            graph.replay()
+            other.synchronize()
+            plain.set_voltage(0, V)
+            plain.step(1)
+            same(sim, plain)
+    sim.close()
+    plain.close()
