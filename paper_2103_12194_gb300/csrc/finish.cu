@@ -161,8 +161,8 @@ __device__ __forceinline__ unsigned int item_tiles(unsigned long long room, uint
 // weights over its CTAs: a barrier, a flush of the charge grid and an empty
 // pipeline, about as long as 16 electron tiles of a CTA.  (A CTA whose range
 // held ten small gaps took far longer than the others: k_push on 32 uneven gaps
-// 242 us, 201 with this; 24 or 96 instead of 48 run the same.)  No more than a CTA's share, which populations
-// of few tiles are spread over.
+// 242 us, 201 with this; 24 or 96 instead of 48 run the same.)  No more than a
+// CTA's share, which populations of few tiles are spread over.
 __device__ __forceinline__ long long seg_cost(const DeviceRefs& r, long long total) {
   return min((long long)kSegCost, total / r.push_grid);
 }
@@ -241,8 +241,8 @@ __device__ void plan_next_warp(const DeviceRefs& r) {
 }
 
 // Plan the next step from the tiles in use (all threads of one CTA):
-// particle-kernel tiles and their weights per segment, repacking chunks per segment and collision items per instance,
-// as exclusive block scans in rounds of kFinThreads entries.
+// particle-kernel tiles and their weights and repacking chunks per segment and
+// collision items per instance, as exclusive block scans in rounds of kFinThreads entries.
 __device__ void plan_next(const DeviceRefs& r, long long* s_buf) {
   __shared__ long long s_carry[5];
   const int n_seg = r.n_inst * 2;
@@ -557,7 +557,8 @@ __device__ __forceinline__ void finish_nodes(const InstDev& P, int block, long l
 // nodes of all instances in turn; the last kBirthCtas place the births.  No CTA
 // waits for another, and the longest chain is that of an instance's state: 12
 // us a step at 256 cells with the whole deposit and the Poisson sums in that
-// CTA, 16 at 4096 and 39 at 21832.  mode 1: plan only (one CTA).
+// CTA, 16 at 4096 and 39 at 21832; 8, 10 and 11 spread like this, births
+// included.  mode 1: plan only (one CTA).
 __global__ void __launch_bounds__(kFinThreads) k_finish(DeviceRefs r, int mode, int n_field) {
   __shared__ long long s_i64[32];
   __shared__ __int128 s_i128[32];
@@ -619,7 +620,7 @@ __global__ void __launch_bounds__(kFinThreads) k_finish(DeviceRefs r, int mode, 
 // species, one warp per tile, into a copy of the grid in shared memory when
 // its markers outnumber the nodes (smem != 0): with every marker's two adds
 // going to the same few lines of global memory 8e6 markers on 4097 nodes took
-// 280 us, 55 with the copies.
+// 280 us, 87 with the copies.
 constexpr int kDepositThreads = 512;
 template <typename R>
 __global__ void __launch_bounds__(kDepositThreads) k_deposit(DeviceRefs r, int inst, int smem) {
