@@ -442,13 +442,25 @@ int write_inst_state(slpic_ctx* c, int i) {
   return put(c, c->d_istate + i, &c->his[i], sizeof(InstState));
 }
 
+// The plan of the next step no longer holds: it is made anew before that step
+// runs, by begin_steps, or at once where steps that a caller captured may run
+// next (their graph holds a plan only if one was due at the capture).
+int replan(slpic_ctx* c) {
+  c->plan_due = true;
+  if (!c->uncached) return SLPIC_OK;
+  launch_finish(c->refs, 1, c->stream);
+  CK(cudaGetLastError(), "plan");
+  c->plan_due = false;
+  return uploaded(c);
+}
+
 // Set the state of a store to what the host now holds; `tail` is its first
-// free slot.  The next step is planned anew before it runs.
+// free slot.
 int write_state(slpic_ctx* c, int inst, int sp, const SpeciesState& st, int64_t tail) {
   c->hs[2 * inst + sp] = st;
   c->tail[2 * inst + sp] = tail;
-  c->plan_due = true;
-  return put(c, c->d_sstate + inst * 2 + sp, &st, sizeof st);
+  if (int rc = put(c, c->d_sstate + inst * 2 + sp, &st, sizeof st)) return rc;
+  return replan(c);
 }
 
 // (the state is known)
@@ -846,8 +858,7 @@ int apply_shape(slpic_ctx* c, int warps, int coll_per_sm) {
   c->push_grid = c->refs.push_grid = c->sms * bps;
   c->collide_per_sm = coll_per_sm;
   c->collide_grid = c->sms * std::min(coll_per_sm, c->collide_resident);
-  c->plan_due = true;
-  return SLPIC_OK;
+  return replan(c);
 }
 
 // The seven marker arrays of a caller (cell, off, vx, vy, vz, w_j, id), in
@@ -1427,7 +1438,7 @@ int slpic_clear_error(slpic_ctx* c) {
       CK(cudaMemsetAsync(P.rho_acc[s], 0, (P.n_cells + 1) * 8, c->stream), "clear");
   }
   c->known = false;
-  c->plan_due = true;
+  if (int rc = replan(c)) return rc;
   return drain(c);
 }
 
@@ -2180,8 +2191,7 @@ extern "C" int slpic_load(slpic_ctx* c, const void* buf, size_t size) {
     c->dep_dirty[i] = 0;
     c->dep_step[i] = r.is.step;
   }
-  c->plan_due = true;
-  return SLPIC_OK;
+  return SLPIC_OK;  // (planned anew with the loads)
 }
 
 extern "C" int slpic_set_spin_limit(slpic_ctx* c, uint32_t polls) {

@@ -1,0 +1,44 @@
+"""Steps captured into a caller's graph after the next step had been planned:
+replayed after the stores have changed, they run on a plan of the new ones."""
+import pytest
+
+from paper_2103_12194_gb300 import inputs
+
+from .test_gpu_host_state import make, same
+from .test_gpu_parity import mixed_state, slpic  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("field_mode", [0, 1])
+def test_replays_after_the_stores_have_changed(slpic, field_mode):  # noqa: F811
+    import torch
+    stream = torch.cuda.Stream()
+    spec = inputs.gap_spec(n_cells=64, V=300.0, pd_torr_cm=5.0, gamma_se=0.3,
+                           field_mode=field_mode, charge_shift=24)
+    sim, plain = make(slpic, field_mode, stream), make(slpic, field_mode)
+    for s in (sim, plain):
+        s.step(1)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream, capture_error_mode="thread_local"):
+        sim.step(1)
+
+    def load(n, seed):
+        def change(s):
+            for sp, m in enumerate(mixed_state(spec, n, n // 2, seed=seed)):
+                s.load(0, sp, m)
+        return change
+
+    for change in (load(300, 1), load(20000, 2), load(300, 3),
+                   lambda s: s.seed(0, 0, 9000, slpic.SEED_GAP, e_lo=1.0, e_hi=50.0),
+                   lambda s: s.clear_error(),
+                   lambda s: s.set_launch_shape(8, 2),
+                   load(1, 4)):
+        for s in (sim, plain):
+            change(s)
+        with torch.cuda.stream(stream):
+            graph.replay()
+        plain.step(1)
+        same(sim, plain)
+    sim.close()
+    plain.close()
