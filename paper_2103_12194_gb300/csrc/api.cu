@@ -124,6 +124,9 @@ struct slpic_ctx {
   // Recorded after the last upload; `loose` while that may not have arrived.
   cudaEvent_t loose_ev = nullptr;
   bool loose = false;
+  // Recorded after the last steps; `running` while they may not have finished.
+  cudaEvent_t steps_ev = nullptr;
+  bool running = false;
   // The instances' and stores' state as the host knows it; `known` while no
   // step has run since it was read (a step captured into a caller's graph runs
   // unseen: such a context always reads it again).
@@ -176,11 +179,11 @@ int set_device(slpic_ctx* c) {
   return SLPIC_OK;
 }
 
-bool capturing(const slpic_ctx* c) {
+bool capturing(cudaStream_t s) {
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  return c->stream && cudaStreamIsCapturing(c->stream, &st) == cudaSuccess &&
-         st != cudaStreamCaptureStatusNone;
+  return s && cudaStreamIsCapturing(s, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone;
 }
+bool capturing(const slpic_ctx* c) { return capturing(c->stream); }
 
 // Wait for the stream and deliver the reads queued on it (fails while the
 // stream is being captured; the reads are then dropped).
@@ -189,32 +192,39 @@ int drain(slpic_ctx* c) {
   if (e == cudaSuccess) {
     for (const auto& r : c->reads) std::memcpy(r.to, r.from, r.bytes);
     c->pin_used = 0;
-    c->loose = false;
+    c->loose = c->running = false;
   }
   c->reads.clear();
   if (e == cudaSuccess) return SLPIC_OK;
   return cuda_fail(c, e, "stream synchronize");
 }
 
-// Wait for the uploads alone: not by the stream, which may be the caller's to
-// destroy or in capture by now.
-int settle(slpic_ctx* c) {
-  if (!c->loose) return SLPIC_OK;
+// Wait for an event that was recorded while `pending`: not by the stream, which
+// may be the caller's to destroy or in capture by now.
+int wait_event(slpic_ctx* c, cudaEvent_t ev, bool* pending) {
+  if (!*pending) return SLPIC_OK;
   cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-  CK(cudaThreadExchangeStreamCaptureMode(&mode), "uploads");
-  const cudaError_t e = cudaEventSynchronize(c->loose_ev);
-  CK(cudaThreadExchangeStreamCaptureMode(&mode), "uploads");
-  if (e != cudaSuccess) return cuda_fail(c, e, "uploads");
-  c->loose = false;
+  CK(cudaThreadExchangeStreamCaptureMode(&mode), "wait");
+  const cudaError_t e = cudaEventSynchronize(ev);
+  CK(cudaThreadExchangeStreamCaptureMode(&mode), "wait");
+  if (e != cudaSuccess) return cuda_fail(c, e, "wait");
+  *pending = false;
+  return SLPIC_OK;
+}
+// Wait for the uploads alone.
+int settle(slpic_ctx* c) { return wait_event(c, c->loose_ev, &c->loose); }
+
+int record(slpic_ctx* c, cudaEvent_t* ev, bool* pending) {
+  if (!*ev) CK(cudaEventCreateWithFlags(ev, cudaEventDisableTiming), "event");
+  CK(cudaEventRecord(*ev, c->stream), "event");
+  *pending = true;
   return SLPIC_OK;
 }
 
 // Note that the stream holds uploads the host has not waited for.  Steps that
 // a caller captured may run on any stream: they find every upload arrived.
 int uploaded(slpic_ctx* c) {
-  if (!c->loose_ev) CK(cudaEventCreateWithFlags(&c->loose_ev, cudaEventDisableTiming), "event");
-  CK(cudaEventRecord(c->loose_ev, c->stream), "event");
-  c->loose = true;
+  if (int rc = record(c, &c->loose_ev, &c->loose)) return rc;
   return c->uncached ? settle(c) : SLPIC_OK;
 }
 
@@ -719,7 +729,7 @@ int materialize_deposit(slpic_ctx* c, int i) {
   CK(cudaGetLastError(), "deposit");
   c->dep_dirty[i] = 0;
   c->dep_step[i] = c->his[i].step;
-  return SLPIC_OK;
+  return uploaded(c);
 }
 
 void mark_stepped(slpic_ctx* c) {
@@ -951,6 +961,7 @@ int slpic_destroy(slpic_ctx* c) {
   for (void* p : c->allocs) cudaFree(p);
   if (c->pin) cudaFreeHost(c->pin);
   if (c->loose_ev) cudaEventDestroy(c->loose_ev);
+  if (c->steps_ev) cudaEventDestroy(c->steps_ev);
   if (c->capture_stream) cudaStreamDestroy(c->capture_stream);
   delete c;
   return SLPIC_OK;
@@ -958,13 +969,20 @@ int slpic_destroy(slpic_ctx* c) {
 
 int slpic_set_stream(slpic_ctx* c, void* stream) {
   if (!c) return SLPIC_ERR_INVALID_ARG;
-  // uploads queued on the old stream come before all that follows
-  if (c->committed && c->stream != (cudaStream_t)stream) {
+  // what the context has queued on the old stream comes before all that
+  // follows; a stream in capture cannot wait for it, so the host does
+  cudaStream_t to = (cudaStream_t)stream;
+  if (c->committed && c->stream != to && (c->loose || c->running)) {
     if (int rc = set_device(c)) return rc;
-    if (int rc = settle(c)) return rc;
-    c->pin_used = 0;
+    if (capturing(to)) {
+      if (int rc = settle(c)) return rc;
+      if (int rc = wait_event(c, c->steps_ev, &c->running)) return rc;
+    } else {
+      if (c->loose) CK(cudaStreamWaitEvent(to, c->loose_ev, 0), "set stream");
+      if (c->running) CK(cudaStreamWaitEvent(to, c->steps_ev, 0), "set stream");
+    }
   }
-  c->stream = (cudaStream_t)stream;
+  c->stream = to;
   return SLPIC_OK;
 }
 
@@ -1353,14 +1371,11 @@ int slpic_reset_counters(slpic_ctx* c, int inst) {
   return zero_counters(c, inst);
 }
 
-int slpic_step(slpic_ctx* c, int64_t n) {
-  if (!c || n < 0) return fail(c, SLPIC_ERR_INVALID_ARG, "bad step count");
-  if (int rc = prepare(c)) return rc;
-  c->last_launches = 0;
-  if (n > 0) {
-    mark_stepped(c);
-    if (int rc = begin_steps(c)) return rc;
-  }
+}  // extern "C"
+
+namespace {
+
+int launch_steps(slpic_ctx* c, int64_t n) {
   if (c->profiling) {
     for (int64_t k = 0; k < n; ++k) {
       if (c->ev_used + 2 > c->ev.size()) {
@@ -1401,6 +1416,23 @@ int slpic_step(slpic_ctx* c, int64_t n) {
   }
   CK(cudaGetLastError(), "step");
   return SLPIC_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+int slpic_step(slpic_ctx* c, int64_t n) {
+  if (!c || n < 0) return fail(c, SLPIC_ERR_INVALID_ARG, "bad step count");
+  if (int rc = prepare(c)) return rc;
+  c->last_launches = 0;
+  if (n == 0) return SLPIC_OK;
+  mark_stepped(c);
+  if (int rc = begin_steps(c)) return rc;
+  const int rc = launch_steps(c, n);
+  if (capturing(c)) return rc;
+  const int rc2 = record(c, &c->steps_ev, &c->running);
+  return rc ? rc : rc2;
 }
 
 int slpic_step_small(slpic_ctx* c, int64_t n, int64_t* done) {

@@ -436,9 +436,57 @@ static void replay_after_changes() {
   both([](slpic_ctx* c) { ok(slpic_set_launch_shape(c, 8, 2)); }, "launch shape");
 }
 
+// A change of stream right after steps: what follows on the new stream finds
+// them finished, also through a stream that did nothing, into a capture, or
+// when the old stream is gone.
+static void stream_changed_after_steps() {
+  enum { kRead, kLoad, kSeed, kCapture, kTwice, kDestroyed, kRefused, kEnd };
+  for (int from = 0; from < 2; ++from)
+    for (int what = kRead; what < kEnd; ++what) {
+      cudaStream_t a = from ? stream() : nullptr, b = stream();
+      Sim sim(a), plain;
+      sim.load(300), plain.load(300);
+      ok(slpic_step(sim.c, 40)), ok(slpic_step(plain.c, 40));
+      if (what == kRefused)  // (its first act is the deposit of the markers that are there)
+        for (const Sim* p : {&sim, &plain})
+          expect(slpic_seed(p->c, 0, 0, 1 << 20, SLPIC_SEED_REST, 0, 0, 0, 1) == SLPIC_ERR_CAPACITY,
+                 "too many markers");
+      if (what == kDestroyed && a) cudaStreamDestroy(a);
+      if (what == kTwice) ok(slpic_set_stream(sim.c, stream()));
+      cudaGraph_t g = nullptr;
+      if (what == kCapture) cudaStreamBeginCapture(b, cudaStreamCaptureModeRelaxed);
+      ok(slpic_set_stream(sim.c, b));
+      if (what == kCapture) {
+        cudaGraphExec_t e;
+        ok(slpic_step(sim.c, 1)), ok(slpic_step(plain.c, 1));
+        expect(cudaStreamEndCapture(b, &g) == cudaSuccess, "the capture is invalid");
+        cudaGraphInstantiate(&e, g, 0);
+        cudaGraphLaunch(e, b);
+      }
+      for (const Sim* p : {&sim, &plain}) {
+        if (what == kLoad) p->load(200);
+        if (what == kSeed) ok(slpic_seed(p->c, 0, 0, 70, SLPIC_SEED_REST, 0, 0, 0, 1));
+        if (what == kLoad || what == kSeed) ok(slpic_step(p->c, 2));
+      }
+      int64_t q[2][9];
+      if (what == kRefused) {
+        ok(slpic_read_charge(sim.c, 0, 0, q[0], 9));
+        ok(slpic_read_charge(plain.c, 0, 0, q[1], 9));
+        expect(std::equal(q[0], q[0] + 9, q[1]), "charge after a change of stream");
+      }
+      expect(sim.vx() == plain.vx(), "markers after a change of stream");
+      slpic_tallies t[2];
+      int64_t n[2] = {0, 0};
+      ok(slpic_read_history(sim.c, 0, &t[0], 1, &n[0]));
+      ok(slpic_read_history(plain.c, 0, &t[1], 1, &n[1]));
+      expect(n[0] == n[1], "steps after a change of stream");
+    }
+}
+
 int main(int argc, char** argv) {
   const std::map<std::string, std::function<void()>> all = {
       {"replay_after_changes", replay_after_changes},
+      {"stream_changed_after_steps", stream_changed_after_steps},
   };
   if (argc != 2 || !all.count(argv[1])) return 2;
   all.at(argv[1])();

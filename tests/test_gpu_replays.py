@@ -1,5 +1,5 @@
-"""Steps captured into a caller's graph after the next step had been planned:
-replayed after the stores have changed, they run on a plan of the new ones."""
+"""Steps that the host has not waited for: replayed in a caller's graph after the
+stores have changed, and in flight on a stream that the context leaves."""
 import pytest
 
 from paper_2103_12194_gb300 import inputs
@@ -40,5 +40,38 @@ def test_replays_after_the_stores_have_changed(slpic, field_mode):  # noqa: F811
             graph.replay()
         plain.step(1)
         same(sim, plain)
+    sim.close()
+    plain.close()
+
+
+@pytest.mark.parametrize("own", [False, True])
+@pytest.mark.parametrize("call", ["count", "load", "seed"])
+def test_change_of_stream_right_after_steps(slpic, call, own):  # noqa: F811
+    """Calls on a new stream find the steps of the old one (the NULL stream, or
+    one that does not wait for it) finished."""
+    import torch
+    spec = inputs.gap_spec(n_cells=64, V=300.0, pd_torr_cm=5.0, gamma_se=0.3, field_mode=1,
+                           charge_shift=24)
+    plain = make(slpic, 1)
+    plain.step(40)
+    plain.synchronize()
+    old = torch.cuda.Stream() if own else torch.cuda.default_stream()
+    sim = make(slpic, 1, old)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(old):
+        torch.cuda._sleep(20_000_000)  # about 10 ms: the steps start after the calls below
+    sim.step(40)
+    sim.set_stream(torch.cuda.Stream())
+    for s in (sim, plain):
+        if call == "load":
+            for sp, m in enumerate(mixed_state(spec, 500, 200, seed=9)):
+                s.load(0, sp, m)
+        elif call == "seed":
+            s.seed(0, 0, 700, slpic.SEED_GAP, e_lo=1.0, e_hi=50.0)
+        else:
+            s.count(0, 0)
+        if call != "count":
+            s.step(3)
+    same(sim, plain)
     sim.close()
     plain.close()
