@@ -127,6 +127,7 @@ struct slpic_ctx {
   // Recorded after the last steps; `running` while they may not have finished.
   cudaEvent_t steps_ev = nullptr;
   bool running = false;
+  cudaEvent_t null_ev = nullptr;  // see follow_null
   // The instances' and stores' state as the host knows it; `known` while no
   // step has run since it was read (a step captured into a caller's graph runs
   // unseen: such a context always reads it again).
@@ -228,6 +229,19 @@ int uploaded(slpic_ctx* c) {
   return c->uncached ? settle(c) : SLPIC_OK;
 }
 
+// What the context's stream does from here on comes after the work so far of
+// the NULL stream, and so of the streams that the NULL stream waits for.
+int follow_null(slpic_ctx* c) {
+  if (!c->stream) return SLPIC_OK;
+  if (!c->null_ev)
+    CK(cudaEventCreateWithFlags(&c->null_ev, cudaEventDisableTiming), "event");
+  CK(cudaEventRecord(c->null_ev, nullptr), "event");
+  CK(cudaStreamWaitEvent(c->stream, c->null_ev, 0), "event");
+  return SLPIC_OK;
+}
+// The same where steps that a caller captured may be running there.
+int follow_replays(slpic_ctx* c) { return c->uncached ? follow_null(c) : SLPIC_OK; }
+
 // Room for `bytes` bytes of pinned memory until the next drain.
 int pin_room(slpic_ctx* c, size_t bytes, char** p) {
   const size_t need = (bytes + 15) & ~size_t(15);
@@ -310,6 +324,7 @@ int sync(slpic_ctx* c) {
   }
   if (capturing(c)) return drain(c);
   if (c->known) return SLPIC_OK;
+  if (int rc = follow_replays(c)) return rc;
   if (int rc = ask_state(c)) return rc;
   if (int rc = drain(c)) return rc;
   return take_state(c);
@@ -320,6 +335,7 @@ int sync(slpic_ctx* c) {
 int read_with_state(slpic_ctx* c, void* host, const void* dev, size_t bytes, int* err) {
   if (capturing(c)) return drain(c);
   const bool ask = !c->known;
+  if (int rc = follow_replays(c)) return rc;
   if (ask)
     if (int rc = ask_state(c)) return rc;
   if (int rc = get(c, host, dev, bytes)) return rc;
@@ -962,6 +978,7 @@ int slpic_destroy(slpic_ctx* c) {
   if (c->pin) cudaFreeHost(c->pin);
   if (c->loose_ev) cudaEventDestroy(c->loose_ev);
   if (c->steps_ev) cudaEventDestroy(c->steps_ev);
+  if (c->null_ev) cudaEventDestroy(c->null_ev);
   if (c->capture_stream) cudaStreamDestroy(c->capture_stream);
   delete c;
   return SLPIC_OK;
@@ -1462,6 +1479,7 @@ int slpic_clear_error(slpic_ctx* c) {
   if (!c) return SLPIC_ERR_INVALID_ARG;
   if (!c->committed) return SLPIC_OK;
   if (int rc = set_device(c)) return rc;
+  if (int rc = follow_replays(c)) return rc;
   CK(cudaMemsetAsync(&c->d_ctrl->error, 0, sizeof(int), c->stream), "clear");
   for (int i = 0; i < c->n_inst; ++i) {
     const InstDev& P = c->h_inst[i];
@@ -1587,6 +1605,7 @@ int slpic_read_field(slpic_ctx* c, int inst, double* phi, double* E, int64_t n) 
   }
   // the step keeps only the node field; phi is formed from the last deposit
   // (in the frozen-field mode it stays the vacuum solution)
+  if (int rc = follow_replays(c)) return rc;
   if (P.field_mode == 1 && c->stepped[inst]) {
     launch_phi(c->refs, inst, P.n_cells, c->stream);
     CK(cudaGetLastError(), "read field");

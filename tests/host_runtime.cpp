@@ -483,10 +483,46 @@ static void stream_changed_after_steps() {
     }
 }
 
+// Steps that a caller replays on the NULL stream, or on one that it waits for,
+// come before the calls that follow on a stream that does not wait for it.
+static void replays_on_the_null_stream() {
+  for (int mode : {SLPIC_FIELD_FROZEN, SLPIC_FIELD_POISSON})
+    for (cudaStream_t on : {(cudaStream_t) nullptr, stream(true)})
+      for (int what = 0; what < 6; ++what) {
+        cudaStream_t s = stream();
+        Sim sim(s, mode), plain(nullptr, mode);
+        sim.load(300), plain.load(300);
+        cudaGraphExec_t g = captured(sim, s, 1);
+        cudaStreamSynchronize(nullptr);
+        cudaGraphLaunch(g, on), cudaGraphLaunch(g, on);
+        ok(slpic_step(plain.c, 2));
+        double f[2][2][9];
+        int64_t q[2][9], n[2];
+        slpic_tallies t;
+        const slpic_ctx* c = sim.c;
+        for (const Sim* p : {&sim, &plain}) {
+          const int k = p->c != c;
+          if (what == 0) ok(slpic_read_field(p->c, 0, f[k][0], f[k][1], 9));
+          if (what == 1) ok(slpic_read_charge(p->c, 0, 0, q[k], 9));
+          if (what == 2) ok(slpic_read_history(p->c, 0, &t, 1, &n[k]));
+          if (what == 3) ok(slpic_seed(p->c, 0, 0, 70, SLPIC_SEED_REST, 0, 0, 0, 1));
+          if (what == 4) ok(slpic_clear_error(p->c));
+          if (what == 5) ok(slpic_read_tallies(p->c, 0, &t));
+          if (!k) expect(!on || on->done == on->ops.size(), "replays after a call");
+        }
+        if (what == 0) expect(!std::memcmp(f[0], f[1], sizeof f[0]), "field after replays");
+        if (what == 1) expect(!std::memcmp(q[0], q[1], sizeof q[0]), "charge after replays");
+        if (what == 2) expect(n[0] == n[1], "steps after replays");
+        const std::vector<float> a = sim.vx(), b = plain.vx();
+        expect(a == b, "markers after replays");
+      }
+}
+
 int main(int argc, char** argv) {
   const std::map<std::string, std::function<void()>> all = {
       {"replay_after_changes", replay_after_changes},
       {"stream_changed_after_steps", stream_changed_after_steps},
+      {"replays_on_the_null_stream", replays_on_the_null_stream},
   };
   if (argc != 2 || !all.count(argv[1])) return 2;
   all.at(argv[1])();

@@ -1,5 +1,6 @@
 """Steps that the host has not waited for: replayed in a caller's graph after the
 stores have changed, and in flight on a stream that the context leaves."""
+import numpy as np
 import pytest
 
 from paper_2103_12194_gb300 import inputs
@@ -72,6 +73,32 @@ def test_change_of_stream_right_after_steps(slpic, call, own):  # noqa: F811
             s.count(0, 0)
         if call != "count":
             s.step(3)
+    same(sim, plain)
+    sim.close()
+    plain.close()
+
+
+@pytest.mark.parametrize("call", ["count", "field", "charge", "history", "seed"])
+def test_replays_on_the_null_stream(slpic, call):  # noqa: F811
+    """A call on a stream that does not wait for the NULL stream finds the
+    steps replayed there finished."""
+    import torch
+    field_mode = 0 if call == "charge" else 1
+    stream = torch.cuda.Stream()
+    sim, plain = make(slpic, field_mode, stream), make(slpic, field_mode)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream, capture_error_mode="thread_local"):
+        sim.step(2)
+    plain.step(4)
+    plain.synchronize()
+    args = {"field": (0,), "history": (0,),
+            "seed": (0, 0, 700, slpic.SEED_GAP, 1.0, 1.0, 50.0)}.get(call, (0, 0))
+    want = getattr(plain, call)(*args)
+    torch.cuda._sleep(20_000_000)
+    graph.replay()
+    graph.replay()
+    got = getattr(sim, call)(*args)
+    assert np.array_equal(np.asarray(got), np.asarray(want))
     same(sim, plain)
     sim.close()
     plain.close()
