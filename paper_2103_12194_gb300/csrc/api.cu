@@ -1313,6 +1313,8 @@ int load_common(slpic_ctx* c, int inst, int species, const Arrays& src, int64_t 
   void* f[7];
   std::memcpy(f, src.f, sizeof f);
   bool direct = kind == cudaMemcpyDeviceToDevice;
+  if (n > 0)  // (work on the NULL stream may be filling them)
+    if (int rc = follow_null(c)) return rc;
   for (int k = 0; k < 7 && direct && n > 0; ++k)
     direct = kernel_readable(c, f[k], field_bytes(c, k, (size_t)n), field_bytes(c, k, 1));
   if (n > 0 && !direct) {

@@ -518,11 +518,39 @@ static void replays_on_the_null_stream() {
       }
 }
 
+// Device arrays, and pinned ones, that work on the NULL stream fills, loaded on
+// a stream that does not wait for it.
+static void device_arrays() {
+  Sim sim(stream()), plain;
+  Host h(500, 3.0f);
+  const void* src[7] = {h.soa.cell, h.soa.off, h.soa.vx, h.soa.vy, h.soa.vz, h.soa.wj, h.soa.id};
+  void* d[7];
+  for (int k = 0; k < 7; ++k) cudaMalloc(&d[k], 2000);
+  sim.load(10), plain.load(500, 3.0f);
+  for (int k = 0; k < 7; ++k) cudaMemcpyAsync(d[k], src[k], 2000, cudaMemcpyHostToDevice, nullptr);
+  slpic_soa_f32 soa = {(int32_t*)d[0], (float*)d[1], (float*)d[2],   (float*)d[3],
+                       (float*)d[4],   (float*)d[5], (uint32_t*)d[6]};
+  ok(slpic_load_particles_device(sim.c, 0, 0, &soa, 500, 500));
+  expect(sim.vx() == plain.vx(), "markers from device arrays");
+  void* p[7];
+  for (int k = 0; k < 7; ++k) {
+    cudaHostAlloc(&p[k], 2000, 0);
+    std::memset(p[k], 0, 2000);
+    cudaMemcpyAsync(p[k], d[k], 2000, cudaMemcpyDeviceToHost, nullptr);
+  }
+  slpic_soa_f32 pinned = {(int32_t*)p[0], (float*)p[1], (float*)p[2],   (float*)p[3],
+                          (float*)p[4],   (float*)p[5], (uint32_t*)p[6]};
+  sim.load(10);
+  ok(slpic_load_particles(sim.c, 0, 0, &pinned, 500, 500));
+  expect(sim.vx() == plain.vx(), "markers from pinned arrays");
+}
+
 int main(int argc, char** argv) {
   const std::map<std::string, std::function<void()>> all = {
       {"replay_after_changes", replay_after_changes},
       {"stream_changed_after_steps", stream_changed_after_steps},
       {"replays_on_the_null_stream", replays_on_the_null_stream},
+      {"device_arrays", device_arrays},
   };
   if (argc != 2 || !all.count(argv[1])) return 2;
   all.at(argv[1])();

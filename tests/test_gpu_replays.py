@@ -102,3 +102,26 @@ def test_replays_on_the_null_stream(slpic, call):  # noqa: F811
     same(sim, plain)
     sim.close()
     plain.close()
+
+
+def test_device_arrays_filled_on_the_null_stream(slpic):  # noqa: F811
+    """load_device on a stream that does not wait for the NULL stream takes the
+    values that work queued there writes."""
+    import torch
+    sim, plain = make(slpic, 0, torch.cuda.Stream()), make(slpic, 0)
+    m = sim.particles(0, 0)
+    host = {k: torch.from_numpy(v.view(np.int32) if k == "id" else v).pin_memory()
+            for k, v in m.items()}
+    dev = {k: torch.zeros_like(v, device="cuda") for k, v in host.items()}
+    sim.count(0, 0)
+    torch.cuda.synchronize()
+    torch.cuda._sleep(20_000_000)
+    for k in dev:
+        dev[k].copy_(host[k], non_blocking=True)
+    sim.load_device(0, 0, dev, next_id=len(m["id"]))
+    plain.load(0, 0, m, next_id=len(m["id"]))
+    for s in (sim, plain):
+        s.step(2)
+    same(sim, plain)
+    sim.close()
+    plain.close()
