@@ -714,6 +714,9 @@ int commit(slpic_ctx* c) {
   c->push_grid = c->refs.push_grid = sms * bps;
   c->move_grid = sms * 2;
   c->collide_grid = sms * std::min(c->collide_per_sm, c->collide_resident);
+  // the copies and fills above went through the NULL stream, and the context's
+  // need not wait for that one
+  CK(cudaStreamSynchronize(nullptr), "set-up");
   c->hs.assign(nseg, SpeciesState{});
   c->his.assign(c->n_inst, InstState{});
   c->tail.assign(nseg, 0);
@@ -2230,21 +2233,23 @@ extern "C" int slpic_load(slpic_ctx* c, const void* buf, size_t size) {
     }
     // the counters, tallies, field and deposit as saved (the loads above
     // set the seeded and live weights from the markers)
-    if (int rc = drain(c)) return rc;
+    auto up = [&](void* dev, const void* from, size_t bytes) {
+      return cudaMemcpyAsync(dev, from, bytes, cudaMemcpyHostToDevice, c->stream);
+    };
     c->his[i] = r.is;
-    CK(cudaMemcpy(c->d_istate + i, &r.is, sizeof r.is, cudaMemcpyHostToDevice), "load");
-    CK(cudaMemcpy(P.total, &r.total, sizeof r.total, cudaMemcpyHostToDevice), "load");
-    CK(cudaMemcpy(P.ring, ring, sizeof(TallyRec) * P.ring_len, cudaMemcpyHostToDevice), "load");
-    CK(cudaMemcpy(P.phi, phi, nn * 8, cudaMemcpyHostToDevice), "load");
-    CK(cudaMemcpy(P.E64, e64, nn * 8, cudaMemcpyHostToDevice), "load");
-    CK(cudaMemcpy(P.E32, e32, nn * 4, cudaMemcpyHostToDevice), "load");
-    for (int s = 0; s < 2; ++s)
-      CK(cudaMemcpy(P.rho_last[s], rho[s], nn * 8, cudaMemcpyHostToDevice), "load");
+    if (int rc = write_inst_state(c, i)) return rc;
+    if (int rc = put(c, P.total, &r.total, sizeof r.total)) return rc;
+    CK(up(P.ring, ring, sizeof(TallyRec) * P.ring_len), "load");
+    CK(up(P.phi, phi, nn * 8), "load");
+    CK(up(P.E64, e64, nn * 8), "load");
+    CK(up(P.E32, e32, nn * 4), "load");
+    for (int s = 0; s < 2; ++s) CK(up(P.rho_last[s], rho[s], nn * 8), "load");
+    if (int rc = drain(c)) return rc;  // (the buffer is the caller's)
     c->stepped[i] = (char)r.stepped;
     c->dep_dirty[i] = 0;
     c->dep_step[i] = r.is.step;
   }
-  return SLPIC_OK;  // (planned anew with the loads)
+  return SLPIC_OK;  // (the next step is planned anew with the loads)
 }
 
 extern "C" int slpic_set_spin_limit(slpic_ctx* c, uint32_t polls) {

@@ -545,12 +545,39 @@ static void device_arrays() {
   expect(sim.vx() == plain.vx(), "markers from pinned arrays");
 }
 
+// A snapshot restored, and a context set up, on a stream that does not wait for
+// the NULL stream.
+static void copies_on_the_null_stream() {
+  Sim plain(nullptr, SLPIC_FIELD_FROZEN);
+  plain.load(300);
+  ok(slpic_step(plain.c, 1));
+  int64_t q[2][9];
+  size_t size = 0;
+  ok(slpic_seed(plain.c, 0, 1, 50, SLPIC_SEED_REST, 0, 0, 0, 1));
+  ok(slpic_step(plain.c, 1));
+  ok(slpic_save(plain.c, nullptr, 0, &size));
+  std::vector<char> snap(size);
+  ok(slpic_save(plain.c, snap.data(), size, &size));
+  ok(slpic_read_charge(plain.c, 0, 1, q[1], 9));
+  cudaStreamSynchronize(nullptr);
+  Sim sim(stream());
+  int64_t n = 0;
+  ok(slpic_count(sim.c, 0, 0, &n));
+  expect(g_null.done == g_null.ops.size(), "copies of the set-up");
+  ok(slpic_load(sim.c, snap.data(), size));
+  expect(g_null.done == g_null.ops.size(), "copies of the snapshot");
+  ok(slpic_read_charge(sim.c, 0, 1, q[0], 9));
+  expect(std::equal(q[0], q[0] + 9, q[1]), "charge of a snapshot");
+  expect(sim.vx() == plain.vx(), "markers of a snapshot");
+}
+
 int main(int argc, char** argv) {
   const std::map<std::string, std::function<void()>> all = {
       {"replay_after_changes", replay_after_changes},
       {"stream_changed_after_steps", stream_changed_after_steps},
       {"replays_on_the_null_stream", replays_on_the_null_stream},
       {"device_arrays", device_arrays},
+      {"copies_on_the_null_stream", copies_on_the_null_stream},
   };
   if (argc != 2 || !all.count(argv[1])) return 2;
   all.at(argv[1])();

@@ -27,7 +27,8 @@ def binary(tmp_path_factory):
 
 
 @pytest.mark.parametrize("scenario", ["replay_after_changes", "stream_changed_after_steps",
-                                      "replays_on_the_null_stream", "device_arrays"])
+                                      "replays_on_the_null_stream", "device_arrays",
+                                      "copies_on_the_null_stream"])
 def test_host_side(binary, scenario):
     p = subprocess.run([binary, scenario], capture_output=True, text=True, timeout=60)
     assert p.returncode == 0, p.stdout + p.stderr
