@@ -1508,8 +1508,8 @@ int slpic_count(slpic_ctx* c, int inst, int species, int64_t* n) {
 
 namespace {
 
-// Marker arrays up to this size are read through pinned memory, all seven with
-// one wait; larger ones straight into the caller's arrays.
+// Marker arrays up to this size are read through pinned memory, with one wait
+// for as many as fit there; larger ones straight into the caller's arrays.
 constexpr size_t kPinnedRead = size_t(1) << 20;
 
 int read_common(slpic_ctx* c, int inst, int species, const Arrays& host, int64_t capacity,
@@ -1547,7 +1547,14 @@ int read_common(slpic_ctx* c, int inst, int species, const Arrays& host, int64_t
       if (b <= kPinnedRead) {
         if (int r3 = get(c, host.f[k], f[k], b)) return r3;
       } else {
-        CK(cudaMemcpyAsync(host.f[k], f[k], b, cudaMemcpyDeviceToHost, c->stream), "read");
+        const cudaError_t e =
+            cudaMemcpyAsync(host.f[k], f[k], b, cudaMemcpyDeviceToHost, c->stream);
+        if (e != cudaSuccess) {
+          // nothing of this call writes to the caller's arrays after it
+          c->reads.clear();
+          drain(c);
+          return cuda_fail(c, e, "read");
+        }
       }
     }
     if (int r3 = drain(c)) return r3;

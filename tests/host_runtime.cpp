@@ -571,12 +571,34 @@ static void copies_on_the_null_stream() {
   expect(sim.vx() == plain.vx(), "markers of a snapshot");
 }
 
+// A read of markers that fails on the way leaves nothing behind that would
+// write to the caller's arrays later.
+static void failed_read() {
+  const int n = 200000;  // the cells go through pinned memory, the reals do not
+  Sim sim(nullptr, SLPIC_FIELD_FROZEN, n);
+  ok(slpic_set_precision(sim.c, 64));
+  ok(slpic_seed(sim.c, 0, 0, n, SLPIC_SEED_REST, 0, 0, 0, 1));
+  int64_t got = 0;
+  ok(slpic_count(sim.c, 0, 0, &got));
+  std::vector<int32_t> cell(n, -7);
+  std::vector<uint32_t> id(n);
+  std::vector<double> r(5 * n);
+  slpic_soa_f64 soa = {cell.data(), r.data(), r.data() + n, r.data() + 2 * n, r.data() + 3 * n,
+                       r.data() + 4 * n, id.data()};
+  g_fail_copy = 1;
+  expect(slpic_read_particles_f64(sim.c, 0, 0, &soa, n, &got) == SLPIC_ERR_CUDA, "a failing copy");
+  slpic_tallies t;
+  ok(slpic_read_tallies(sim.c, 0, &t));
+  expect(std::count(cell.begin(), cell.end(), -7) == n, "an array written after its call");
+}
+
 int main(int argc, char** argv) {
   const std::map<std::string, std::function<void()>> all = {
       {"replay_after_changes", replay_after_changes},
       {"stream_changed_after_steps", stream_changed_after_steps},
       {"replays_on_the_null_stream", replays_on_the_null_stream},
       {"device_arrays", device_arrays},
+      {"failed_read", failed_read},
       {"copies_on_the_null_stream", copies_on_the_null_stream},
   };
   if (argc != 2 || !all.count(argv[1])) return 2;

@@ -27,7 +27,7 @@ def binary(tmp_path_factory):
 
 
 @pytest.mark.parametrize("scenario", ["replay_after_changes", "stream_changed_after_steps",
-                                      "replays_on_the_null_stream", "device_arrays",
+                                      "replays_on_the_null_stream", "device_arrays", "failed_read",
                                       "copies_on_the_null_stream"])
 def test_host_side(binary, scenario):
     p = subprocess.run([binary, scenario], capture_output=True, text=True, timeout=60)
