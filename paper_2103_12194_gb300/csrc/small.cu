@@ -487,8 +487,10 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(DeviceRefs r, long l
       }
     }
     __syncthreads();
-    // (the step is not committed then)
-    if (single ? sh.err : *((volatile int*)&ctrl->error)) break;
+    // (the step is not committed then.  Its own errors alone: another CTA may
+    // set the device's word between two threads' reads of it, and the CTA must
+    // leave as one; it stops for that at the next grid barrier)
+    if (sh.err) break;
 
     // ---- 3. counts, fills and where the stores end ---------------------------
     if (t < 2) {
