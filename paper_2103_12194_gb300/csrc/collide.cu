@@ -97,7 +97,10 @@ __global__ void __launch_bounds__(coll_warps<R>() * 32, sizeof(R) == 4 ? 1 : 3)
   constexpr int W = coll_warps<R>();
   step_kernel_entry();
   Control* ctrl = r.ctrl;
-  if (*((volatile int*)&ctrl->error)) return;
+  // (as one: an item of another CTA that does not fit its store may set the
+  // word between two threads' reads of it, and thread 0 sets the counter that
+  // hands out the items)
+  if (__syncthreads_or(*((volatile int*)&ctrl->error))) return;
   const unsigned int n_items = ctrl->n_coll_items;
   // (k_finish plans the next step while the births are still placed)
   if (blockIdx.x == 0)

@@ -815,7 +815,9 @@ __global__ void __launch_bounds__(kMoveThreads) k_move(DeviceRefs r) {
   constexpr int kPerLaneTiles = kMoveChunkTiles / 32;
   step_kernel_entry();
   Control* ctrl = r.ctrl;
-  if (*((volatile int*)&ctrl->error)) return;
+  // (as one: a wait of another CTA that runs out may set the word between two
+  // threads' reads of it, and the chunks are handed out by thread 0)
+  if (__syncthreads_or(*((volatile int*)&ctrl->error))) return;
   // the field of the step's Poisson solves, a block of nodes at a time
   for (int u = blockIdx.x; u < r.n_field; u += gridDim.x) {
     const int inst = field_inst(r, u);
