@@ -28,8 +28,9 @@
 // The births are not placed here.  Their slots and serial numbers follow the
 // (tile, slot) order of their parents over the whole instance, which only the
 // counts of all items give: each item leaves its number of births and, in
-// order, the records of its ionizations, and the next kernel (k_finish, beside
-// the end of the step) places them (place_births).  Placing them here took an
+// order, the records of its ionizations (or where its emitted electrons are
+// staged), and the next kernel (k_finish, beside the end of the step) places
+// them (place_births).  Placing them here took an
 // ordered look-back over the chunks and three barriers a chunk: CTAs waited
 // for the slowest before them.
 //
@@ -84,6 +85,24 @@ __device__ __forceinline__ void add_counter(const DeviceRefs& r, int inst, int k
   if (te + n + n_see > (unsigned long long)P.sp[kElectron].cap_tiles * kTile ||
       ti + n > (unsigned long long)P.sp[kIon].cap_tiles * kTile)
     atomicCAS(&r.ctrl->error, 0, kErrCapacity);
+}
+
+// The slots of the staging that the electrons emitted by ion tiles k0 .. k1 - 1
+// lie in, in order, from list[0] on (one warp; rare, kept out of line).
+__device__ __noinline__ void list_emissions(const uint32_t* births, uint32_t k0, uint32_t k1,
+                                            uint32_t* list) {
+  const uint32_t lane = threadIdx.x & 31;
+  for (uint32_t k = k0 + lane; k - lane < k1; k += 32) {
+    const uint32_t n = k < k1 ? births[k] : 0u;
+    uint32_t inc = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+      if (lane >= (uint32_t)o) inc += y;
+    }
+    for (uint32_t e = 0; e < n; ++e) list[inc - n + e] = k * kTile + e;
+    list += __shfl_sync(0xFFFFFFFFu, inc, 31);
+  }
 }
 
 }  // namespace
@@ -351,6 +370,11 @@ __global__ void __launch_bounds__(coll_warps<R>() * 32, sizeof(R) == 4 ? 1 : 3)
             const uint32_t k1 = min(k0 + kCollIonTiles, r.sstate[inst * 2 + kIon].n_tiles);
             for (uint32_t k = k0 + lane; k < k1; k += 32) births += I.births[k];
             births = __reduce_add_sync(0xFFFFFFFFu, births);
+            if (births)
+              list_emissions(I.births, k0, k1,
+                             reinterpret_cast<uint32_t*>(
+                                 I.buf[r.sstate[inst * 2 + kIon].cur ^ 1u]) +
+                                 (size_t)k0 * kTile);
           } else {
             // wt consecutive tiles, tile kw + j at lane j: their candidates are
             // numbered in (tile, slot) order

@@ -353,6 +353,7 @@ __device__ __noinline__ void place_births(const DeviceRefs& r, int b, int nb, ui
     const SpeciesDev& E = P.sp[kElectron];
     const Markers<R> me{E.buf[B.cur[0]]}, mi{P.sp[kIon].buf[B.cur[1]]};
     const uint32_t* list = reinterpret_cast<const uint32_t*>(E.buf[B.cur[0] ^ 1u]);
+    const uint32_t* ilist = reinterpret_cast<const uint32_t*>(P.sp[kIon].buf[B.cur[1] ^ 1u]);
     const unsigned int e_items = B.e_items;
     for (; i0 < end; i0 += kFinThreads) {
       // prefixes of up to kFinThreads items
@@ -379,14 +380,11 @@ __device__ __noinline__ void place_births(const DeviceRefs& r, int b, int nb, ui
           born_pair<R>(P, pe, mi[B.tail[1] + rank], cr.cell, cr.off, cr.wj, cr.id, step, cr.vx,
                        B.next_id[0] + rank, B.next_id[1] + rank);
         } else {
-          // emitted at the cathode by an ion of the item's tiles
-          uint32_t k = (local - e_items) * kCollIonTiles, e = q, f;
-          while (e >= (f = P.sp[kIon].births[k])) {
-            e -= f;
-            ++k;
-          }
-          write_marker(pe, 0, (R)0, (R)0, (R)0, (R)0,
-                       reinterpret_cast<const R*>(E.stage_w)[(size_t)k * kTile + e],
+          // emitted at the cathode by an ion of the item's tiles (looking for
+          // the tile here, one count after the other, took k_finish from 15 to
+          // 28 us on 3e7 ions that emit 10 electrons a step)
+          const uint32_t o = ilist[(size_t)(local - e_items) * kCollIonTiles * kTile + q];
+          write_marker(pe, 0, (R)0, (R)0, (R)0, (R)0, reinterpret_cast<const R*>(E.stage_w)[o],
                        kGenBit | ((B.next_id[0] + rank) & kSerialMask));
         }
       }

@@ -234,7 +234,8 @@ struct SpeciesDev {
   void* crec;         // electrons: [cap_tiles * kTile] CandRec<R>, the tile's
                       // null-collision candidates in slot order (during a step
                       // the buffer that is not in use holds, from an item's
-                      // first slot on, the numbers of its ionizations' records)
+                      // first slot on, the numbers of its ionizations' records,
+                      // and that of the ions where its emissions are staged)
   uint32_t* n_cand;   // electrons: [cap_tiles] candidates per tile
   uint32_t cap_tiles;
   uint32_t pad;
