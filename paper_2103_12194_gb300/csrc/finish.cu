@@ -94,10 +94,9 @@ struct FieldShared {
 };
 __device__ __forceinline__ void poisson_field(const InstDev& P, int block, FieldShared& sh) {
   constexpr int kPer = kFieldNodes / kMoveThreads;
-  static_assert(kPer == 4, "two 16-byte loads of each deposit");
   const int N = P.n_cells, t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int k0 = block * kFieldNodes + t * kPer;
-  long long net[kPer] = {0, 0, 0, 0};
+  long long net[kPer] = {};
 #pragma unroll
   for (int j = 0; j < kPer; ++j) {
     const int k = k0 + j;
@@ -119,7 +118,9 @@ __device__ __forceinline__ void poisson_field(const InstDev& P, int block, Field
       sh.D1 = (P.V + P.pois_C * (double)W) / (double)N;
     }
   }
-  const long long loc = net[0] + net[1] + net[2] + net[3];
+  long long loc = 0;
+#pragma unroll
+  for (int j = 0; j < kPer; ++j) loc += net[j];
   const long long inc = warp_incl_scan(loc, lane);
   if (lane == 31) sh.w[warp] = inc;
   __syncthreads();

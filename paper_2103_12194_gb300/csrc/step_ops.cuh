@@ -468,28 +468,23 @@ __device__ T block_incl_scan(T v, T* buf) {
   return r;
 }
 
-// Net deposit (ions minus electrons) at node k of the last step: from the
-// CTA's shared copy when there is one, else from the last deposit.
-__device__ __forceinline__ long long net_at(const InstDev& P, const long long* s_net, int k) {
-  return s_net ? s_net[k] : P.rho_last[kIon][k] - P.rho_last[kElectron][k];
-}
-
-// The exact integer sums of the 1D Poisson solve over the last step's net
-// deposit (all threads of a kThreads CTA; thread t covers k = k0 ..
-// k0 + chunk - 1 of 1..N): returns D_1 = (V + C J_N) / N and writes I_{k0}.
-template <int kThreads = kFinThreads>
+// The exact integer sums of the 1D Poisson solve over a step's net deposit (ions
+// minus electrons, in the CTA's shared memory; all threads of a kThreads CTA;
+// thread t covers k = k0 .. k0 + chunk - 1 of 1..N): returns D_1 = (V + C J_N)
+// / N and writes I_{k0}.
+template <int kThreads>
 __device__ double poisson_d1(const InstDev& P, const long long* s_net, int k0, int chunk,
                              long long* s_i64, __int128* s_i128, long long* I_k0) {
   const int N = P.n_cells;
   long long loc = 0;
-  for (int k = k0; k < k0 + chunk && k <= N - 1; ++k) loc += net_at(P, s_net, k);
+  for (int k = k0; k < k0 + chunk && k <= N - 1; ++k) loc += s_net[k];
   const long long inc = block_incl_scan<long long, kThreads>(loc, s_i64);
   long long Ik = inc - loc;  // I_k at the chunk start (exclusive of net_k)
   *I_k0 = Ik;
   __int128 locJ = 0;
   for (int k = k0; k < k0 + chunk && k <= N; ++k) {
     locJ += (__int128)Ik;
-    if (k <= N - 1) Ik += net_at(P, s_net, k);
+    if (k <= N - 1) Ik += s_net[k];
   }
   const __int128 incJ = block_incl_scan<__int128, kThreads>(locJ, s_i128);
   // one thread forms D_1 (FP64 is scarce on this part) and shares it
