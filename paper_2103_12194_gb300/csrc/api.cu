@@ -709,6 +709,7 @@ int commit(slpic_ctx* c) {
   int sms = 0;
   CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device), "attributes");
   c->sms = sms;
+  c->refs.coll_share = (unsigned int)std::max(kCollPerSm * sms / c->n_inst, 1);
   c->max_push_warps = max_warps;
   c->blocks_per_sm = bps;
   c->push_grid = c->refs.push_grid = sms * bps;

@@ -149,12 +149,12 @@ __device__ __forceinline__ void poisson_field(const InstDev& P, int block, Field
 
 // Tiles per electron collision item of an instance of n_tiles electron tiles:
 // `room` of them hold kCollTarget candidates.  Fewer where the instance would
-// not give its share of kCollSpread items, but in float not below an eighth of
-// room (a round of 32 candidates).
-__device__ __forceinline__ unsigned int item_tiles(unsigned long long room, uint32_t n_tiles,
-                                                   int n_inst, int fp64) {
-  const unsigned long long share = (unsigned long long)n_tiles * n_inst / kCollSpread;
-  const unsigned long long most = min(room, max(share, fp64 ? 1ull : room / 8u));
+// not give coll_share items, but in float not below an eighth of room (a round
+// of 32 candidates).
+__device__ __forceinline__ unsigned int item_tiles(const DeviceRefs& r, unsigned long long room,
+                                                   uint32_t n_tiles) {
+  const unsigned long long share = n_tiles / r.coll_share;
+  const unsigned long long most = min(room, max(share, r.fp64 ? 1ull : room / 8u));
   return (unsigned int)min(max(most, 1ull), (unsigned long long)kCollMaxTiles);
 }
 
@@ -194,7 +194,7 @@ __device__ void plan_next_warp(const DeviceRefs& r) {
     const int i = lane * (kPlanPerLane / 2) + j;
     nc[j] = 0;
     if (i < r.n_inst) {
-      const long long T = item_tiles(r.coll_room[i], r.sstate[2 * i].n_tiles, r.n_inst, r.fp64);
+      const long long T = item_tiles(r, r.coll_room[i], r.sstate[2 * i].n_tiles);
       r.coll_tiles[i] = (unsigned int)T;
       nc[j] = ((long long)r.sstate[2 * i].n_tiles + T - 1) / T +
               ((long long)r.sstate[2 * i + 1].n_tiles + kCollIonTiles - 1) / kCollIonTiles;
@@ -295,7 +295,7 @@ __device__ void plan_next(const DeviceRefs& r, long long* s_buf) {
     const int i = base + t;
     long long nc = 0;
     if (i < r.n_inst) {
-      const long long T = item_tiles(r.coll_room[i], r.sstate[2 * i].n_tiles, r.n_inst, r.fp64);
+      const long long T = item_tiles(r, r.coll_room[i], r.sstate[2 * i].n_tiles);
       r.coll_tiles[i] = (unsigned int)T;
       nc = ((long long)r.sstate[2 * i].n_tiles + T - 1) / T +
            ((long long)r.sstate[2 * i + 1].n_tiles + kCollIonTiles - 1) / kCollIonTiles;
@@ -418,7 +418,7 @@ __device__ __forceinline__ void plan_single(const DeviceRefs& r, const StateShar
     if (sh.x[s].compact) mv += (sh.x[s].n_tiles_old + kMoveChunkTiles - 1) / kMoveChunkTiles;
   }
   r.ctrl->seg_cost = 0u;
-  const unsigned int T = item_tiles(room, sh.st[0].n_tiles, 1, r.fp64);
+  const unsigned int T = item_tiles(r, room, sh.st[0].n_tiles);
   r.coll_tiles[0] = T;
   r.coll_start[0] = 0u;
   plan_totals(r, 2, ns, w, mv,

@@ -324,11 +324,12 @@ struct ChunkStatus {
 // most kCollMaxTiles: small enough that an item holds about kCollTarget
 // candidates at the instance's last step's density, and, down to a round of 32
 // candidates (in double, where the FP64 unit of each SM counts, down to one
-// tile), that the instance gives its share of kCollSpread items (16 per SM).
+// tile), that the instance gives its share of kCollPerSm items per SM
+// (DeviceRefs::coll_share).
 constexpr int kCollMaxTiles = 32;
 constexpr int kCollIonTiles = 256;
 constexpr int kCollTarget = 128;
-constexpr int kCollSpread = 2432;
+constexpr int kCollPerSm = 16;
 // (a bound of the tiles that hold that many candidates)
 constexpr int kCollMaxRoom = 64 * kCollMaxTiles;
 // CTAs of k_finish beside the instances' own: those that place the births, and
@@ -372,6 +373,7 @@ struct DeviceRefs {
   int smem_nodes;         // deposit grid nodes in shared memory (0: global atomics)
   int push_warps;         // warps per particle-kernel CTA
   int push_grid;          // its CTAs
+  unsigned int coll_share;  // collision items an instance should give at least (see kCollPerSm)
   int coll_nodes;         // collision kernel: deposit grid nodes in shared memory (0: none)
   int fp64;               // marker path in double precision (else float)
   int n_field;            // blocks of kFieldNodes nodes of all instances
