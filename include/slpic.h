@@ -123,7 +123,9 @@ int slpic_create(slpic_ctx** out, int device, int n_instances);
 int slpic_destroy(slpic_ctx* ctx);
 
 /* Stream for all device work of ctx (a cudaStream_t, e.g. PyTorch's current
- * stream); NULL = the legacy default stream. */
+ * stream); NULL = the legacy default stream.  Work that ctx has queued on its
+ * stream until now comes before what follows on the new one; the old one is
+ * not used again. */
 int slpic_set_stream(slpic_ctx* ctx, void* cuda_stream);
 
 /* Gap of instance `inst` (Sec. IV): width d [m], n_cells >= 2 uniform cells,
@@ -165,7 +167,7 @@ int slpic_set_cross_sections_levels(slpic_ctx* ctx, int inst, int lo_exp2,
  * plus one tile).  Only electrons collide (Sec. IV).  Device memory per slot
  * of capacity: two buffers of the seven marker fields (56 B in FP32, 96 B in
  * FP64), and for electrons a null-collision candidate record (32 B in FP32,
- * 64 B in FP64) and the staging of emitted electrons (28 B or 48 B per ion
+ * 64 B in FP64) and the staging of emitted electrons (4 B or 8 B per ion
  * slot). */
 int slpic_set_species(slpic_ctx* ctx, int inst, int species, double mass,
                       double charge, double v_lim, int64_t capacity);
@@ -218,7 +220,8 @@ int slpic_set_precision(slpic_ctx* ctx, int bits);
 int slpic_load_particles(slpic_ctx* ctx, int inst, int species,
                          const slpic_soa_f32* host, int64_t n,
                          uint32_t next_id);
-/* Same from device arrays (device-to-device copies, no host staging). */
+/* Same from device arrays (no host staging).  The arrays must be complete when
+ * the work so far on ctx's stream and on the NULL stream is. */
 int slpic_load_particles_device(slpic_ctx* ctx, int inst, int species,
                                 const slpic_soa_f32* dev, int64_t n,
                                 uint32_t next_id);
@@ -421,9 +424,10 @@ int slpic_multiplication(slpic_ctx* ctx, int64_t steps_per_window, int n_windows
 
 /* Launch shape of the step: warps per CTA of the particle kernel (a
  * multiple of 4, at most 20; each warp owns a 128-slot tile) and CTAs per
- * SM of the collision kernel (1..32; as many run as fit).  While the warps' stages leave room
- * for the largest instance's charge grid in shared memory the kernel
- * deposits there; with more warps it deposits to global memory.  The
+ * SM of the collision kernel (1..32; as many run as fit: one in FP32, where
+ * every value is the same launch, and three in FP64).  While the warps'
+ * stages leave room for the largest instance's charge grid in shared memory
+ * the particle kernel deposits there; with more warps it deposits to global memory.  The
  * library's own choice is the most warps that leave that room, and 8.
  * Results do not depend on the shape, bit for bit: tiles are independent,
  * deposits are integer sums and births are ordered by (tile, slot). */
@@ -432,7 +436,8 @@ int slpic_get_launch_shape(slpic_ctx* ctx, int* push_warps, int* collide_ctas_pe
 /* Autotuner: times candidate shapes on the context's own markers and keeps
  * the fastest per marker-step; writes it to the out arguments (may be
  * NULL).  It tries every warp count, then collision CTAs per SM of
- * 2, 4, 8 and 16, running steps_each steps of the simulation for each.
+ * 2, 4, 8 and 16 (values that are the same launch do not compete), running
+ * steps_each steps of the simulation for each.
  * These are real steps: the state advances by (push candidates + 4) *
  * steps_each steps, exactly as slpic_step would have advanced it. */
 int slpic_autotune(slpic_ctx* ctx, int64_t steps_each, int* push_warps,

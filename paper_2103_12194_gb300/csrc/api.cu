@@ -1856,13 +1856,16 @@ extern "C" int slpic_autotune(slpic_ctx* c, int64_t steps_each, int* push_warps,
     }
   }
   const int cc_try[4] = {2, 4, 8, 16};
+  int best_grid = c->collide_grid;
   for (int k = 0; k < 4; ++k) {
     if (int rc = apply_shape(c, best_w, cc_try[k])) return rc;
     double t = 0;
     if (int rc = time_shape(c, steps_each, &t)) return rc;
-    if (t < best) {
+    // (values above what is resident are the launch that was timed before)
+    if (t < best && c->collide_grid != best_grid) {
       best = t;
       best_cc = cc_try[k];
+      best_grid = c->collide_grid;
     }
   }
   if (int rc = apply_shape(c, best_w, best_cc)) return rc;
