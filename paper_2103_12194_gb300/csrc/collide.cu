@@ -116,10 +116,7 @@ __global__ void __launch_bounds__(coll_warps<R>() * 32, sizeof(R) == 4 ? 1 : 3)
   constexpr int W = coll_warps<R>();
   step_kernel_entry();
   Control* ctrl = r.ctrl;
-  // (as one: an item of another CTA that does not fit its store may set the
-  // word between two threads' reads of it, and thread 0 sets the counter that
-  // hands out the items)
-  if (__syncthreads_or(*((volatile int*)&ctrl->error))) return;
+  const int stop = *((volatile int*)&ctrl->error);
   const unsigned int n_items = ctrl->n_coll_items;
   // (k_finish plans the next step while the births are still placed)
   if (blockIdx.x == 0)
@@ -153,7 +150,9 @@ __global__ void __launch_bounds__(coll_warps<R>() * 32, sizeof(R) == 4 ? 1 : 3)
     for (int k = threadIdx.x; k < tag_nodes; k += blockDim.x) s_rho[k] = 0ull;
   if (threadIdx.x < ACC_COUNT) s_acc[threadIdx.x] = 0ull;
   if (threadIdx.x == 0) s_next = i0 + W;
-  __syncthreads();
+  // (as one: an item of another CTA that does not fit its store may set the
+  // word between two threads' reads of it)
+  if (__syncthreads_or(stop)) return;
 
   CollQueues<R>& Q = reinterpret_cast<CollQueues<R>*>(coll_smem)[warp];
   unsigned int item = i0 + warp;
