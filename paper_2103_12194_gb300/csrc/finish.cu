@@ -815,16 +815,14 @@ __global__ void __launch_bounds__(kMoveThreads) k_move(DeviceRefs r) {
   step_kernel_entry();
   Control* ctrl = r.ctrl;
   // (as one: a wait of another CTA that runs out may set the word between two
-  // threads' reads of it, and the chunks are handed out by thread 0; read
-  // together with what decides whether there is anything to repack)
-  const int stop = *((volatile int*)&ctrl->error);
-  const unsigned int n_chunks = *((volatile unsigned int*)&ctrl->n_move_chunks);
-  if (__syncthreads_or(stop)) return;
+  // threads' reads of it, and the chunks are handed out by thread 0)
+  if (__syncthreads_or(*((volatile int*)&ctrl->error))) return;
   // the field of the step's Poisson solves, a block of nodes at a time
   for (int u = blockIdx.x; u < r.n_field; u += gridDim.x) {
     const int inst = field_inst(r, u);
     if (r.inst[inst].field_mode == 1) poisson_field(r.inst[inst], u - r.field_start[inst], s_field);
   }
+  const unsigned int n_chunks = ctrl->n_move_chunks;
   if (n_chunks == 0) return;
   const unsigned int epoch = ctrl->epoch;
   const int n_seg = r.n_inst * 2;

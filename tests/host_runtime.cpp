@@ -62,6 +62,9 @@ static void add(CUstream_st* s, Work w, CUevent_st* wait = nullptr) {
     s->capture->work.push_back(std::move(w));
     return;
   }
+  if (s == &g_null)
+    for (CUstream_st* b : g_streams)
+      if (b->blocking && b->capture) b->invalid = true;
   CUstream_st::Op op{std::move(w), {}};
   if (wait && wait->stream) op.after.push_back({wait->stream, wait->upto});
   if (s == &g_null) {
@@ -191,6 +194,9 @@ cudaError_t cudaStreamSynchronize(cudaStream_t s) {
 cudaError_t cudaStreamIsCapturing(cudaStream_t s, cudaStreamCaptureStatus* st) {
   *st = of(s)->capture ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
   return cudaSuccess;
+}
+cudaError_t cudaStreamGetFlags(cudaStream_t s, unsigned int* flags) {
+  return *flags = of(s)->blocking ? cudaStreamDefault : cudaStreamNonBlocking, cudaSuccess;
 }
 cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode* m) {
   static cudaStreamCaptureMode mode = cudaStreamCaptureModeGlobal;
@@ -441,9 +447,9 @@ static void replay_after_changes() {
 // when the old stream is gone.
 static void stream_changed_after_steps() {
   enum { kRead, kLoad, kSeed, kCapture, kTwice, kDestroyed, kRefused, kEnd };
-  for (int from = 0; from < 2; ++from)
+  for (int from = 0; from < 5; ++from)
     for (int what = kRead; what < kEnd; ++what) {
-      cudaStream_t a = from ? stream() : nullptr, b = stream();
+      cudaStream_t a = from % 3 ? stream(from == 2) : nullptr, b = stream(from > 2);
       Sim sim(a), plain;
       sim.load(300), plain.load(300);
       ok(slpic_step(sim.c, 40)), ok(slpic_step(plain.c, 40));
@@ -458,8 +464,9 @@ static void stream_changed_after_steps() {
       ok(slpic_set_stream(sim.c, b));
       if (what == kCapture) {
         cudaGraphExec_t e;
-        ok(slpic_step(sim.c, 1)), ok(slpic_step(plain.c, 1));
+        ok(slpic_step(sim.c, 1));
         expect(cudaStreamEndCapture(b, &g) == cudaSuccess, "the capture is invalid");
+        ok(slpic_step(plain.c, 1));
         cudaGraphInstantiate(&e, g, 0);
         cudaGraphLaunch(e, b);
       }
