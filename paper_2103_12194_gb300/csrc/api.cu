@@ -1716,12 +1716,13 @@ int slpic_read_wait_stats(slpic_ctx* c, int64_t* waits, int64_t* longest) {
   if (!c || !waits || !longest) return SLPIC_ERR_INVALID_ARG;
   if (int rc = prepare(c)) return rc;
   int rc = sync(c);
-  Control h;
-  CK(cudaMemcpy(&h, c->d_ctrl, sizeof h, cudaMemcpyDeviceToHost), "wait stats");
-  *waits = h.spin_waits;
-  *longest = h.spin_max;
-  unsigned int z[2] = {0u, 0u};
-  CK(cudaMemcpy(&c->d_ctrl->spin_waits, z, sizeof z, cudaMemcpyHostToDevice), "wait stats");
+  unsigned int h[2] = {0u, 0u};  // spin_waits, spin_max
+  const unsigned int z[2] = {0u, 0u};
+  if (int r2 = get(c, h, &c->d_ctrl->spin_waits, sizeof h)) return r2;
+  if (int r2 = put(c, &c->d_ctrl->spin_waits, z, sizeof z)) return r2;
+  if (int r2 = drain(c)) return r2;
+  *waits = h[0];
+  *longest = h[1];
   return rc;
 }
 
@@ -2268,10 +2269,7 @@ extern "C" int slpic_set_spin_limit(slpic_ctx* c, uint32_t polls) {
   c->spin_limit = polls;
   if (!c->d_ctrl) return SLPIC_OK;
   if (int rc = set_device(c)) return rc;
-  CK(cudaStreamSynchronize(c->stream), "spin limit");
-  CK(cudaMemcpy(&c->d_ctrl->spin_limit, &polls, sizeof polls, cudaMemcpyHostToDevice),
-     "spin limit");
-  return SLPIC_OK;
+  return put(c, &c->d_ctrl->spin_limit, &polls, sizeof polls);
 }
 
 extern "C" int slpic_test_skip_barrier(slpic_ctx* c, int inst, int64_t barrier) {
@@ -2279,12 +2277,10 @@ extern "C" int slpic_test_skip_barrier(slpic_ctx* c, int inst, int64_t barrier) 
   if (inst < -1 || inst >= c->n_inst || barrier < 0)
     return fail(c, SLPIC_ERR_INVALID_ARG, "skip barrier: instance in [-1, n_inst), barrier >= 0");
   if (int rc = prepare(c)) return rc;
-  CK(cudaStreamSynchronize(c->stream), "skip barrier");
   const int cta = inst + 1;
   const long long b = inst < 0 ? 0 : (long long)barrier;
-  CK(cudaMemcpy(&c->d_ctrl->skip_cta, &cta, sizeof cta, cudaMemcpyHostToDevice), "skip barrier");
-  CK(cudaMemcpy(&c->d_ctrl->skip_barrier, &b, sizeof b, cudaMemcpyHostToDevice), "skip barrier");
-  return SLPIC_OK;
+  if (int rc = put(c, &c->d_ctrl->skip_cta, &cta, sizeof cta)) return rc;
+  return put(c, &c->d_ctrl->skip_barrier, &b, sizeof b);
 }
 
 extern "C" int slpic_multiplication(slpic_ctx* c, int64_t steps_per_window, int n_windows,

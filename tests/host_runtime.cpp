@@ -571,6 +571,13 @@ static void copies_on_the_null_stream() {
   int64_t n = 0;
   ok(slpic_count(sim.c, 0, 0, &n));
   expect(g_null.done == g_null.ops.size(), "copies of the set-up");
+  ok(slpic_set_spin_limit(sim.c, 1000));
+  expect(g_null.done == g_null.ops.size(), "copy of the spin limit");
+  ok(slpic_test_skip_barrier(sim.c, 0, 3));
+  expect(g_null.done == g_null.ops.size(), "copies of the skipped barrier");
+  int64_t waits = 0, longest = 0;
+  ok(slpic_read_wait_stats(sim.c, &waits, &longest));
+  expect(g_null.done == g_null.ops.size(), "copies of the wait statistics");
   ok(slpic_load(sim.c, snap.data(), size));
   expect(g_null.done == g_null.ops.size(), "copies of the snapshot");
   ok(slpic_read_charge(sim.c, 0, 1, q[0], 9));
