@@ -23,8 +23,8 @@
 //     plain loads into registers, prefetched into L2, left its latency exposed
 //     (5 % slower where few instructions hide it).
 //   What bounds it: instruction issue under a speed limit (8e6 limited
-//   electrons on 4096 cells: 131 us, 417 warp instructions per 32 markers at
-//   68 % of the issue rate, DRAM at 2.2 TB/s; with a copy and an address per
+//   electrons on 4096 cells: 129 us, 416 warp instructions per 32 markers at
+//   69 % of the issue rate, DRAM at 2.2 TB/s; with a copy and an address per
 //   field and the IEEE roots and quotients 179 us and 546), the memory system
 //   without one (6e6 unlimited ions: 48 us with the deposit, 66 before).
 //   - Of unlimited ions only the front of the block is copied: cell, offset and
